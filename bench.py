@@ -196,7 +196,7 @@ def dist_env():
 # kernel, from ncu captures summarised in profiles/ncu_traffic.json. Each entry names the
 # sources that define the kernel and their SHA-256 at capture time: a kernel changed since its
 # capture reports null.
-KERNEL_SOURCES = {"group_stream_kernel": ["grouped.cu", "common.cuh", "launch.h"],
+KERNEL_SOURCES = {"group_stream_kernel": ["stream.cu", "common.cuh", "launch.h"],
                   "x_survey_bulk_kernel": ["prep.cu", "common.cuh", "launch.h"],
                   "x_survey_kernel": ["prep.cu", "common.cuh", "launch.h"]}
 

@@ -544,14 +544,14 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
   pr.key32 = groups && pl.FY <= 0xffffffffull;
   if (pr.key32) {
     uint32_t* k32 = nullptr;
-    STC_TRY(ar.alloc(&k32, (size_t)nY));
+    STC_TRY(ar.alloc(&k32, (size_t)nY + 1));
     pr.yfk = k32;
   } else {
     u64* k64 = nullptr;
     STC_TRY(ar.alloc(&k64, (size_t)nY));
     pr.yfk = k64;
   }
-  STC_TRY(ar.alloc(&pr.yv, (size_t)nY));
+  STC_TRY(ar.alloc(&pr.yv, (size_t)nY + 1));
   // X's arrays too, before any launch: the stages' events then enclose device work, not the
   // host's allocation calls.
   pr.sv.count = &pr.ctr->ns;
@@ -570,7 +570,7 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
   STC_CUDA(launch_y_count(Y->coords, nY, pl.ky, ycnt, status, ctx->sms, s, nonempty));
   STC_CUDA(scan_u32(ycnt, pr.yoff, (int64_t)bins, scr, s));
   STC_CUDA(cudaMemcpyAsync(ycur, pr.yoff, bins * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
-  STC_CUDA(launch_y_scatter(Y->coords, Y->vals, nY, pl.ky, ycur, pr.yfk, pr.key32, pr.yv, ctx->sms, s));
+  STC_CUDA(launch_y_scatter(Y->coords, Y->vals, nY, pl.ky, pl.FY, ycur, pr.yfk, pr.key32, pr.yv, ctx->sms, s));
   tm.mark(0);
 
   // X: find each entry's Y run and count the products exactly (Section 4.3).
@@ -600,7 +600,7 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
   const uint64_t cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)target / alpha) + 1));
   const uint64_t out_cap = std::min(target, cap);
   uint64_t b = sizeof(Counters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
-  b += (uint64_t)nY * 16 + (uint64_t)nX * 24;
+  b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
   b += (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
   b += cap * 16 + out_cap * (4ull * pl.ocols + 8);
   return b;
@@ -613,7 +613,7 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
 uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
   const uint64_t out = std::min<uint64_t>(P, pl.F);
   uint64_t b = sizeof(Counters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
-  b += (uint64_t)nY * 16 + (uint64_t)nX * (24 + 16);
+  b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
   b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
   b += out * (4ull * pl.ocols + 8);
   return b;
@@ -622,10 +622,10 @@ uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
 // Counters of the grouping and binning passes, read back with the first host sync.
 struct GroupCounters {
   uint32_t count[kMaxClasses + 4];
-  unsigned stream_nrec;  // streamed (group, segment) records
+  unsigned nholes;       // pieces of the streamed reservations that hold no output
   u64 huge_slots;
   u64 out_cap;
-  u64 stream_holes;      // positions of streamed reservations that hold no output
+  u64 holes;             // their positions
   u64 fill_counters[2];
 };
 
@@ -687,7 +687,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     // With AUTO, groups that fit the warp classes keep their hash tables (a bitmap sweep costs
     // a fixed amount per segment).
     b.dense_min = o.accumulator == STC_ACC_DENSE ? 0 : (b.tmax[1] + 1) * nseg;
-    b.stream_cap = dense_stream_cap();
+    b.stream_cap = stream_cap();
     b.stash_cap = dense_stash_cap();
     for (int d = 0; d < 3; d++) STC_TRY(ar.alloc(&b.dense_list[d], maxg));
   }
@@ -776,32 +776,33 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     STC_CUDA(launch_group_classes(a, wide, direct, b, hg.count, ctx->sms, s));
     STC_CUDA(launch_group_huge(a, hh, wide, ctx->sms, s));
   }
-  StreamArgs sa{};
   const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
+  StreamArgs sa{};
   if (dense_rows && !lane_rows) {
     // Streamed groups go last: every other kernel's outputs then lie below the final count.
     STC_CUDA(launch_group_dense(a, pr.yoff, nseg, seg, b.dense_list[2], hg.count[kMaxClasses + 3], b.dense_list[1],
                                 hg.count[kMaxClasses + 2], ctx->sms, s));
     if (nstream) {
-      STC_TRY(ar.alloc(&sa.rec, (size_t)nstream * nseg));
-      sa.nrec = &gc->stream_nrec;
-      sa.holes = &gc->stream_holes;
-      const bool fixed_rows = !pl.op.pow2 && pl.op.ident && pl.op.order >= 2 && pl.op.order <= 8;
-      STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, fixed_rows, ctx->sms, s));
+      STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms)));
+      sa.nholes = &gc->nholes;
+      sa.hole_total = &gc->holes;
+      sa.ny_entries = (uint32_t)Y->nnz;
+      STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, ctx->sms, s));
     }
   }
   tm.mark(4);
   u64 holes = 0;
-  if (nstream) STC_CUDA(cudaMemcpyAsync(&holes, &gc->stream_holes, sizeof(u64), cudaMemcpyDeviceToHost, s));
+  if (nstream) STC_CUDA(cudaMemcpyAsync(&holes, &gc->holes, sizeof(u64), cudaMemcpyDeviceToHost, s));
   Counters h2{};
   STC_TRY(read_counters(pr, s, h2));
   r->nnz = (int64_t)(h2.nz - holes);
   if (holes) {
-    if (holes >= (1ull << 32)) return fail(STC_ERR_UNSUPPORTED, "more than 2^32 repeated products in streamed groups");
-    uint32_t* src_pos = nullptr;
-    STC_TRY(ar.alloc(&src_pos, (size_t)holes));
-    STC_CUDA(launch_stream_fill(sa.rec, sa.nrec, (u64)r->nnz, holes, src_pos, gc->fill_counters, r->coords,
-                                r->vals, pl.ocols, &pr.ctr->status, ctx->sms, s));
+    u64* dst = nullptr;
+    uint8_t* marked = nullptr;
+    STC_TRY(ar.alloc(&dst, (size_t)holes));
+    STC_TRY(ar.alloc(&marked, (size_t)holes));
+    STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, (u64)r->nnz, holes, marked, dst, gc->fill_counters, r->coords,
+                              r->vals, pl.ocols, &pr.ctr->status, ctx->sms, s));
     tm.mark(5);
   }
   r->stats.out_capacity = out_cap;

@@ -66,8 +66,13 @@ __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint
       int c = 0;
       while (c < b.nclasses && t > b.tmax[c]) c++;
       if (b.dense_list[0] && t >= b.dense_min) {
-        // Streamed groups reserve one output position per product (their repeats' records).
-        const int d = (bnd <= b.stream_cap && 2 * bnd <= FY) ? 0 : (bnd <= b.stash_cap ? 2 : 1);
+        // The streaming kernel pays for every repeat, the stash kernel for every product. Measured
+        // on 8,192 groups of 6,400 products: 30,000 free keys 0.59 against 0.81 ms, 10,000 keys
+        // 0.70 against 0.78, 4,096 keys 0.87 against 0.71; of 7,680 products over 10,000 keys 0.82
+        // against 0.79. Past the stash's capacity the choice is between streaming and the rank
+        // kernel's two passes. Streamed groups reserve one output position per product.
+        const bool stashed = bnd <= b.stash_cap;
+        const int d = bnd <= b.stream_cap && (4 * bnd <= 3 * FY || (!stashed && bnd <= FY)) ? 0 : (stashed ? 2 : 1);
         my_cap += d == 0 ? bnd : t;
         const uint32_t idx = atomicAdd(b.count + kMaxClasses + 1 + d, 1u);
         b.dense_list[d][idx] = (uint32_t)g;
@@ -1045,8 +1050,8 @@ __global__ void __launch_bounds__(THREADS, 2) group_bitmap_kernel(GroupArgs a, c
 }
 
 
-// ---- product stash: groups whose product count fits the stash (the common case of the
-// bitmap path). Pass 1 forms every product once (Y key and value read together, one round
+// ---- product stash: groups whose product count fits the stash and that repeat many keys (the
+// streaming kernel takes the others). Pass 1 forms every product once (Y key and value read together, one round
 // trip) and marks its free key in a bitmap over the segment: the first product of a key is
 // the one that finds its bit clear. First products take consecutive places at the front of
 // the stash (their order is the group's output order); repeats take places from the back
@@ -1343,371 +1348,6 @@ __global__ void __launch_bounds__(kStashThreads, 2) group_stash_kernel(GroupArgs
     }
   }
 }
-
-
-// ---- output streaming: groups whose product count fits kStreamCap (the common case of the
-// bitmap path). Each group segment reserves as many output positions as it has products.
-// Pass 1 forms every product once and marks its free key in a bitmap over the segment; the
-// first product of a key (the one that finds its bit clear) writes its output entry at once,
-// at the next place from the front of the reservation. A repeat writes its key and value as
-// a temporary record at the next place from the back and marks its key in a second bitmap.
-// After a block barrier (which orders the block's own stores before its later reads and
-// atomics) the repeated keys are ranked, their first products' places looked up, and every
-// repeat adds its value to that entry with an L2 atomic. The back of the reservation (the repeats' records) becomes a hole; after all
-// groups, holes below the final output count are filled with the entries above it.
-
-#ifndef STREAM_U
-#define STREAM_U 3
-#endif
-#ifndef STREAM_MINB
-#define STREAM_MINB 4
-#endif
-constexpr int kStreamThreads = 256;
-constexpr uint32_t kStreamEntries = 256;  // X entries staged per chunk
-constexpr uint32_t kStreamCap = 8192;     // products of one group segment
-constexpr uint32_t kStreamSlots = kStreamCap / 32 + kStreamEntries;
-// Shared memory: key bitmap, repeat bitmap, slot table, X values, first-product keys, and the
-// rank -> place map of the repeated keys.
-static_assert(kStreamCap % 4 == 0, "the fix-up reads the first-product keys four at a time");
-constexpr size_t kStreamSmem = (size_t)kBitmapWords * 8 + (size_t)kStreamSlots * 8 + (size_t)kStreamEntries * 8 +
-                               (size_t)kStreamCap * 2 + (size_t)kStreamCap;
-
-// FIXED: output rows of 2..8 coordinates in concatenation order with some length not a power
-// of two, decoded into registers and stored in pairs (store_row_fixed); a separate
-// instantiation so that the power-of-two kernel keeps its own code.
-template <int U, bool FIXED>
-__global__ void __launch_bounds__(kStreamThreads, STREAM_MINB) group_stream_kernel(GroupArgs a, const uint32_t* __restrict__ yoff,
-                                                                        uint32_t nseg, uint32_t seg,
-                                                                        const uint32_t* __restrict__ list,
-                                                                        uint32_t count, StreamArgs sa) {
-  constexpr int T = kStreamThreads, NW = T / 32;
-  constexpr uint32_t CH = kStreamEntries;
-  extern __shared__ __align__(16) unsigned char smem[];
-  const uint32_t nwords = seg >> 5;
-  uint32_t* const bits = reinterpret_cast<uint32_t*>(smem);              // key marks, then repeat ranks
-  uint32_t* const rbits = bits + kBitmapWords;                           // keys met again
-  uint2* const stab = reinterpret_cast<uint2*>(rbits + kBitmapWords);   // slot table
-  double* const sx = reinterpret_cast<double*>(stab + kStreamSlots);    // X values of the chunk
-  uint16_t* const pk = reinterpret_cast<uint16_t*>(sx + CH);            // keys of the first products
-  uint16_t* const map = pk + kStreamCap;                                 // repeat rank -> first place
-  __shared__ u64 warp_tot[NW + 1];
-  __shared__ OutTarget tg;
-  __shared__ u64 s_gbase;
-  __shared__ uint32_t s_cnt;
-  // Order-4 power-of-two outputs: each coordinate is either constant over the segment or a bit
-  // field of the segment-relative free key fy = q * seg + fk; coordinate = cst | (fy >> sh) & mk.
-  __shared__ int4 s_cst;
-  __shared__ uint4 s_sh, s_mk;
-  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  const uint32_t lt = lanemask_lt();
-  const uint64_t keep = policy_evict_last();
-  const uint64_t pol = policy_evict_first();
-  const uint32_t* yfk = static_cast<const uint32_t*>(a.yfk);
-  for (uint32_t i = threadIdx.x; i < 2 * kBitmapWords; i += T) bits[i] = 0;
-  if (threadIdx.x == 0) s_cnt = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *sa.nrec = count * nseg;  // one record per (group, segment)
-  // Prefetched staging of the next group (when it fits one chunk).
-  uint32_t pf_g = 0, pf_x0 = 0, pf_x1 = 0, pf_ck = 0, pf_ys = 0, pf_ye = 0;
-  double pf_v = 0.0;
-  auto prefetch = [&](uint32_t gi) {
-    if (gi >= count) return;
-    pf_g = list[gi];
-    pf_x0 = a.goff[pf_g];
-    pf_x1 = a.goff[pf_g + 1];
-    if (pf_x1 - pf_x0 <= CH && threadIdx.x < pf_x1 - pf_x0) {
-      pf_ck = a.gx.ck[pf_x0 + threadIdx.x];
-      pf_v = a.gx.v[pf_x0 + threadIdx.x];
-      if (nseg == 1) {
-        pf_ys = __ldg(yoff + pf_ck);
-        pf_ye = __ldg(yoff + pf_ck + 1);
-      }
-    }
-  };
-  prefetch(blockIdx.x);
-  if (threadIdx.x < 32) {  // warp 0 resolves the targets: no plan cached yet
-    if (threadIdx.x == 0) tg.prob = kNoProb;
-    __syncwarp();
-  }
-  for (uint32_t gi = blockIdx.x; gi < count; gi += gridDim.x) {
-    const uint32_t g = pf_g, x0 = pf_x0, x1 = pf_x1;
-    const bool one_chunk = x1 - x0 <= CH;
-    if ((threadIdx.x >> 5) == 0) resolve_target_warp(a, g, 0, tg);  // warp 0; published by later barriers
-    const uint32_t my_ck = pf_ck, my_ys = pf_ys, my_ye = pf_ye;
-    const double my_v = pf_v;
-    prefetch(gi + gridDim.x);
-    for (uint32_t q = 0; q < nseg; q++) {
-      if (threadIdx.x == 0 && tg.op.order == 4 && tg.op.pow2) {
-        // Published by the staging scan's barriers below.
-        const uint32_t b = 63 - __clzll(tg.FY);
-        uint32_t c[4], sh[4], mk[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const uint32_t sk = tg.op.shift[k], mkk = (uint32_t)tg.op.mod[k] - 1;
-          const bool cst = sk >= b;
-          c[k] = cst ? (uint32_t)(tg.zrow >> sk) & mkk : 0u;
-          sh[k] = cst ? 0u : sk;
-          mk[k] = cst ? 0u : mkk;
-        }
-        s_cst = make_int4((int32_t)c[0], (int32_t)c[1], (int32_t)c[2], (int32_t)c[3]);
-        s_sh = make_uint4(sh[0], sh[1], sh[2], sh[3]);
-        s_mk = make_uint4(mk[0], mk[1], mk[2], mk[3]);
-      }
-      // The segment's products, reserved up front (a separate count pass for long groups).
-      uint32_t Pq = 0;
-      if (!one_chunk) {
-        for (uint32_t c0 = x0; c0 < x1; c0 += CH) {
-          const uint32_t n = (x1 - c0 < CH) ? x1 - c0 : CH;
-          uint32_t len = 0;
-          if (threadIdx.x < n) {
-            const u64 b = (u64)a.gx.ck[c0 + threadIdx.x] * nseg + q;
-            len = __ldg(yoff + b + 1) - __ldg(yoff + b);
-          }
-          uint32_t tot;
-          block_exscan_u32<T>(len, &tot, warp_tot);
-          Pq += tot;
-        }
-        if (Pq == 0) {
-          if (threadIdx.x == 0) sa.rec[(u64)gi * nseg + q] = StreamRec{0, 0, 0};
-          continue;
-        }
-        if (threadIdx.x == 0) s_gbase = atomicAdd(tg.counter, (u64)Pq);
-      }
-      // ---- pass 1, one chunk of X entries at a time.
-      for (uint32_t c0 = x0; c0 < x1; c0 += CH) {
-        const uint32_t n = (x1 - c0 < CH) ? x1 - c0 : CH;
-        uint32_t ys = 0, len = 0;
-        if (threadIdx.x < n) {
-          sx[threadIdx.x] = one_chunk ? my_v : a.gx.v[c0 + threadIdx.x];
-          if (one_chunk && nseg == 1) {
-            ys = my_ys;
-            len = my_ye - my_ys;
-          } else {
-            const uint32_t ck = one_chunk ? my_ck : a.gx.ck[c0 + threadIdx.x];
-            const u64 b = (u64)ck * nseg + q;
-            ys = __ldg(yoff + b);
-            len = __ldg(yoff + b + 1) - ys;
-          }
-        }
-        // Products (high bits) and slots (low 12 bits) before each entry, in one scan; a
-        // one-chunk group reserves its outputs between the scan's two barriers.
-        const uint32_t nslot = (len + 31) >> 5;
-        uint32_t x = (len << 12) | nslot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-          if ((int)lane >= o) x += y;
-        }
-        if (lane == 31) warp_tot[warp] = x;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-          const uint32_t t = (int)lane < NW ? (uint32_t)warp_tot[lane] : 0u;
-          uint32_t inc = t;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if ((int)lane >= o) inc += y;
-          }
-          if ((int)lane < NW) warp_tot[lane] = inc - t;
-          if (lane == 31) {
-            warp_tot[NW] = inc;
-            if (one_chunk && (inc >> 12)) s_gbase = atomicAdd(tg.counter, (u64)(inc >> 12));
-          }
-        }
-        __syncthreads();
-        const uint32_t tot = (uint32_t)warp_tot[NW], S = tot & 4095u;
-        if (one_chunk) Pq = tot >> 12;
-        {
-          uint32_t s = ((uint32_t)warp_tot[warp] + x - ((len << 12) | nslot)) & 4095u;
-          if (threadIdx.x < n) {
-            for (uint32_t k = 0; k < len; k += 32, s++) {
-              const uint32_t live = len - k < 32 ? len - k : 32;
-              stab[s] = make_uint2(ys + k, live | (threadIdx.x << 8));
-            }
-          }
-        }
-        __syncthreads();
-        if (Pq == 0) continue;
-        const u64 gbase = s_gbase;
-        const u64 zseg = tg.zrow + (u64)q * seg;
-        int32_t* const coords = tg.coords;
-        double* const vals = tg.vals;
-        const int oz = tg.op.order;
-        const bool v4 = oz == 4 && tg.op.pow2 && ((reinterpret_cast<uintptr_t>(coords) & 15u) == 0);
-        for (uint32_t sb = warp; sb < S; sb += NW * U) {
-          uint32_t f[U], e[U];
-          double y[U];
-          bool ok[U], in[U];
-#pragma unroll
-          for (int u = 0; u < U; u++) {
-            const uint32_t si = sb + u * NW;
-            in[u] = si < S;
-            ok[u] = false;
-            if (in[u]) {
-              const uint2 rec = stab[si];
-              ok[u] = lane < (rec.y & 255u);
-              const uint32_t j = rec.x + (ok[u] ? lane : 0u);
-              e[u] = rec.y >> 8;
-              f[u] = ld_keep_u32(yfk + j, keep);
-              y[u] = ld_keep_f64(a.yv + j, keep);
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < U; u++) {
-            if (in[u]) {
-              const uint32_t fk = f[u] & (seg - 1);
-              const double prod = __dmul_rn(sx[e[u]], y[u]);
-              const uint32_t w = fk >> 5, bit = 1u << (fk & 31);
-              bool first = false;
-              if (ok[u]) {
-                first = (atomicOr(bits + w, bit) & bit) == 0;
-                if (!first) atomicOr(rbits + w, bit);
-              }
-              const uint32_t fm = __ballot_sync(0xffffffffu, first);
-              const uint32_t rm = __ballot_sync(0xffffffffu, ok[u] && !first);
-              uint32_t base = 0;
-              if (lane == 0) base = atomicAdd(&s_cnt, (uint32_t)__popc(fm) | ((uint32_t)__popc(rm) << 16));
-              base = __shfl_sync(0xffffffffu, base, 0);
-              if (ok[u]) {
-                if (first) {
-                  const uint32_t place = (base & 0xffffu) + __popc(fm & lt);
-                  pk[place] = (uint16_t)fk;
-                  const u64 pos = gbase + place;
-                  if (v4) {
-                    const uint32_t fy = q * seg + fk;
-                    const int4 cb = s_cst;
-                    const uint4 sh = s_sh, mk = s_mk;
-                    const int4 cv = make_int4(cb.x | (int32_t)((fy >> sh.x) & mk.x), cb.y | (int32_t)((fy >> sh.y) & mk.y),
-                                              cb.z | (int32_t)((fy >> sh.z) & mk.z), cb.w | (int32_t)((fy >> sh.w) & mk.w));
-                    st_stream_v4(coords + pos * 4, cv, pol);
-                    vals[pos] = prod;  // default policy: a repeat may still add to it
-                  } else {
-                    store_output<FIXED>(coords, vals, pos, zseg + fk, prod, tg.op, pol);
-                  }
-                } else {
-                  const u64 pos = gbase + Pq - 1 - ((base >> 16) + __popc(rm & lt));
-                  if (oz) coords[pos * oz] = (int32_t)fk;
-                  vals[pos] = prod;
-                }
-              }
-            }
-          }
-        }
-        if (!one_chunk) __syncthreads();
-      }
-      if (Pq == 0) {
-        if (threadIdx.x == 0) sa.rec[(u64)gi * nseg + q] = StreamRec{0, 0, 0};
-        continue;
-      }
-      // The block barrier orders every thread's earlier global stores (first products, repeats'
-      // records) before the later reads and atomics of the block's threads, which are the only
-      // ones that touch this group's reservation; no device-wide fence is needed.
-      __syncthreads();
-      const uint32_t nkeys = s_cnt & 0xffffu, reps = s_cnt >> 16;
-      if (reps) {
-        const u64 gbase = s_gbase;
-        // Rank the repeated keys; the key marks are no longer needed and hold the ranks.
-        const uint32_t wpt = (nwords + T - 1) / T;
-        const uint32_t w0 = threadIdx.x * wpt, w1 = w0 + wpt < nwords ? w0 + wpt : nwords;
-        uint32_t sum = 0;
-        for (uint32_t w = w0; w < w1; w++) sum += __popc(rbits[w]);
-        uint32_t nrk;
-        uint32_t r = block_exscan_u32<T>(sum, &nrk, warp_tot);
-        for (uint32_t w = w0; w < w1; w++) {
-          bits[w] = r;
-          r += __popc(rbits[w]);
-        }
-        __syncthreads();
-        // Four first-product keys per 8-byte load (pk holds kStreamCap entries, so reading up
-        // to the next multiple of four stays inside it; entries past nkeys are skipped).
-        for (uint32_t q = threadIdx.x; q < (nkeys + 3) / 4; q += T) {
-          const uint2 four = reinterpret_cast<const uint2*>(pk)[q];
-#pragma unroll
-          for (int t = 0; t < 4; t++) {
-            const uint32_t i = q * 4 + t;
-            const uint32_t fk = ((t < 2 ? four.x : four.y) >> ((t & 1) * 16)) & 0xffffu;
-            const uint32_t w = fk >> 5, bit = 1u << (fk & 31), rw = rbits[w];
-            if (i < nkeys && (rw & bit)) map[bits[w] + __popc(rw & (bit - 1))] = (uint16_t)i;
-          }
-        }
-        __syncthreads();
-        const int oz = tg.op.order;
-        for (uint32_t k = threadIdx.x; k < reps; k += T) {
-          const u64 pos = gbase + Pq - 1 - k;
-          const uint32_t fk = oz ? (uint32_t)__ldcg(tg.coords + pos * oz) : 0u;
-          const double v = __ldcg(tg.vals + pos);
-          const uint32_t w = fk >> 5, bit = 1u << (fk & 31);
-          atomicAdd(tg.vals + gbase + map[bits[w] + __popc(rbits[w] & (bit - 1))], v);
-        }
-        if (threadIdx.x == 0) atomicAdd(sa.holes, (u64)reps);
-        __syncthreads();  // the lookups above read the bitmaps cleared below
-      }
-      // Every streamed segment is recorded, at its own index (list position, segment): those
-      // whose outputs end above the final count are the sources of the hole filling, whatever
-      // their repeats.
-      if (threadIdx.x == 0) sa.rec[(u64)gi * nseg + q] = StreamRec{s_gbase, nkeys, Pq};
-      // ---- clear the bitmaps for the next segment or group.
-      for (uint32_t i = threadIdx.x; i < nwords / 4; i += T) {
-        reinterpret_cast<uint4*>(bits)[i] = make_uint4(0, 0, 0, 0);
-        reinterpret_cast<uint4*>(rbits)[i] = make_uint4(0, 0, 0, 0);
-      }
-      if (nwords < 4 && threadIdx.x < nwords) bits[threadIdx.x] = rbits[threadIdx.x] = 0;
-      if (threadIdx.x == 0) s_cnt = 0;
-      __syncthreads();
-    }
-  }
-}
-
-// Hole filling after the streaming kernel (its reservations are the last ones, so every
-// other kernel's outputs lie below the final count). Sources: the entries of streamed
-// segments at positions >= nnz; holes: the repeats' records below nnz. Both are numbered
-// through atomic counters; hole k receives source k.
-__global__ void __launch_bounds__(256) stream_sources_kernel(const StreamRec* __restrict__ rec,
-                                                             const unsigned* __restrict__ nrec, u64 nnz,
-                                                             uint32_t* __restrict__ src_pos, u64* __restrict__ src_count) {
-  const unsigned lane = lane_id();
-  const unsigned nr = *nrec;
-  for (unsigned i = blockIdx.x * 8 + (threadIdx.x >> 5); i < nr; i += gridDim.x * 8) {
-    const StreamRec r = rec[i];
-    const u64 lo = r.base > nnz ? r.base : nnz, hi = r.base + r.firsts;
-    if (lo >= hi) continue;
-    u64 k0 = 0;
-    if (lane == 0) k0 = atomicAdd(src_count, hi - lo);
-    k0 = __shfl_sync(0xffffffffu, k0, 0);
-    for (u64 p = lo + lane; p < hi; p += 32) src_pos[k0 + (p - lo)] = (uint32_t)(p - nnz);
-  }
-}
-
-__global__ void __launch_bounds__(256) stream_fill_kernel(const StreamRec* __restrict__ rec,
-                                                          const unsigned* __restrict__ nrec, u64 nnz,
-                                                          const uint32_t* __restrict__ src_pos, u64 nsrc,
-                                                          u64* __restrict__ hole_count, int32_t* __restrict__ coords,
-                                                          double* __restrict__ vals, int oz, uint32_t* status) {
-  const unsigned lane = lane_id();
-  const unsigned nr = *nrec;
-  for (unsigned i = blockIdx.x * 8 + (threadIdx.x >> 5); i < nr; i += gridDim.x * 8) {
-    const StreamRec r = rec[i];
-    const u64 lo = r.base + r.firsts, hi0 = r.base + r.products, hi = hi0 < nnz ? hi0 : nnz;
-    if (lo >= hi) continue;
-    u64 k0 = 0;
-    if (lane == 0) k0 = atomicAdd(hole_count, hi - lo);
-    k0 = __shfl_sync(0xffffffffu, k0, 0);
-    for (u64 h = lo + lane; h < hi; h += 32) {
-      const u64 k = k0 + (h - lo);
-      if (k >= nsrc) {
-        atomicOr(status, kStatOutOverflow);
-        continue;
-      }
-      const u64 s = nnz + src_pos[k];
-      if (oz == 4 && ((reinterpret_cast<uintptr_t>(coords) & 15u) == 0)) {
-        reinterpret_cast<int4*>(coords)[h] = reinterpret_cast<const int4*>(coords)[s];
-      } else {
-        for (int q = 0; q < oz; q++) coords[h * oz + q] = coords[s * oz + q];
-      }
-      vals[h] = vals[s];
-    }
-  }
-}
-
 
 // ---- small groups: one warp per group, each warp with its own table (group-per-warp
 // granularity). Everything a group needs stays inside its warp, so warp-level
@@ -2427,39 +2067,6 @@ cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, i
 }
 
 uint32_t dense_stash_cap() { return kStashCap; }
-uint32_t dense_stream_cap() { return kStreamCap; }
-
-cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
-                                const uint32_t* list, uint32_t count, StreamArgs sa, bool fixed_rows, int sms,
-                                cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  if (seg < 64 || seg > kDenseSeg) return cudaErrorInvalidValue;
-  constexpr int U = STREAM_U;
-  auto kern = fixed_rows ? group_stream_kernel<U, true> : group_stream_kernel<U, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmem);
-  if (e != cudaSuccess) return e;
-  int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kStreamThreads, kStreamSmem);
-  if (e != cudaSuccess) return e;
-  if (per_sm < 1) per_sm = 1;
-  const uint32_t cap = (uint32_t)(sms * per_sm);
-  kern<<<count < cap ? count : cap, kStreamThreads, kStreamSmem, s>>>(a, yoff, nseg, seg, list, count, sa);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stream_fill(const StreamRec* rec, const unsigned* nrec, u64 nnz, u64 holes_total, uint32_t* src_pos,
-                               u64* counters2, int32_t* coords, double* vals, int oz, uint32_t* status, int sms,
-                               cudaStream_t s) {
-  if (holes_total == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(counters2, 0, 2 * sizeof(u64), s);
-  if (e != cudaSuccess) return e;
-  const unsigned g = (unsigned)sms * 8;
-  stream_sources_kernel<<<g, 256, 0, s>>>(rec, nrec, nnz, src_pos, counters2);
-  stream_fill_kernel<<<g, 256, 0, s>>>(rec, nrec, nnz, src_pos, holes_total, counters2 + 1, coords, vals, oz, status);
-  note_launch(2);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_group_dense(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                const uint32_t* stash_list, uint32_t stash_count, const uint32_t* rank_list,

@@ -41,8 +41,10 @@ cudaError_t launch_key_scatter(const u64* keys, int64_t n, u64 k, uint32_t* curs
 // keys that have at least one Y entry.
 cudaError_t launch_y_count(const int32_t* coords, int64_t n, const KeyPlan& p, uint32_t* cnt,
                            uint32_t* status, int sms, cudaStream_t s, uint32_t* nonempty = nullptr);
-// yfk receives 32-bit free keys when key32 is set (F_Y < 2^32), 64-bit ones otherwise.
-cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p,
+// yfk receives 32-bit free keys when key32 is set (F_Y < 2^32), 64-bit ones otherwise. 32-bit
+// arrays hold n + 1 entries: the last has the key stream_dead_key(FY) and the value 0.
+uint32_t stream_dead_key(u64 FY);
+cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p, u64 FY,
                              uint32_t* cursor, void* yfk, bool key32, double* yv, int sms, cudaStream_t s);
 
 // X entries whose contract key has a non-empty Y run ("survivors"), compacted, with the
@@ -161,10 +163,9 @@ struct Bins {
   u64 tmax[kMaxClasses];      // a group goes to the first class with t <= tmax
   uint32_t* list[kMaxClasses];
   uint32_t* count;            // [kMaxClasses + 4]: classes, overflow groups, stream, rank, stash
-  // Bitmap-row accumulation (single contractions with per-segment runs): groups with
-  // t >= dense_min go to the stream list (0) when B_g <= stream_cap and repeats are expected
-  // to be few (2 B_g <= F_Y), else to the stash list (2) when B_g <= stash_cap, else to the
-  // rank list (1). A streamed group's output bound is B_g itself.
+  // Dense rows (single contractions with per-segment runs): groups with t >= dense_min go to
+  // the stream list (0), the stash list (2) or the rank list (1) by their size and expected
+  // repeats (bin_groups_kernel). A streamed group's output bound is B_g itself.
   uint32_t* dense_list[3];    // null when not used
   u64 dense_min;
   u64 stream_cap;
@@ -322,38 +323,44 @@ cudaError_t launch_batch_group(const BatchArgs& ba, GroupedX gx, const Bins& b, 
 // Bitmap-row accumulation: each group's outputs are found one free-key segment at a time
 // through a bitmap over the segment's free keys. `yoff` are the per-(contract key, segment)
 // run offsets; seg is the segment width (a power of two, 64 <= seg <= kDenseSeg). Groups
-// with at most dense_stash_cap() products (per segment) go to the stash kernel, the others
+// with at most dense_stash_cap() products (per segment) may go to the stash kernel, the others
 // to the rank kernel.
 constexpr uint32_t kDenseSeg = 65536;
 constexpr size_t kBitmapSmemPerCta = 112 * 1024;  // two CTAs per SM
 uint32_t dense_stash_cap();
 
-// Streamed bitmap rows: per group segment, its reservation and counts, for the hole filling
-// that follows.
-struct StreamRec {
-  u64 base;           // first reserved position
-  uint32_t firsts;    // outputs (first products), at [base, base + firsts)
-  uint32_t products;  // reserved positions
+// ------------------------------------------------------------------ streamed groups (stream.cu)
+// Positions reserved by the streaming kernel that no output took.
+struct StreamHole {
+  u64 pos;
+  u64 len;
 };
 struct StreamArgs {
-  StreamRec* rec;
-  unsigned* nrec;  // records: one per (streamed group, segment), [list position * nseg + segment]
-  u64* holes;      // total repeats (positions that hold no output at the end)
+  StreamHole* holes;    // [stream_max_holes]
+  unsigned* nholes;
+  u64* hole_total;
+  uint32_t ny_entries;  // entries of Y; the arrays hold one more (stream_dead_key)
+  // Set by launch_group_stream: how the Y free key decodes into the output coordinates.
+  uint32_t dead;            // stream_dead_key(F_Y)
+  uint32_t rsh[4], rmk[4];  // order-4 power-of-two rows: coordinate q has (key >> rsh) & rmk
+  int ny;                   // other rows: digits of the Y part, last mode first
+  uint32_t ymod[6], ymagic[6], ysh1[6], ysh2[6];
 };
+uint32_t stream_cap();  // most products of a streamed group
+size_t stream_max_holes(uint32_t count, uint32_t nseg, int sms);
+// Launched after every other accumulation kernel, so that the positions it reserves are the last
+// ones.
+cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
+                                const uint32_t* list, uint32_t count, const StreamArgs& sa, int sms, cudaStream_t s);
+// Moves the entries at and above nnz into the holes below it. total: positions of all holes;
+// marked [total] and dst [total] are scratch.
+cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, u64 nnz, u64 total, uint8_t* marked,
+                             u64* dst, u64* counters2, int32_t* coords, double* vals, int oz, uint32_t* status,
+                             int sms, cudaStream_t s);
+
 // Lane-private dense rows for output rows of at most 64 free keys (FY <= 64, 32-bit Y free
 // keys): one warp per group g in [0, ngroups) (empty groups skipped), outputs in key order.
 cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, int sms, cudaStream_t s);
-uint32_t dense_stream_cap();
-// Streamed groups (B_g <= dense_stream_cap()); launched after every other accumulation kernel.
-// fixed_rows: the output plan has 2..8 modes in concatenation order, not all powers of two.
-cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
-                                const uint32_t* list, uint32_t count, StreamArgs sa, bool fixed_rows, int sms,
-                                cudaStream_t s);
-// Moves the entries above nnz into the holes below it.
-// holes_total < 2^32 (positions above nnz are kept as 32-bit offsets).
-cudaError_t launch_stream_fill(const StreamRec* rec, const unsigned* nrec, u64 nnz, u64 holes_total, uint32_t* src_pos,
-                               u64* counters2, int32_t* coords, double* vals, int oz, uint32_t* status, int sms,
-                               cudaStream_t s);
 cudaError_t launch_group_dense(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                const uint32_t* stash_list, uint32_t stash_count, const uint32_t* rank_list,
                                uint32_t rank_count, int sms, cudaStream_t s);

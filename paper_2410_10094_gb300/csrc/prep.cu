@@ -106,7 +106,11 @@ template <int ORDER, bool VEC, typename YK>
 __global__ void __launch_bounds__(kThreads) y_scatter_kernel(const int32_t* __restrict__ coords,
                                                              const double* __restrict__ vals, int64_t n, KeyPlan p,
                                                              uint32_t* __restrict__ cursor, YK* __restrict__ yfk,
-                                                             double* __restrict__ yv) {
+                                                             double* __restrict__ yv, uint32_t dead) {
+  if (sizeof(YK) == 4 && blockIdx.x == 0 && threadIdx.x == 0) {
+    yfk[n] = (YK)dead;
+    yv[n] = 0.0;
+  }
   const int64_t step = (int64_t)gridDim.x * kThreads * kRows;
   for (int64_t base = (int64_t)blockIdx.x * kThreads * kRows + threadIdx.x; base < n; base += step) {
     uint64_t ck[kRows], fk[kRows];
@@ -769,16 +773,16 @@ cudaError_t launch_y_count(const int32_t* coords, int64_t n, const KeyPlan& p, u
   });
 }
 
-cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p,
+cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p, u64 FY,
                              uint32_t* cursor, void* yfk, bool key32, double* yv, int sms, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const unsigned g = grid_for((n + kRows - 1) / kRows, sms);
   return dispatch_order(p.order, vec_ok(coords, p.order), [&]<int O, bool V>() {
     if (key32)
       y_scatter_kernel<O, V, uint32_t>
-          <<<g, kThreads, 0, s>>>(coords, vals, n, p, cursor, static_cast<uint32_t*>(yfk), yv);
+          <<<g, kThreads, 0, s>>>(coords, vals, n, p, cursor, static_cast<uint32_t*>(yfk), yv, stream_dead_key(FY));
     else
-      y_scatter_kernel<O, V, u64><<<g, kThreads, 0, s>>>(coords, vals, n, p, cursor, static_cast<u64*>(yfk), yv);
+      y_scatter_kernel<O, V, u64><<<g, kThreads, 0, s>>>(coords, vals, n, p, cursor, static_cast<u64*>(yfk), yv, 0u);
     note_launch();
     return cudaGetLastError();
   });
