@@ -770,7 +770,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   a.bout = dbo;
   a.bnz = &pr.ctr->nz;
   if (lane_rows) {
-    STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, ctx->sms, s));
+    STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, h.P, ctx->sms, s));
   } else {
     const bool direct = !wide && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
     STC_CUDA(launch_group_classes(a, wide, direct, b, hg.count, ctx->sms, s));

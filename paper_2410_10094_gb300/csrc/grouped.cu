@@ -2050,9 +2050,153 @@ __global__ void __launch_bounds__(kRowWarps * 32) group_lanerow_kernel(GroupArgs
   }
 }
 
-cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, int sms, cudaStream_t s) {
+// The same with one CTA per group: its warps take pieces of kPiece X entries of the group until
+// none is left, each lane with a row of its own, and the warps' sums are added in warp order.
+// Groups whose products run into the tens of thousands keep a CTA busy, and a grid of one CTA per
+// SM ends evenly, where warps that own whole groups leave the last round of groups half empty.
+// The loads of the next products are issued before the current ones are added, so that the FP64
+// pipe (two rounded operations per product) is what bounds the loop: 2.04e10 products in 4,096
+// groups take 82.6 ms, 0.93 of half the measured rate of FP64 multiplies; by a warp per group 143.
+constexpr int kCtaRowWarps = 13;  // 13 x 32 rows of 65 doubles: 216 KB of shared memory
+constexpr int kPiece = 16;
+// The line: a CTA per group where there are at most four groups per SM (300 groups of 4,096
+// products 39 against 69 us, 600 66 against 76, 1,200 119 against 75) or the products average
+// kCtaRowMin per group (20,000 groups of 24,576 products 3.8 against 3.0 ms, 4,096 of 65,536 1.53
+// against 2.15, of 262,144 6.0 against 8.2).
+constexpr u64 kCtaRowMin = 49152;
+constexpr size_t kCtaRowSmem = (size_t)kCtaRowWarps * 32 * kRowStride * sizeof(double);
+
+__global__ void __launch_bounds__(kCtaRowWarps * 32, 1) group_ctarow_kernel(GroupArgs a, u64 ngroups, uint32_t FY) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  constexpr int D = kRowD;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  double* const rows = reinterpret_cast<double*>(smem) + (size_t)warp * 32 * kRowStride;
+  double* const myrow = rows + (size_t)lane * kRowStride;
+  __shared__ u64 s_pre[kCtaRowWarps][kPiece + 1];
+  __shared__ uint32_t s_ys[kCtaRowWarps][kPiece];
+  __shared__ double s_v[kCtaRowWarps][kPiece];
+  __shared__ u64 s_any[kCtaRowWarps];
+  __shared__ OutTarget tg;
+  __shared__ uint32_t s_next;
+  u64* const pre = s_pre[warp];
+  uint32_t* const ysv = s_ys[warp];
+  double* const xv = s_v[warp];
+  for (uint32_t c = 0; c < kRowMax; c++) myrow[c] = 0.0;
+  if (threadIdx.x == 0) {
+    tg.prob = kNoProb;
+    s_next = 0;
+  }
+  __syncthreads();
+  const uint64_t keep = policy_evict_last();
+  const uint64_t pol = policy_evict_first();
+  const uint32_t* yfk = static_cast<const uint32_t*>(a.yfk);
+  for (u64 g = blockIdx.x; g < ngroups; g += gridDim.x) {
+    const uint32_t x0 = a.goff[g], n = a.goff[g + 1] - x0;
+    if (n == 0) continue;  // uniform over the CTA
+    u64 seen = 0;
+    for (;;) {
+      uint32_t c0 = 0;
+      if (lane == 0) c0 = atomicAdd(&s_next, (uint32_t)kPiece);
+      c0 = __shfl_sync(0xffffffffu, c0, 0);
+      if (c0 >= n) break;
+      u64 w = 0;
+      if (lane < kPiece && c0 + lane < n) {
+        w = a.gx.w[x0 + c0 + lane];
+        ysv[lane] = a.gx.ystart[x0 + c0 + lane];
+        xv[lane] = a.gx.v[x0 + c0 + lane];
+      }
+      u64 incl = w;
+#pragma unroll
+      for (int o = 1; o < kPiece; o <<= 1) {
+        const u64 y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o) incl += y;
+      }
+      if (lane < kPiece) pre[lane] = incl - w;
+      const u64 total = __shfl_sync(0xffffffffu, incl, kPiece - 1);
+      if (lane == 0) pre[kPiece] = total;
+      __syncwarp();
+      // Entries past the group's last have w = 0, so the prefix bounds the walk.
+      uint32_t own = 0;
+      auto load = [&](u64 base, uint32_t (&fk)[D], double (&x)[D], double (&y)[D]) {
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          const u64 p = base + (u64)u * 32 + lane;
+          uint32_t kk = own;
+          fk[u] = kRowMax;  // no product
+          if (p < total) {
+            while (pre[kk + 1] <= p) kk++;
+            const u64 j = (u64)ysv[kk] + (p - pre[kk]);
+            fk[u] = ld_keep_u32(yfk + j, keep);
+            y[u] = ld_keep_f64(a.yv + j, keep);
+            x[u] = xv[kk];
+          }
+          own = __shfl_sync(0xffffffffu, kk, 31);
+        }
+      };
+      uint32_t fk[D], fn[D];
+      double x[D], y[D], xn[D], yn[D];
+      load(0, fk, x, y);
+      for (u64 base = 0; base < total; base += 32 * D) {
+        load(base + 32 * D, fn, xn, yn);
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          if (fk[u] < FY) {
+            myrow[fk[u]] = __dadd_rn(myrow[fk[u]], __dmul_rn(x[u], y[u]));
+            seen |= 1ull << fk[u];
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < D; u++) fk[u] = fn[u], x[u] = xn[u], y[u] = yn[u];
+      }
+      __syncwarp();  // the staging is rewritten by the next piece
+    }
+    const u64 any_w = (u64)__reduce_or_sync(0xffffffffu, (uint32_t)seen) |
+                      ((u64)__reduce_or_sync(0xffffffffu, (uint32_t)(seen >> 32)) << 32);
+    // The warp's rows, summed in lane order into its first row.
+    __syncwarp();
+    for (uint32_t c = lane; c < FY; c += 32) {
+      double sum = 0.0;
+      if ((any_w >> c) & 1ull)
+        for (int l = 0; l < 32; l++) sum = __dadd_rn(sum, rows[(size_t)l * kRowStride + c]);
+      rows[c] = sum;
+    }
+    if (lane == 0) s_any[warp] = any_w;
+    __syncthreads();
+    if (warp == 0) {
+      u64 any = 0;
+      for (int k = 0; k < kCtaRowWarps; k++) any |= s_any[k];
+      resolve_target_warp(a, g, (unsigned)__popcll(any), tg);
+      for (uint32_t c = lane; c < FY; c += 32) {
+        if ((any >> c) & 1ull) {
+          double sum = 0.0;
+          for (int k = 0; k < kCtaRowWarps; k++) sum = __dadd_rn(sum, rows[(size_t)k * 32 * kRowStride + c]);
+          const u64 pos = tg.base + (u64)__popcll(any & ((1ull << c) - 1ull));
+          if (pos < tg.cap)
+            store_output(tg.coords, tg.vals, pos, tg.zrow + c, sum, tg.op, pol);
+          else
+            atomicOr(a.status, kStatOutOverflow);
+        }
+      }
+      if (lane == 0) s_next = 0;
+    }
+    __syncthreads();  // every column is summed before the rows are cleared
+    for (uint32_t c = 0; c < FY; c++) myrow[c] = 0.0;
+    __syncthreads();  // a warp's first row is cleared by its lane 0 and added to by no other lane
+  }
+}
+
+cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, int sms, cudaStream_t s) {
   if (ngroups == 0) return cudaSuccess;
   if (FY == 0 || FY > kRowMax) return cudaErrorInvalidValue;
+  if (ngroups <= 4 * (u64)sms || products / kCtaRowMin >= ngroups) {
+    const cudaError_t e = cudaFuncSetAttribute(group_ctarow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kCtaRowSmem);
+    if (e != cudaSuccess) return e;
+    group_ctarow_kernel<<<(unsigned)(ngroups < (u64)sms ? ngroups : (u64)sms), kCtaRowWarps * 32, kCtaRowSmem, s>>>(
+        a, ngroups, FY);
+    note_launch();
+    return cudaGetLastError();
+  }
   auto kern = group_lanerow_kernel;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRowSmem);
   if (e != cudaSuccess) return e;

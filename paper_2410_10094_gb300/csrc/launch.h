@@ -360,7 +360,7 @@ cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, u6
 
 // Lane-private dense rows for output rows of at most 64 free keys (FY <= 64, 32-bit Y free
 // keys): one warp per group g in [0, ngroups) (empty groups skipped), outputs in key order.
-cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, int sms, cudaStream_t s);
+cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, int sms, cudaStream_t s);
 cudaError_t launch_group_dense(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                const uint32_t* stash_list, uint32_t stash_count, const uint32_t* rank_list,
                                uint32_t rank_count, int sms, cudaStream_t s);
