@@ -227,6 +227,13 @@ struct Arena {
     *out = static_cast<T*>(p);
     return STC_OK;
   }
+  // Gives one block back, in stream order.
+  void release(void* p) {
+    const size_t b = keep(p);
+    if (!b) return;
+    cudaFreeAsync(p, s);
+    ctx->held -= b;
+  }
   size_t keep(void* p) {
     for (size_t i = 0; i < blocks.size(); i++)
       if (blocks[i].p == p) {
@@ -615,7 +622,7 @@ uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
   uint64_t b = sizeof(Counters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
   b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
-  b += out * (4ull * pl.ocols + 8);
+  b += out * (4ull * pl.ocols + 8);  // the positions chunked reservations leave over only where there is room
   return b;
 }
 
@@ -731,15 +738,32 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
                           (o.accumulator == STC_ACC_AUTO && h.P >= kRowsMinPerOutput * pl.FX * pl.FY));
   if (lane_rows) r->stats.accumulator = STC_ACC_ROWS;
 
-  const uint64_t out_cap = hg.out_cap;
+  uint64_t out_cap = hg.out_cap;
   HugeGroups hh{};
   hh.count = lane_rows ? 0u : hg.count[kMaxClasses];
   hh.countp = gc->count + kMaxClasses;
   hh.list = b.huge_list;
   hh.off = b.huge_off;
   hh.cap = b.huge_cap;
-  STC_TRY(ar.alloc(&r->coords, out_cap * (size_t)pl.ocols));
-  STC_TRY(ar.alloc(&r->vals, out_cap));
+  const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
+  bool direct = !wide && !lane_rows && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
+  // Room for the positions that chunked reservations may leave over, where the budget has it.
+  uint32_t chunk = direct ? warp_chunk(hg.count, out_cap, ctx->sms) : 0u;
+  const uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
+  if (out_cap + slack >= 0xffffffffull ||
+      (chunk && (ar.alloc(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
+                 ar.alloc(&r->vals, out_cap + slack) != STC_OK))) {
+    chunk = 0;
+    if (r->coords) ar.release(r->coords);
+    r->coords = nullptr;
+    r->vals = nullptr;
+  }
+  if (chunk) {
+    out_cap += slack;
+  } else {
+    STC_TRY(ar.alloc(&r->coords, out_cap * (size_t)pl.ocols));
+    STC_TRY(ar.alloc(&r->vals, out_cap));
+  }
   if (hh.count) {
     STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
     STC_TRY(ar.alloc(&hh.vals, hg.huge_slots));
@@ -769,30 +793,32 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   a.status = &pr.ctr->status;
   a.bout = dbo;
   a.bnz = &pr.ctr->nz;
+  StreamArgs sa{};
+  if (nstream || chunk) {
+    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms) +
+                                    (chunk ? warp_chunk_warps(hg.count, ctx->sms) : 0u)));
+    sa.nholes = &gc->nholes;
+    sa.hole_total = &gc->holes;
+    sa.ny_entries = (uint32_t)Y->nnz;
+    a.chunk = chunk;
+    a.holes = sa.holes;
+    a.nholes = sa.nholes;
+    a.hole_total = sa.hole_total;
+  }
   if (lane_rows) {
     STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, h.P, ctx->sms, s));
   } else {
-    const bool direct = !wide && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
     STC_CUDA(launch_group_classes(a, wide, direct, b, hg.count, ctx->sms, s));
     STC_CUDA(launch_group_huge(a, hh, wide, ctx->sms, s));
   }
-  const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
-  StreamArgs sa{};
   if (dense_rows && !lane_rows) {
-    // Streamed groups go last: every other kernel's outputs then lie below the final count.
     STC_CUDA(launch_group_dense(a, pr.yoff, nseg, seg, b.dense_list[2], hg.count[kMaxClasses + 3], b.dense_list[1],
                                 hg.count[kMaxClasses + 2], ctx->sms, s));
-    if (nstream) {
-      STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms)));
-      sa.nholes = &gc->nholes;
-      sa.hole_total = &gc->holes;
-      sa.ny_entries = (uint32_t)Y->nnz;
-      STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, ctx->sms, s));
-    }
+    STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, ctx->sms, s));
   }
   tm.mark(4);
   u64 holes = 0;
-  if (nstream) STC_CUDA(cudaMemcpyAsync(&holes, &gc->holes, sizeof(u64), cudaMemcpyDeviceToHost, s));
+  if (nstream || chunk) STC_CUDA(cudaMemcpyAsync(&holes, &gc->holes, sizeof(u64), cudaMemcpyDeviceToHost, s));
   Counters h2{};
   STC_TRY(read_counters(pr, s, h2));
   r->nnz = (int64_t)(h2.nz - holes);

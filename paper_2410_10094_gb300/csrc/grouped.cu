@@ -7,6 +7,8 @@
 // key, Section 4.1.1), groups are binned by table size class, and each class runs one
 // persistent kernel whose CTAs take one group at a time with the table in shared memory.
 // Groups too large for shared memory use a table region in global memory.
+#include <algorithm>
+
 #include "launch.h"
 
 namespace stc {
@@ -45,24 +47,46 @@ __global__ void __launch_bounds__(kThreads) x_group_scatter_kernel(Survivors sv,
   }
 }
 
-// One warp per X free key g: the group's bound B_g (Section 4.3) is the sum of its entries'
-// run lengths, read from the grouped X. Non-empty groups go to the first class whose table
-// holds t = min(B_g, F_Y); larger ones get a region of the overflow table.
+// The bound B_g of every X free key's group (Section 4.3) is the sum of its entries' run lengths,
+// read from the grouped X. Non-empty groups go to the first class whose table holds
+// t = min(B_g, F_Y); larger ones get a region of the overflow table. A warp takes `per` consecutive
+// groups, one per lane: short ones are summed by their lane, long ones by all lanes in turn; then
+// each list gets one reservation for the warp's groups. (With a warp and a reservation per group,
+// the counters' atomics took 0.27 ms for 4e5 groups, each on one of a few addresses.)
 __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint32_t* __restrict__ goff,
-                                                              const uint32_t* __restrict__ gw, u64 FY, Bins b) {
+                                                              const uint32_t* __restrict__ gw, u64 FY, Bins b,
+                                                              uint32_t per) {
   __shared__ u64 s_cap[kThreads / 32];
   const unsigned lane = lane_id();
   u64 my_cap = 0;
-  for (u64 g = (u64)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); g < FX;
-       g += (u64)gridDim.x * (kThreads / 32)) {
-    const uint32_t x0 = goff[g], x1 = goff[g + 1];
-    if (x0 == x1) continue;
+  for (u64 g0 = ((u64)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * per; g0 < FX;
+       g0 += (u64)gridDim.x * (kThreads / 32) * per) {
+    const u64 g = g0 + lane;
+    uint32_t x0 = 0, x1 = 0;
+    if (lane < per && g < FX) {
+      x0 = goff[g];
+      x1 = goff[g + 1];
+    }
     u64 bnd = 0;
-    for (uint32_t i = x0 + lane; i < x1; i += 32) bnd += gw[i];
+    if (__any_sync(0xffffffffu, x1 - x0 > 8)) {
+      unsigned todo = __ballot_sync(0xffffffffu, x1 > x0);
+      while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const uint32_t a = __shfl_sync(0xffffffffu, x0, l), e = __shfl_sync(0xffffffffu, x1, l);
+        u64 sum = 0;
+        for (uint32_t i = a + lane; i < e; i += 32) sum += gw[i];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) bnd += __shfl_xor_sync(0xffffffffu, bnd, o);
-    if (lane == 0) {
-      const u64 t = bnd < FY ? bnd : FY;
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((int)lane == l) bnd = sum;
+      }
+    } else {
+      for (uint32_t i = x0; i < x1; i++) bnd += gw[i];
+    }
+    // list: 0..kMaxClasses-1 the classes, kMaxClasses the overflow groups, then the dense lists.
+    int list = -1;
+    const u64 t = bnd < FY ? bnd : FY;
+    if (x1 > x0) {
       int c = 0;
       while (c < b.nclasses && t > b.tmax[c]) c++;
       if (b.dense_list[0] && t >= b.dense_min) {
@@ -74,17 +98,32 @@ __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint
         const bool stashed = bnd <= b.stash_cap;
         const int d = bnd <= b.stream_cap && (4 * bnd <= 3 * FY || (!stashed && bnd <= FY)) ? 0 : (stashed ? 2 : 1);
         my_cap += d == 0 ? bnd : t;
-        const uint32_t idx = atomicAdd(b.count + kMaxClasses + 1 + d, 1u);
-        b.dense_list[d][idx] = (uint32_t)g;
+        list = kMaxClasses + 1 + d;
       } else if (c < b.nclasses) {
         my_cap += t;
-        const uint32_t idx = atomicAdd(b.count + c, 1u);
-        b.list[c][idx] = (uint32_t)g;
+        list = c;
       } else if (t > (1ull << 30)) {
         atomicOr(b.status, kStatTooLarge);
       } else {
         my_cap += t;
-        const uint32_t idx = atomicAdd(b.count + kMaxClasses, 1u);
+        list = kMaxClasses;
+      }
+    }
+    unsigned todo = __ballot_sync(0xffffffffu, list >= 0);
+    while (todo) {
+      const int l = __ffs(todo) - 1;
+      const int cur = __shfl_sync(0xffffffffu, list, l);
+      const unsigned in = __ballot_sync(0xffffffffu, list == cur);
+      todo &= ~in;
+      uint32_t idx = 0;
+      if ((int)lane == l) idx = atomicAdd(b.count + cur, (uint32_t)__popc(in));
+      idx = __shfl_sync(0xffffffffu, idx, l) + __popc(in & lanemask_lt());
+      if (list != cur) continue;
+      if (cur < kMaxClasses) {
+        b.list[cur][idx] = (uint32_t)g;
+      } else if (cur > kMaxClasses) {
+        b.dense_list[cur - kMaxClasses - 1][idx] = (uint32_t)g;
+      } else {
         u64 cap = 64;
         while (cap < 2 * t) cap <<= 1;
         b.huge_list[idx] = (uint32_t)g;
@@ -93,6 +132,8 @@ __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint
       }
     }
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) my_cap += __shfl_xor_sync(0xffffffffu, my_cap, o);
   if (lane == 0) s_cap[threadIdx.x >> 5] = my_cap;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -134,6 +175,14 @@ __device__ __forceinline__ void resolve_target_warp(const GroupArgs& a, u64 g, u
   p = __shfl_sync(0xffffffffu, p, 0);
   const bool fresh = t.prob != p;
   __syncwarp();  // every lane has read t.prob before lane 0 rewrites it
+  if (!fresh && !a.gprob) {  // a single contraction's next group: only the row and the base differ
+    if (lane == 0) {
+      t.zrow = g * t.FY;
+      t.base = n ? atomicAdd(t.counter, (u64)n) : 0;
+    }
+    __syncwarp();
+    return;
+  }
   const BatchOut* bo = a.bout + p;
   if (fresh) {
     const u64* src = reinterpret_cast<const u64*>(&bo->op);
@@ -1703,6 +1752,210 @@ cudaError_t launch_warp_direct_class(const GroupArgs& a, const uint32_t* list, c
   return cudaGetLastError();
 }
 
+// ---- small groups of a single contraction: a warp takes PK groups at a time and treats their X
+// entries as one list, with one table whose keys carry the group's number in their top bits, so that
+// PK groups share every load, scan and table clearing that a group alone would wait for. Output
+// positions come from chunks that the warp reserves (GroupArgs::chunk): all groups of the contraction
+// draw on one counter, whose atomics serialise. Otherwise as group_warp_direct_kernel.
+// Measured on 4e5 groups of 63 products (lengths 100, order 5 with order 4, 5e5 entries each): 0.61
+// against 0.88 ms; on 4,096 groups of 95 the four groups of a warp wait for one another longer than
+// the idle warps would help (60 against 40 us), so few groups keep a warp each.
+constexpr uint32_t kPackMinGroups = 16384;
+constexpr uint32_t kPackSlots = 1024;
+constexpr uint32_t kPackBits = 30;  // bits of the free key where PK > 1
+struct alignas(16) PackSlice {
+  uint32_t keys[kPackSlots];
+  uint32_t spos[kPackSlots];  // output position of the key in the slot
+  u64 pre[33];
+  u64 zrow[4];
+  uint32_t ystart[32];
+  uint32_t top[32];  // the entry's group, in the key's top bits
+  double v[32];
+};
+
+template <int PK, int D>
+__global__ void __launch_bounds__(256) group_pack_kernel(const __grid_constant__ GroupArgs a,
+                                                         const uint32_t* __restrict__ list,
+                                                         const uint32_t* __restrict__ countp) {
+  constexpr int WARPS = 8;
+  const uint32_t count = *countp;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint32_t lt = lanemask_lt();
+  PackSlice& ws = reinterpret_cast<PackSlice*>(smem)[warp];
+  for (uint32_t i = lane; i < kPackSlots / 4; i += 32)
+    reinterpret_cast<uint4*>(ws.keys)[i] = make_uint4(kEmpty32, kEmpty32, kEmpty32, kEmpty32);
+  __syncwarp();
+  const uint64_t keep = policy_evict_last();
+  const uint64_t pol = policy_evict_first();
+  const uint32_t* const yfk = static_cast<const uint32_t*>(a.yfk);
+  u64 cur = 0;  // positions [cur, cur + rem) are this warp's to fill
+  uint32_t rem = 0;
+  const uint32_t packs = (count + PK - 1) / PK, step = gridDim.x * WARPS;
+  // The next pack's groups (lane q holds the q-th) and their entries' ranges are loaded ahead.
+  uint32_t g_n = 0, x0_n = 0, x1_n = 0, g_nn = 0;
+  auto number = [&](uint32_t pk) {
+    return lane < PK && pk < packs && pk * PK + lane < count ? __ldg(list + pk * PK + lane) : kEmpty32;
+  };
+  auto range = [&]() {
+    x0_n = x1_n = 0;
+    if (g_n != kEmpty32) {
+      x0_n = __ldg(a.goff + g_n);
+      x1_n = __ldg(a.goff + g_n + 1);
+    }
+  };
+  const uint32_t pk0 = blockIdx.x * WARPS + warp;
+  g_n = number(pk0);
+  range();
+  g_nn = packs - 1 >= step && pk0 < packs - step ? number(pk0 + step) : kEmpty32;
+  for (uint32_t pk = pk0; pk < packs; pk += step) {
+    const uint32_t x0 = x0_n, n = x1_n - x0_n;
+    if (lane < PK) ws.zrow[lane] = (u64)g_n * a.FY;
+    const bool more = packs - pk > step;
+    g_n = g_nn;
+    if (more) {
+      range();
+      g_nn = packs - pk - step > step ? number(pk + 2 * step) : kEmpty32;
+    }
+    // Entry e of the pack belongs to group q where off_q <= e < off_{q+1}.
+    uint32_t incl_n = n;
+    if (PK > 1) {
+#pragma unroll
+      for (int o = 1; o < PK; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl_n, o);
+        if ((int)lane >= o) incl_n += y;
+      }
+    }
+    const uint32_t total_n = __shfl_sync(0xffffffffu, incl_n, PK - 1);
+    const uint32_t from = x0 - (incl_n - n);  // lane q: what an entry's number in the pack adds to
+    for (uint32_t c0 = 0; c0 < total_n; c0 += 32) {
+      const uint32_t e = c0 + lane;
+      uint32_t q = 0;
+#pragma unroll
+      for (int i = 0; i + 1 < PK; i++) q += e >= __shfl_sync(0xffffffffu, incl_n, i);
+      const uint32_t xi = __shfl_sync(0xffffffffu, from, q) + e;
+      u64 w = 0;
+      if (e < total_n) {
+        w = __ldg(a.gx.w + xi);
+        ws.ystart[lane] = __ldg(a.gx.ystart + xi);
+        ws.v[lane] = __ldg(a.gx.v + xi);
+        if (PK > 1) ws.top[lane] = q << kPackBits;
+      }
+      u64 incl = w;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const u64 y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o) incl += y;
+      }
+      ws.pre[lane] = incl - w;
+      const u64 total = __shfl_sync(0xffffffffu, incl, 31);
+      if (lane == 0) ws.pre[32] = total;
+      __syncwarp();
+      // Entries past the last have w = 0, so the prefix bounds the walk.
+      uint32_t own = 0;
+      for (u64 base = 0; base < total; base += 32 * D) {
+        uint32_t key[D];
+        double prod[D];
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          const u64 p = base + (u64)u * 32 + lane;
+          uint32_t kk = own;
+          key[u] = kEmpty32;
+          if (p < total) {
+            while (ws.pre[kk + 1] <= p) kk++;
+            const u64 j = (u64)ws.ystart[kk] + (p - ws.pre[kk]);
+            key[u] = ld_keep_u32(yfk + j, keep);
+            if (PK > 1) key[u] |= ws.top[kk];
+            prod[u] = __dmul_rn(ws.v[kk], ld_keep_f64(a.yv + j, keep));
+          }
+          own = __shfl_sync(0xffffffffu, kk, 31);
+        }
+        int slot[D];
+        uint32_t m[D];
+        uint32_t nclaim = 0;
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          slot[u] = -1;
+          bool mine = false;
+          if (key[u] != kEmpty32) {
+            slot[u] = bucket_claim<uint32_t, kPackSlots>(ws.keys, key[u], &mine);
+            if (slot[u] < 0) atomicOr(a.status, kStatTableFull);
+          }
+          m[u] = __ballot_sync(0xffffffffu, mine);
+          nclaim += __popc(m[u]);
+        }
+        // nclaim positions: the i-th is pa + i below na, pb + i from there on.
+        u64 pa = cur, pb = 0;
+        uint32_t na = nclaim;
+        if (nclaim <= rem) {
+          cur += nclaim;
+          rem -= nclaim;
+        } else {
+          const uint32_t extra = nclaim - rem, size = extra > a.chunk ? extra : a.chunk;
+          u64 nb = 0;
+          if (lane == 0) nb = atomicAdd(a.nz, (u64)size);
+          nb = __shfl_sync(0xffffffffu, nb, 0);
+          na = rem;
+          pb = nb - rem;
+          cur = nb + extra;
+          rem = size - extra;
+        }
+        uint32_t off = 0;
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          if ((m[u] >> lane) & 1u) {
+            const uint32_t i = off + __popc(m[u] & lt);
+            const u64 pos = i + (i < na ? pa : pb);
+            ws.spos[slot[u]] = (uint32_t)pos;
+            const uint32_t fk = PK > 1 ? key[u] & ((1u << kPackBits) - 1u) : key[u];
+            if (pos < a.out_cap)
+              store_output(a.coords, a.vals, pos, ws.zrow[PK > 1 ? key[u] >> kPackBits : 0] + fk, prod[u], a.op, pol);
+            else
+              atomicOr(a.status, kStatOutOverflow);
+          }
+          off += __popc(m[u]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < D; u++) {
+          if (slot[u] >= 0 && !((m[u] >> lane) & 1u)) {
+            const u64 pos = ws.spos[slot[u]];
+            if (pos < a.out_cap) atomicAdd(a.vals + pos, prod[u]);
+          }
+        }
+      }
+      __syncwarp();  // the staging is rewritten by the next entries
+    }
+    for (uint32_t i = lane; i < kPackSlots / 4; i += 32)
+      reinterpret_cast<uint4*>(ws.keys)[i] = make_uint4(kEmpty32, kEmpty32, kEmpty32, kEmpty32);
+    __syncwarp();
+  }
+  if (rem && lane == 0) {
+    a.holes[atomicAdd(a.nholes, 1u)] = StreamHole{cur, rem};
+    atomicAdd(a.hole_total, (u64)rem);
+  }
+}
+
+template <int PK>
+cudaError_t launch_pack(const GroupArgs& a, const uint32_t* list, const uint32_t* countp, uint32_t count, int sms,
+                        cudaStream_t s) {
+  if (count == 0) return cudaSuccess;
+  constexpr int WARPS = 8;
+  const size_t smem = WARPS * sizeof(PackSlice);
+  auto kern = group_pack_kernel<PK, 4>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WARPS * 32, smem);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) per_sm = 1;
+  const uint32_t need = (count + PK * WARPS - 1) / (PK * WARPS);
+  const uint32_t cap = (uint32_t)(sms * (per_sm > 8 ? 8 : per_sm));
+  kern<<<need < cap ? need : cap, WARPS * 32, smem, s>>>(a, list, countp);
+  note_launch();
+  return cudaGetLastError();
+}
+
 // ---- direct output: a product that claims a new key writes its output entry at once.
 // The table holds keys and output positions only. A claimer takes a rank inside its round
 // (warp-aggregated); after the round's claims are counted, one atomic per round reserves the
@@ -1901,9 +2154,26 @@ cudaError_t launch_x_group_scatter(Survivors sv, uint32_t* gcur, GroupedX gx, in
 cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, u64 FY, const Bins& b, int sms,
                               cudaStream_t s) {
   if (FX == 0) return cudaSuccess;
-  bin_groups_kernel<<<grid_for((int64_t)FX * 32, sms), kThreads, 0, s>>>(FX, goff, gw, FY, b);
+  // Up to 32 groups per warp, as long as that leaves every SM its 64 warps.
+  const u64 warps = (u64)sms * 64;
+  const uint32_t per = (uint32_t)(FX >= 32 * warps ? 32 : (FX + warps - 1) / warps);
+  bin_groups_kernel<<<grid_for((int64_t)((FX + per - 1) / per) * 32, sms), kThreads, 0, s>>>(FX, goff, gw, FY, b, per);
   note_launch();
   return cudaGetLastError();
+}
+
+uint32_t warp_chunk_warps(const uint32_t* counts, int sms) {
+  const uint32_t most = (uint32_t)sms * 64;
+  return std::min(counts[0], most) + std::min(counts[1], most);
+}
+
+// One reservation per group and round would be one atomic on the same address each, at about 0.7 ns:
+// 0.27 ms for 4e5 groups. Chunks of up to 512 positions per warp cost at most half of the output's
+// bound in positions left over, which are filled from the output's end.
+uint32_t warp_chunk(const uint32_t* counts, u64 out_cap, int sms) {
+  if ((u64)counts[0] + counts[1] < kPackMinGroups) return 0;
+  const u64 c = out_cap / (2 * (u64)warp_chunk_warps(counts, sms));
+  return c < 32 ? 0 : (uint32_t)(c < 512 ? c : 512);
 }
 
 cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct, const Bins& b,
@@ -1914,7 +2184,13 @@ cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct
   uint32_t h[kMaxClasses];
   for (int c = 0; c < kMaxClasses; c++) h[c] = counts ? counts[c] : kCountOnDevice;
   const uint32_t* d = b.count;
-  if (!wide_keys && direct) {
+  if (!wide_keys && direct && !a.gprob && a.FY < (1u << kPackBits) && counts &&
+      (u64)h[0] + h[1] >= kPackMinGroups) {
+    // Small groups of a single contraction, many of them. Four share a table of 1,024 slots where
+    // each takes at most 256 (and the load factor leaves room, as it does for one group in 256).
+    if ((e = launch_pack<4>(a, b.list[0], d + 0, h[0], sms, s))) return e;
+    if ((e = launch_pack<1>(a, b.list[1], d + 1, h[1], sms, s))) return e;
+  } else if (!wide_keys && direct) {
     // The expansion split: products each lane forms per round before the claims of the round.
     if (depth == 0) {
       if ((e = launch_warp_direct_class<256, 4>(a, b.list[0], d + 0, h[0], sms, s))) return e;
@@ -1923,6 +2199,8 @@ cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct
       if ((e = launch_warp_direct_class<256, 2>(a, b.list[0], d + 0, h[0], sms, s))) return e;
       if ((e = launch_warp_direct_class<1024, 2>(a, b.list[1], d + 1, h[1], sms, s))) return e;
     }
+  }
+  if (!wide_keys && direct) {
     if (depth == 0) {
       if ((e = launch_direct_class<4096, 256, 6, 4>(a, b.list[2], d + 2, h[2], sms, s))) return e;
       if ((e = launch_direct_class<8192, 512, 6, 2>(a, b.list[3], d + 3, h[3], sms, s))) return e;

@@ -188,6 +188,12 @@ struct BatchOut {
 };
 static_assert(sizeof(OutPlan) % 8 == 0, "OutPlan must be a whole number of 8-byte words");
 
+// Positions reserved for outputs that none took.
+struct StreamHole {
+  u64 pos;
+  u64 len;
+};
+
 struct GroupArgs {
   const uint32_t* goff;
   GroupedX gx;
@@ -211,6 +217,12 @@ struct GroupArgs {
   // different (run_unique_kernel). A group of one X entry over such a run has one product per
   // output, and the warp kernels write it as a scaled copy of the run without a table.
   const uint8_t* yuniq;
+  // Single contractions: warps of the small classes reserve positions `chunk` at a time (0: as
+  // many as they need) and list what they leave (room for warp_chunk_warps holes).
+  uint32_t chunk;
+  StreamHole* holes;
+  unsigned* nholes;
+  u64* hole_total;
 };
 
 // Where one group's outputs go, resolved once per group.
@@ -252,6 +264,10 @@ cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, 
 cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct, const Bins& b,
                                  const uint32_t* counts, int sms, cudaStream_t s, int depth = 0);
 cudaError_t launch_group_huge(const GroupArgs& a, const HugeGroups& h, bool wide_keys, int sms, cudaStream_t s);
+// Most warps that the warp classes' direct kernels run for these counts, and the chunk of
+// positions each should reserve at a time (GroupArgs::chunk).
+uint32_t warp_chunk_warps(const uint32_t* counts, int sms);
+uint32_t warp_chunk(const uint32_t* counts, u64 out_cap, int sms);
 
 // ------------------------------------------------------------------ batches (batch.cu)
 // One problem of a batch as the device kernels see it.
@@ -330,11 +346,6 @@ constexpr size_t kBitmapSmemPerCta = 112 * 1024;  // two CTAs per SM
 uint32_t dense_stash_cap();
 
 // ------------------------------------------------------------------ streamed groups (stream.cu)
-// Positions reserved by the streaming kernel that no output took.
-struct StreamHole {
-  u64 pos;
-  u64 len;
-};
 struct StreamArgs {
   StreamHole* holes;    // [stream_max_holes]
   unsigned* nholes;
@@ -348,8 +359,6 @@ struct StreamArgs {
 };
 uint32_t stream_cap();  // most products of a streamed group
 size_t stream_max_holes(uint32_t count, uint32_t nseg, int sms);
-// Launched after every other accumulation kernel, so that the positions it reserves are the last
-// ones.
 cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                 const uint32_t* list, uint32_t count, const StreamArgs& sa, int sms, cudaStream_t s);
 // Moves the entries at and above nnz into the holes below it. total: positions of all holes;
