@@ -53,7 +53,12 @@ struct stc_ctx {
   // survey, and the one-global-table path for small output key spaces never waits for it).
   std::mutex rows_mu;
   std::set<uint64_t> rows_shapes;
+  // Page-locked blocks of kPinnedBytes for the counters that calls read back and the small
+  // descriptors they send: as many as calls have run at once, given back with the context.
+  std::mutex pin_mu;
+  std::vector<void*> pins;
 };
+constexpr size_t kPinnedBytes = 2048;
 
 namespace {
 // Picks the load factor for a batch of this bucket; *measure is the candidate to time (or -1).
@@ -191,13 +196,54 @@ struct DeviceGuard {
   }
 };
 
+// One page-locked block of the context's for the duration of a call. Copies to and from it are
+// asynchronous, so it goes back only when the stream has passed them: calls wait for their stream
+// before they return, and a call that fails in between waits here.
+struct Pinned {
+  stc_ctx* ctx;
+  cudaStream_t s;
+  void* p = nullptr;
+  bool busy = false;  // a copy may be in flight
+  Pinned(stc_ctx* c, cudaStream_t st) : ctx(c), s(st) {
+    {
+      std::lock_guard<std::mutex> lk(ctx->pin_mu);
+      if (!ctx->pins.empty()) {
+        p = ctx->pins.back();
+        ctx->pins.pop_back();
+      }
+    }
+    if (!p && cudaMallocHost(&p, kPinnedBytes) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  Pinned(const Pinned&) = delete;
+  Pinned& operator=(const Pinned&) = delete;
+  ~Pinned() {
+    if (!p) return;
+    if (busy) cudaStreamSynchronize(s);
+    try {
+      std::lock_guard<std::mutex> lk(ctx->pin_mu);
+      ctx->pins.push_back(p);
+    } catch (...) {
+      cudaFreeHost(p);
+    }
+  }
+};
+
 // Stream-ordered scratch from the context's pool. Everything still held when the arena
 // dies is returned to the pool in stream order; `keep` hands a block to a result instead.
+// In a context without a budget, small requests share slabs of kSlab bytes: a call makes some
+// thirty of them, at about a microsecond of host time each to take and to return. (A budget
+// counts every request for itself.)
 struct Arena {
+  static constexpr size_t kSlab = 1 << 20, kSlabMost = 1 << 16;
   stc_ctx* ctx;
   cudaStream_t s;
   struct Block { void* p; size_t bytes; };
   std::vector<Block> blocks;
+  char* slab = nullptr;
+  size_t slab_left = 0;
   Arena(stc_ctx* c, cudaStream_t st) : ctx(c), s(st) {}
   ~Arena() {
     for (auto& b : blocks) {
@@ -207,6 +253,22 @@ struct Arena {
   }
   template <typename T>
   stc_status alloc(T** out, size_t count) {
+    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;
+    if (bytes == 0 || bytes > kSlabMost || ctx->budget) return alloc_own(out, count);
+    if (bytes > slab_left) {
+      char* p = nullptr;
+      if (alloc_own(&p, kSlab) != STC_OK) return alloc_own(out, count);
+      slab = p;
+      slab_left = kSlab;
+    }
+    *out = reinterpret_cast<T*>(slab);
+    slab += bytes;
+    slab_left -= bytes;
+    return STC_OK;
+  }
+  // A block of its own, which `keep` and `release` can find.
+  template <typename T>
+  stc_status alloc_own(T** out, size_t count) {
     *out = nullptr;
     const size_t bytes = count * sizeof(T);
     if (bytes == 0) return STC_OK;
@@ -468,6 +530,22 @@ struct Counters {
   uint32_t status; // kStat* bits
 };
 
+// Counters of the grouping and binning passes.
+struct GroupCounters {
+  uint32_t count[kMaxClasses + 4];
+  unsigned nholes;       // pieces of reservations that hold no output
+  u64 huge_slots;
+  u64 out_cap;
+  u64 holes;             // their positions
+  u64 fill_counters[2];
+};
+
+// What a contraction reads back, in one copy.
+struct CallCounters {
+  Counters c;
+  GroupCounters g;
+};
+
 // Per-stage CUDA events when timing is requested.
 struct StageTimer {
   bool on = false;
@@ -518,7 +596,7 @@ struct Prepared {
   bool key32 = false;
   double* yv = nullptr;      // [nY]
   Survivors sv{};
-  Counters* ctr = nullptr;
+  Counters* ctr = nullptr;   // of a CallCounters
   uint32_t* gcnt = nullptr;  // [FX] entries with a Y run per X free key (GROUPED only)
   bool dense = false;        // GROUPED without a survivor list (X re-read by the scatter)
   bool keep_ck = false;      // survivors keep their contract key (dense-row accumulation)
@@ -536,15 +614,20 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
     return fail(STC_ERR_UNSUPPORTED, "contract key space %llu exceeds %llu bins", (unsigned long long)pl.K,
                 (unsigned long long)kMaxDirectBins);
   const int64_t nX = X->nnz, nY = Y->nnz;
-  STC_TRY(ar.alloc(&pr.ctr, 1));
-  STC_CUDA(cudaMemsetAsync(pr.ctr, 0, sizeof(Counters), s));
+  CallCounters* cc = nullptr;
+  STC_TRY(ar.alloc(&cc, 1));
+  pr.ctr = &cc->c;
+  STC_CUDA(cudaMemsetAsync(cc, 0, sizeof(CallCounters), s));
   uint32_t* status = &pr.ctr->status;
 
   // Y: count per contract key, exclusive scan, scatter (Section 4.1.1 counting sort).
   uint32_t *ycnt = nullptr, *ycur = nullptr, *scr = nullptr;
   // The Y counts and, past them, the bitmap of contract keys with entries (one clearing).
   const uint64_t ne_words = (mode != Survey::kDenseGroups && pl.K <= kNonemptyMaxKeys) ? (pl.K + 31) / 32 : 0;
-  STC_TRY(ar.alloc(&ycnt, bins + ne_words));
+  // and, past that, the entries per X free key
+  const uint64_t counts = bins + ne_words + (groups ? pl.FX : 0);
+  STC_TRY(ar.alloc(&ycnt, counts));
+  if (groups) pr.gcnt = ycnt + bins + ne_words;
   STC_TRY(ar.alloc(&pr.yoff, bins + 1));
   STC_TRY(ar.alloc(&ycur, bins));
   STC_TRY(ar.alloc(&scr, (size_t)scan_scratch_elems((int64_t)bins)));
@@ -562,7 +645,6 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
   // X's arrays too, before any launch: the stages' events then enclose device work, not the
   // host's allocation calls.
   pr.sv.count = &pr.ctr->ns;
-  if (groups) STC_TRY(ar.alloc(&pr.gcnt, pl.FX));
   pr.dense = mode == Survey::kDenseGroups;
   uint32_t* nonempty = nullptr;
   if (!pr.dense) {
@@ -573,15 +655,13 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
     STC_TRY(ar.alloc(&pr.sv.v, (size_t)nX));
     if (ne_words) nonempty = ycnt + bins;
   }
-  STC_CUDA(cudaMemsetAsync(ycnt, 0, (bins + ne_words) * sizeof(uint32_t), s));
+  STC_CUDA(cudaMemsetAsync(ycnt, 0, counts * sizeof(uint32_t), s));
   STC_CUDA(launch_y_count(Y->coords, nY, pl.ky, ycnt, status, ctx->sms, s, nonempty));
-  STC_CUDA(scan_u32(ycnt, pr.yoff, (int64_t)bins, scr, s));
-  STC_CUDA(cudaMemcpyAsync(ycur, pr.yoff, bins * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+  STC_CUDA(scan_u32(ycnt, pr.yoff, (int64_t)bins, scr, s, ycur));
   STC_CUDA(launch_y_scatter(Y->coords, Y->vals, nY, pl.ky, pl.FY, ycur, pr.yfk, pr.key32, pr.yv, ctx->sms, s));
   tm.mark(0);
 
   // X: find each entry's Y run and count the products exactly (Section 4.3).
-  if (groups) STC_CUDA(cudaMemsetAsync(pr.gcnt, 0, pl.FX * sizeof(uint32_t), s));
   if (pr.dense) {
     STC_CUDA(launch_x_count(X->coords, nX, pl.kx, pr.yoff, &pr.ctr->P, pr.gcnt, status, ctx->sms, s));
   } else {
@@ -592,10 +672,21 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
   return STC_OK;
 }
 
-stc_status read_counters(const Prepared& pr, cudaStream_t s, Counters& h) {
-  STC_CUDA(cudaMemcpyAsync(&h, pr.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
-  STC_CUDA(cudaStreamSynchronize(s));
-  return status_word(h.status);
+// Reads the call's counters back and waits for the stream; the status word is the caller's to look at.
+stc_status copy_counters(const Prepared& pr, Pinned& pin, CallCounters& h) {
+  static_assert(sizeof(CallCounters) <= kPinnedBytes / 2, "a page-locked block holds the counters and a descriptor");
+  CallCounters* const to = pin.p ? static_cast<CallCounters*>(pin.p) : &h;
+  pin.busy = true;
+  STC_CUDA(cudaMemcpyAsync(to, pr.ctr, sizeof(CallCounters), cudaMemcpyDeviceToHost, pin.s));
+  STC_CUDA(cudaStreamSynchronize(pin.s));
+  pin.busy = false;
+  if (pin.p) h = *to;
+  return STC_OK;
+}
+
+stc_status read_counters(const Prepared& pr, Pinned& pin, CallCounters& h) {
+  STC_TRY(copy_counters(pr, pin, h));
+  return status_word(h.c.status);
 }
 
 // Peak device bytes of the GLOBAL strategy for these counts.
@@ -606,7 +697,7 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
   if (from_f) ns = (uint64_t)nX;
   const uint64_t cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)target / alpha) + 1));
   const uint64_t out_cap = std::min(target, cap);
-  uint64_t b = sizeof(Counters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
+  uint64_t b = sizeof(CallCounters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
   b += (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
   b += cap * 16 + out_cap * (4ull * pl.ocols + 8);
@@ -619,22 +710,12 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
 // twice the output bound.
 uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
   const uint64_t out = std::min<uint64_t>(P, pl.F);
-  uint64_t b = sizeof(Counters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
+  uint64_t b = sizeof(CallCounters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
   b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
   b += out * (4ull * pl.ocols + 8);  // the positions chunked reservations leave over only where there is room
   return b;
 }
-
-// Counters of the grouping and binning passes, read back with the first host sync.
-struct GroupCounters {
-  uint32_t count[kMaxClasses + 4];
-  unsigned nholes;       // pieces of the streamed reservations that hold no output
-  u64 huge_slots;
-  u64 out_cap;
-  u64 holes;             // their positions
-  u64 fill_counters[2];
-};
 
 // GROUPED strategy (Sections 4.1 and 4.3): survivors are counting-sorted by X free key,
 // each group is binned by its table size, and the class kernels accumulate one group per
@@ -676,7 +757,8 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   uint32_t *goff = nullptr, *gcur = nullptr, *scr = nullptr;
   GroupedX gx{};
   Bins b{};
-  GroupCounters* gc = nullptr;
+  Pinned pin(ctx, s);
+  GroupCounters* const gc = &reinterpret_cast<CallCounters*>(pr.ctr)->g;
   STC_TRY(ar.alloc(&goff, pl.FX + 1));
   STC_TRY(ar.alloc(&gcur, pl.FX));
   STC_TRY(ar.alloc(&scr, (size_t)scan_scratch_elems((int64_t)pl.FX)));
@@ -684,7 +766,6 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   STC_TRY(ar.alloc(&gx.w, (size_t)nX));
   STC_TRY(ar.alloc(&gx.v, (size_t)nX));
   if (dense_rows) STC_TRY(ar.alloc(&gx.ck, (size_t)nX));
-  STC_TRY(ar.alloc(&gc, 1));
   b.nclasses = ncls;
   for (int c = 0; c < ncls; c++) {
     b.tmax[c] = (u64)(ga * shapes[c].slots);
@@ -705,22 +786,19 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   b.huge_slots = &gc->huge_slots;
   b.out_cap = &gc->out_cap;
   b.status = &pr.ctr->status;
-  STC_CUDA(cudaMemsetAsync(gc, 0, sizeof(GroupCounters), s));
-  STC_CUDA(scan_u32(pr.gcnt, goff, (int64_t)pl.FX, scr, s));
-  STC_CUDA(cudaMemcpyAsync(gcur, goff, pl.FX * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
+  STC_CUDA(scan_u32(pr.gcnt, goff, (int64_t)pl.FX, scr, s, gcur));
   if (pr.dense) {
     STC_CUDA(launch_x_scatter_dense(X->coords, X->vals, nX, pl.kx, pr.yoff, gcur, gx, &pr.ctr->status, ctx->sms, s));
-    STC_CUDA(cudaMemcpyAsync(&pr.ctr->ns, goff + pl.FX, sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
   } else {
     STC_CUDA(launch_x_group_scatter(pr.sv, gcur, gx, nX, ctx->sms, s));
   }
-  STC_CUDA(launch_bin_groups(pl.FX, goff, gx.w, pl.FY, b, ctx->sms, s));
+  STC_CUDA(launch_bin_groups(pl.FX, goff, gx.w, pl.FY, b, pr.dense ? &pr.ctr->ns : nullptr, ctx->sms, s));
   tm.mark(2);
 
-  Counters h{};
-  GroupCounters hg{};
-  STC_CUDA(cudaMemcpyAsync(&hg, gc, sizeof(GroupCounters), cudaMemcpyDeviceToHost, s));
-  STC_TRY(read_counters(pr, s, h));
+  CallCounters hc{};
+  STC_TRY(read_counters(pr, pin, hc));
+  const Counters& h = hc.c;
+  const GroupCounters hg = hc.g;
   tm.mark(3);
   r->stats.products = h.P;
   r->stats.survivors = h.ns;
@@ -751,9 +829,10 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   uint32_t chunk = direct ? warp_chunk(hg.count, out_cap, ctx->sms) : 0u;
   const uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
   if (out_cap + slack >= 0xffffffffull ||
-      (chunk && (ar.alloc(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
-                 ar.alloc(&r->vals, out_cap + slack) != STC_OK))) {
+      (chunk && (ar.alloc_own(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
+                 ar.alloc_own(&r->vals, out_cap + slack) != STC_OK))) {
     chunk = 0;
+    g_last_error.clear();
     if (r->coords) ar.release(r->coords);
     r->coords = nullptr;
     r->vals = nullptr;
@@ -761,8 +840,8 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   if (chunk) {
     out_cap += slack;
   } else {
-    STC_TRY(ar.alloc(&r->coords, out_cap * (size_t)pl.ocols));
-    STC_TRY(ar.alloc(&r->vals, out_cap));
+    STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
+    STC_TRY(ar.alloc_own(&r->vals, out_cap));
   }
   if (hh.count) {
     STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
@@ -770,7 +849,10 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     STC_CUDA(cudaMemsetAsync(hh.keys, 0xff, hg.huge_slots * sizeof(u64), s));
     STC_CUDA(cudaMemsetAsync(hh.vals, 0, hg.huge_slots * sizeof(double), s));
   }
-  BatchOut hbo{};
+  BatchOut bo_here{};
+  static_assert(sizeof(BatchOut) <= kPinnedBytes / 2, "a page-locked block holds the counters and a descriptor");
+  BatchOut& hbo = pin.p ? *reinterpret_cast<BatchOut*>(static_cast<char*>(pin.p) + kPinnedBytes / 2) : bo_here;
+  hbo = BatchOut{};
   hbo.FY = pl.FY;
   hbo.out_cap = out_cap;
   hbo.coords = r->coords;
@@ -778,6 +860,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   hbo.op = pl.op;
   BatchOut* dbo = nullptr;
   STC_TRY(ar.alloc(&dbo, 1));
+  pin.busy = true;
   STC_CUDA(cudaMemcpyAsync(dbo, &hbo, sizeof(BatchOut), cudaMemcpyHostToDevice, s));
   GroupArgs a{};
   a.goff = goff;
@@ -817,19 +900,36 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, ctx->sms, s));
   }
   tm.mark(4);
-  u64 holes = 0;
-  if (nstream || chunk) STC_CUDA(cudaMemcpyAsync(&holes, &gc->holes, sizeof(u64), cudaMemcpyDeviceToHost, s));
-  Counters h2{};
-  STC_TRY(read_counters(pr, s, h2));
-  r->nnz = (int64_t)(h2.nz - holes);
-  if (holes) {
-    u64* dst = nullptr;
-    uint8_t* marked = nullptr;
+  // The holes are filled from the output's end before their number is known here, with scratch for
+  // as many as are to be expected: the chunks' rests, the streaming CTAs' last groups and the
+  // pieces they drop. More (or no memory for so many) take another pass below.
+  u64 most = 0;
+  u64* dst = nullptr;
+  uint8_t* marked = nullptr;
+  auto fill = [&]() -> stc_status {
+    STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, &pr.ctr->nz, &gc->holes, most, marked, dst, gc->fill_counters,
+                              r->coords, r->vals, pl.ocols, &pr.ctr->status, ctx->sms, s));
+    tm.mark(5);
+    return STC_OK;
+  };
+  if (nstream || chunk) {
+    most = std::min<uint64_t>(out_cap, slack + std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64);
+    if (ar.alloc(&dst, (size_t)most) != STC_OK || ar.alloc(&marked, (size_t)most) != STC_OK) {
+      most = 0;
+      g_last_error.clear();
+    }
+    STC_TRY(fill());
+  }
+  CallCounters hc2{};
+  STC_TRY(read_counters(pr, pin, hc2));
+  const u64 holes = hc2.g.holes;
+  r->nnz = (int64_t)(hc2.c.nz - holes);
+  if (holes > most) {
+    most = holes;
     STC_TRY(ar.alloc(&dst, (size_t)holes));
     STC_TRY(ar.alloc(&marked, (size_t)holes));
-    STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, (u64)r->nnz, holes, marked, dst, gc->fill_counters, r->coords,
-                              r->vals, pl.ocols, &pr.ctr->status, ctx->sms, s));
-    tm.mark(5);
+    STC_TRY(fill());
+    STC_TRY(read_counters(pr, pin, hc2));
   }
   r->stats.out_capacity = out_cap;
   r->mem = adopt(ar, ctx, s, {r->coords, r->vals});
@@ -1266,8 +1366,8 @@ stc_status batch_finish_eager(stc_ctx* ctx, BatchDev& bd, const stc_opts& o, Are
   sz.huge = hg.huge_slots;
   double* vals = nullptr;
   int32_t* coords = nullptr;
-  STC_TRY(run.alloc(&vals, voff[n]));
-  STC_TRY(run.alloc(&coords, coff[n]));
+  STC_TRY(run.alloc_own(&vals, voff[n]));
+  STC_TRY(run.alloc_own(&coords, coff[n]));
   std::vector<BatchOut> hbo = bd.hbo;
   for (int32_t i = 0; i < n; i++) {
     hbo[i].out_cap = hper[n + i];
@@ -1540,6 +1640,7 @@ stc_status stc_destroy(stc_ctx* ctx) {
       if (kv.second.ev0[c]) cudaEventDestroy(kv.second.ev0[c]);
       if (kv.second.ev1[c]) cudaEventDestroy(kv.second.ev1[c]);
     }
+  for (void* p : ctx->pins) cudaFreeHost(p);
   cudaMemPoolDestroy(ctx->pool);
   delete ctx;
   return STC_OK;
@@ -1652,6 +1753,7 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
   }
 
   Prepared pr;
+  Pinned pin(ctx, s);
   STC_TRY(prepare(ctx, ar, X, Y, pl, Survey::kSurvivors, s, tm, pr));
   if (pl.F <= kGlobalFromF && o.table_shrink == 0 && X->nnz > 0 && Y->nnz > 0) {
     // A small output key space: the table and the output are sized from F itself, and P and
@@ -1673,8 +1775,8 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
       STC_TRY(ar.alloc(&t.vals, cap));
       STC_TRY(ar.alloc(&wpre, (size_t)nX + 1));
       STC_TRY(ar.alloc(&wscr, (size_t)scan_scratch_elems(nX)));
-      STC_TRY(ar.alloc(&r->coords, out_cap * (size_t)pl.ocols));
-      STC_TRY(ar.alloc(&r->vals, out_cap));
+      STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
+      STC_TRY(ar.alloc_own(&r->vals, out_cap));
       t.mask = cap - 1;
       STC_CUDA(cudaMemsetAsync(t.keys, 0xff, cap * sizeof(u64), s));
       STC_CUDA(cudaMemsetAsync(t.vals, 0, cap * sizeof(double), s));
@@ -1686,8 +1788,9 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
       STC_CUDA(launch_compact_global(t, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status, ctx->sms,
                                      s));
       tm.mark(5);
-      Counters h{};
-      STC_TRY(read_counters(pr, s, h));
+      CallCounters hc{};
+      STC_TRY(read_counters(pr, pin, hc));
+      const Counters& h = hc.c;
       r->nnz = (int64_t)h.nz;
       r->stats.products = h.P;
       r->stats.survivors = h.ns;
@@ -1708,8 +1811,9 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     *out = r;
     return STC_OK;
   }
-  Counters h{};
-  STC_TRY(read_counters(pr, s, h));
+  CallCounters hc{};
+  STC_TRY(read_counters(pr, pin, hc));
+  const Counters& h = hc.c;
   tm.mark(3);
   if (rows_shape && h.P >= kRowsMinPerOutput * pl.F) rows_note(ctx, sig, true);
 
@@ -1738,8 +1842,8 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
       STC_TRY(ar.alloc(&t.vals, cap));
       STC_TRY(ar.alloc(&wpre, (size_t)h.ns + 1));
       STC_TRY(ar.alloc(&wscr, (size_t)scan_scratch_elems((int64_t)h.ns)));
-      STC_TRY(ar.alloc(&r->coords, out_cap * (size_t)pl.ocols));
-      STC_TRY(ar.alloc(&r->vals, out_cap));
+      STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
+      STC_TRY(ar.alloc_own(&r->vals, out_cap));
       STC_CUDA(scan_u32_u64(pr.sv.w, wpre, (int64_t)h.ns, wscr, s));
       tm.mark(3);
       for (uint64_t c = first_cap;; c = cap) {
@@ -1752,9 +1856,9 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
         STC_CUDA(launch_compact_global(t, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status,
                                        ctx->sms, s));
         tm.mark(5);
-        Counters h2{};
-        STC_CUDA(cudaMemcpyAsync(&h2, pr.ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
-        STC_CUDA(cudaStreamSynchronize(s));
+        CallCounters hc2{};
+        STC_TRY(copy_counters(pr, pin, hc2));
+        const Counters& h2 = hc2.c;
         // A table that overflowed lost products: run the expansion again at full capacity
         // (the compaction wrote at most out_cap entries, all of them overwritten now).
         if (h2.status == kStatTableFull && c < cap) {
@@ -1912,7 +2016,7 @@ stc_status stc_batch_plan_run(stc_batch_plan* pl, void* stream, stc_result** out
   const u64 bytes = vbytes + pl->sizes.coords * 4;
   Arena run(ctx, s);
   unsigned char* block = nullptr;
-  STC_TRY(run.alloc(&block, (size_t)std::max<u64>(bytes, 16)));
+  STC_TRY(run.alloc_own(&block, (size_t)std::max<u64>(bytes, 16)));
   pl->h_args->out = block;
   pl->h_args->out_bytes = bytes;
   STC_CUDA(cudaGraphLaunch(pl->exec, s));
@@ -2005,8 +2109,10 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   const int strategy = pick_strategy(pl, X, Y, STC_STRATEGY_AUTO);
   const bool dense = strategy == STC_STRATEGY_GROUPED && (uint64_t)Y->nnz >= pl.K;
   STC_TRY(prepare(ctx, ar, X, Y, pl, dense ? Survey::kDenseGroups : Survey::kSurvivors, s, tm, pr));
-  Counters h{};
-  STC_TRY(read_counters(pr, s, h));
+  Pinned pin(ctx, s);
+  CallCounters hc{};
+  STC_TRY(read_counters(pr, pin, hc));
+  const Counters& h = hc.c;
   if (products) *products = h.P;
   if (bytes_bound)
     *bytes_bound = strategy == STC_STRATEGY_GROUPED ? grouped_bytes(pl, X->nnz, Y->nnz, h.P)

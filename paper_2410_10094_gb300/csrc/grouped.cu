@@ -55,8 +55,9 @@ __global__ void __launch_bounds__(kThreads) x_group_scatter_kernel(Survivors sv,
 // the counters' atomics took 0.27 ms for 4e5 groups, each on one of a few addresses.)
 __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint32_t* __restrict__ goff,
                                                               const uint32_t* __restrict__ gw, u64 FY, Bins b,
-                                                              uint32_t per) {
+                                                              uint32_t per, unsigned* entries) {
   __shared__ u64 s_cap[kThreads / 32];
+  if (entries && blockIdx.x == 0 && threadIdx.x == 0) *entries = goff[FX];
   const unsigned lane = lane_id();
   u64 my_cap = 0;
   for (u64 g0 = ((u64)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * per; g0 < FX;
@@ -2151,13 +2152,14 @@ cudaError_t launch_x_group_scatter(Survivors sv, uint32_t* gcur, GroupedX gx, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, u64 FY, const Bins& b, int sms,
-                              cudaStream_t s) {
+cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, u64 FY, const Bins& b,
+                              unsigned* entries, int sms, cudaStream_t s) {
   if (FX == 0) return cudaSuccess;
   // Up to 32 groups per warp, as long as that leaves every SM its 64 warps.
   const u64 warps = (u64)sms * 64;
   const uint32_t per = (uint32_t)(FX >= 32 * warps ? 32 : (FX + warps - 1) / warps);
-  bin_groups_kernel<<<grid_for((int64_t)((FX + per - 1) / per) * 32, sms), kThreads, 0, s>>>(FX, goff, gw, FY, b, per);
+  bin_groups_kernel<<<grid_for((int64_t)((FX + per - 1) / per) * 32, sms), kThreads, 0, s>>>(FX, goff, gw, FY, b, per,
+                                                                                            entries);
   note_launch();
   return cudaGetLastError();
 }

@@ -15,7 +15,9 @@ unsigned take_launches();
 // Exclusive prefix sums: out[0] = 0, out[i] = in[0] + ... + in[i-1], out[n] = total.
 // `scratch` holds scan_scratch_elems(n) elements of the output type.
 int64_t scan_scratch_elems(int64_t n);
-cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scratch, cudaStream_t s);
+// out2 (may be null) receives out[0..n-1] as well.
+cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scratch, cudaStream_t s,
+                     uint32_t* out2 = nullptr);
 cudaError_t scan_u32_u64(const uint32_t* in, u64* out, int64_t n, u64* scratch, cudaStream_t s);
 cudaError_t scan_u64(const u64* in, u64* out, int64_t n, u64* scratch, cudaStream_t s);
 // scan_u32_u64 over the first min(*dn, nmax) elements, the count read on the device (the grid
@@ -254,8 +256,9 @@ struct HugeGroups {
 
 cudaError_t launch_x_group_scatter(Survivors sv, uint32_t* gcur, GroupedX gx, int64_t max_ns, int sms,
                                    cudaStream_t s);
-cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, u64 FY, const Bins& b, int sms,
-                              cudaStream_t s);
+// entries (may be null) receives the number of grouped X entries.
+cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, u64 FY, const Bins& b,
+                              unsigned* entries, int sms, cudaStream_t s);
 // direct: the shared-memory classes may write outputs as keys are first claimed (needs 32-bit
 // keys and output positions below 2^32 in every problem). counts: host copies of the class
 // counts (b.count), used to size the grids, or null when only the device knows them. depth:
@@ -361,11 +364,13 @@ uint32_t stream_cap();  // most products of a streamed group
 size_t stream_max_holes(uint32_t count, uint32_t nseg, int sms);
 cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                 const uint32_t* list, uint32_t count, const StreamArgs& sa, int sms, cudaStream_t s);
-// Moves the entries at and above nnz into the holes below it. total: positions of all holes;
-// marked [total] and dst [total] are scratch.
-cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, u64 nnz, u64 total, uint8_t* marked,
-                             u64* dst, u64* counters2, int32_t* coords, double* vals, int oz, uint32_t* status,
-                             int sms, cudaStream_t s);
+// Moves the last of the `*reserved` positions' entries into the holes, of which there are
+// *hole_total positions: the outputs are then the first *reserved - *hole_total. Both are read on
+// the device; with more than `most` hole positions nothing is moved. marked [most] and dst [most]
+// are scratch.
+cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, const u64* reserved,
+                             const u64* hole_total, u64 most, uint8_t* marked, u64* dst, u64* counters2,
+                             int32_t* coords, double* vals, int oz, uint32_t* status, int sms, cudaStream_t s);
 
 // Lane-private dense rows for output rows of at most 64 free keys (FY <= 64, 32-bit Y free
 // keys): one warp per group g in [0, ngroups) (empty groups skipped), outputs in key order.

@@ -11,6 +11,7 @@ constexpr int kThreads = 256;
 constexpr int kItems = 16;
 constexpr int kTile = kThreads * kItems;
 constexpr int kWarps = kThreads / 32;
+constexpr int64_t kRawTiles = 1024;
 
 // Exclusive scan of one value per thread across the block; `total` receives the sum.
 template <typename T>
@@ -63,10 +64,14 @@ __global__ void __launch_bounds__(kThreads) tile_sums_kernel(const TI* __restric
   if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
+// tile_offsets: the exclusive scan of the tiles' sums, or, with `raw`, the sums themselves, which
+// each tile then adds up to its own (one launch less for up to kRawTiles tiles). out2, when given,
+// receives the same prefixes without the total (the cursors of a scatter).
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restrict__ in, int64_t n,
-                                                             TO* __restrict__ out,
-                                                             const TO* __restrict__ tile_offsets, const unsigned* dn) {
+                                                             TO* __restrict__ out, TO* __restrict__ out2,
+                                                             const TO* __restrict__ tile_offsets, bool raw,
+                                                             const unsigned* dn) {
   if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
   // Padded so that thread t's run of kItems consecutive elements spreads over banks.
   __shared__ TO tile[kTile + kTile / 32];
@@ -75,6 +80,14 @@ __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restric
   const int64_t base = (int64_t)blockIdx.x * kTile;
   // A tile past the end writes nothing (the tile starting exactly at the end writes the total).
   if (base > n) return;
+  TO off = 0;
+  if (raw) {
+    TO part = 0;
+    for (unsigned i = threadIdx.x; i < blockIdx.x; i += kThreads) part += tile_offsets[i];
+    block_exclusive_scan<TO>(part, off, warp_sums);  // off receives the sum
+  } else if (tile_offsets) {
+    off = tile_offsets[blockIdx.x];
+  }
 #pragma unroll
   for (int k = 0; k < kItems; k++) {
     const int e = k * kThreads + threadIdx.x;
@@ -91,7 +104,6 @@ __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restric
   }
   TO total;
   const TO ex = block_exclusive_scan<TO>(sum, total, warp_sums);
-  const TO off = tile_offsets ? tile_offsets[blockIdx.x] : TO(0);
   TO run = off + ex;
 #pragma unroll
   for (int k = 0; k < kItems; k++) {
@@ -103,7 +115,10 @@ __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restric
   for (int k = 0; k < kItems; k++) {
     const int e = k * kThreads + threadIdx.x;
     const int64_t i = base + e;
-    if (i < n) out[i] = tile[at(e)];
+    if (i < n) {
+      out[i] = tile[at(e)];
+      if (out2) out2[i] = tile[at(e)];
+    }
   }
   // The total goes after the last element, written by the tile that holds position n (the
   // last tile when n is one past its end).
@@ -113,11 +128,11 @@ __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restric
 
 template <typename TI, typename TO>
 cudaError_t exclusive_scan(const TI* in, TO* out, int64_t n, TO* scratch, cudaStream_t s,
-                           const unsigned* dn = nullptr) {
+                           const unsigned* dn = nullptr, TO* out2 = nullptr) {
   if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(TO), s);
   const int64_t nb = (n + kTile - 1) / kTile;
   if (nb == 1) {
-    tile_scan_kernel<TI, TO><<<1, kThreads, 0, s>>>(in, n, out, nullptr, dn);
+    tile_scan_kernel<TI, TO><<<1, kThreads, 0, s>>>(in, n, out, out2, nullptr, false, dn);
     note_launch();
     return cudaGetLastError();
   }
@@ -127,9 +142,12 @@ cudaError_t exclusive_scan(const TI* in, TO* out, int64_t n, TO* scratch, cudaSt
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  e = exclusive_scan<TO, TO>(sums, offs, nb, scratch + 2 * nb + 1, s);
-  if (e != cudaSuccess) return e;
-  tile_scan_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, out, offs, dn);
+  const bool raw = nb <= kRawTiles;
+  if (!raw) {
+    e = exclusive_scan<TO, TO>(sums, offs, nb, scratch + 2 * nb + 1, s);
+    if (e != cudaSuccess) return e;
+  }
+  tile_scan_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, out, out2, raw ? sums : offs, raw, dn);
   note_launch();
   return cudaGetLastError();
 }
@@ -152,8 +170,9 @@ int64_t scan_scratch_elems(int64_t n) {
   return 2 * nb + 1 + scan_scratch_elems(nb);
 }
 
-cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scratch, cudaStream_t s) {
-  return exclusive_scan<uint32_t, uint32_t>(in, out, n, scratch, s);
+cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scratch, cudaStream_t s,
+                     uint32_t* out2) {
+  return exclusive_scan<uint32_t, uint32_t>(in, out, n, scratch, s, nullptr, out2);
 }
 cudaError_t scan_u32_u64(const uint32_t* in, u64* out, int64_t n, u64* scratch, cudaStream_t s) {
   return exclusive_scan<uint32_t, u64>(in, out, n, scratch, s);

@@ -470,12 +470,18 @@ __global__ void __launch_bounds__(T, 4)
   if (threadIdx.x == 0) add_hole(cur, left);
 }
 
-// Holes below nnz become destinations (numbered through *ndst), those above it are marked.
+// Holes below the final count nnz become destinations (numbered through *ndst), those above it are
+// marked.
 __global__ void __launch_bounds__(256) hole_mark_kernel(const StreamHole* __restrict__ holes,
-                                                        const unsigned* __restrict__ nholes, u64 nnz,
+                                                        const unsigned* __restrict__ nholes,
+                                                        const u64* __restrict__ reserved,
+                                                        const u64* __restrict__ hole_total, u64 most,
                                                         uint8_t* __restrict__ marked, u64* __restrict__ dst,
                                                         u64* __restrict__ ndst) {
   const unsigned lane = lane_id(), n = *nholes;
+  const u64 tail = *hole_total;
+  if (tail > most) return;
+  const u64 nnz = *reserved - tail;
   for (unsigned i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
     const StreamHole h = holes[i];
     const u64 end = h.pos + h.len, cut = end < nnz ? end : (h.pos < nnz ? nnz : h.pos);
@@ -489,10 +495,15 @@ __global__ void __launch_bounds__(256) hole_mark_kernel(const StreamHole* __rest
 }
 
 // The entries of [nnz, nnz + tail) that are no holes move to the destinations.
-__global__ void __launch_bounds__(256) hole_fill_kernel(const uint8_t* __restrict__ marked, u64 tail, u64 nnz,
+__global__ void __launch_bounds__(256) hole_fill_kernel(const uint8_t* __restrict__ marked,
+                                                        const u64* __restrict__ reserved,
+                                                        const u64* __restrict__ hole_total, u64 most,
                                                         const u64* __restrict__ dst, u64* __restrict__ nsrc,
                                                         int32_t* __restrict__ coords, double* __restrict__ vals,
                                                         int oz, uint32_t* status) {
+  const u64 tail = *hole_total;
+  if (tail > most) return;
+  const u64 nnz = *reserved - tail;
   for (u64 t0 = ((u64)blockIdx.x * 256 + threadIdx.x) & ~31ull; t0 < tail; t0 += (u64)gridDim.x * 256) {
     const u64 t = t0 + lane_id();
     const bool has = t < tail && !marked[t];
@@ -581,18 +592,18 @@ cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32
                   : launch_rows<false>(a, yoff, nseg, seg, list, count, sa, rows, sms, s);
 }
 
-cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, u64 nnz, u64 total, uint8_t* marked,
-                             u64* dst, u64* counters2, int32_t* coords, double* vals, int oz, uint32_t* status,
-                             int sms, cudaStream_t s) {
-  if (total == 0) return cudaSuccess;
+cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, const u64* reserved,
+                             const u64* hole_total, u64 most, uint8_t* marked, u64* dst, u64* counters2,
+                             int32_t* coords, double* vals, int oz, uint32_t* status, int sms, cudaStream_t s) {
+  if (most == 0) return cudaSuccess;
   cudaError_t e = cudaMemsetAsync(counters2, 0, 2 * sizeof(u64), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(marked, 0, total, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(marked, 0, most, s);
   if (e != cudaSuccess) return e;
-  const unsigned g = (unsigned)sms * 8;
-  hole_mark_kernel<<<(unsigned)sms, 256, 0, s>>>(holes, nholes, nnz, marked, dst, counters2);
-  const u64 want = (total + 255) / 256;
-  hole_fill_kernel<<<(unsigned)(want < g ? want : g), 256, 0, s>>>(marked, total, nnz, dst, counters2 + 1, coords,
-                                                                   vals, oz, status);
+  const u64 g = (u64)sms * 8, want = (most + 255) / 256;
+  hole_mark_kernel<<<(unsigned)(want < (u64)sms ? want : (u64)sms), 256, 0, s>>>(holes, nholes, reserved, hole_total,
+                                                                                most, marked, dst, counters2);
+  hole_fill_kernel<<<(unsigned)(want < g ? want : g), 256, 0, s>>>(marked, reserved, hole_total, most, dst,
+                                                                   counters2 + 1, coords, vals, oz, status);
   note_launch(2);
   return cudaGetLastError();
 }
