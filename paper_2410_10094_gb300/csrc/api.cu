@@ -346,6 +346,9 @@ struct Plan {
   KeyPlan kx{}, ky{};
   OutPlan op{};
   uint64_t K = 1, FX = 1, FY = 1, F = 1;
+  uint64_t Kb = 1;         // bins that Y's contract keys are counted in: K, or with an id map n_Y
+  bool id_map = false;     // contract keys replaced by dense ids through a bitmap (KeyPlan::idmap)
+  bool report_ids = false; // ... in a call that is to report their number
   int32_t oz = 0;
   int32_t ocols = 0;      // int32 words per output entry: oz, or 2 for a 64-bit output key
   bool keys_out = false;  // outputs are keys (row-major over the output shape), not coordinates
@@ -406,7 +409,7 @@ stc_status make_plan(const stc_coo* X, const stc_coo* Y, int32_t m, const int32_
     acc *= (unsigned __int128)X->shape[cx[i]];
     if (acc > (unsigned __int128)UINT64_MAX) return fail(STC_ERR_KEY_OVERFLOW, "contract key space exceeds 2^64");
   }
-  pl.K = (uint64_t)acc;
+  pl.K = pl.Kb = (uint64_t)acc;
 
   // Free keys: row-major over the free modes in ascending order.
   std::vector<int> xf, yf;
@@ -538,6 +541,7 @@ struct GroupCounters {
   u64 out_cap;
   u64 holes;             // their positions
   u64 fill_counters[2];
+  uint32_t ids;          // distinct contract keys of Y (with an id map)
 };
 
 // What a contraction reads back, in one copy.
@@ -591,6 +595,7 @@ struct StageTimer {
 // The device state shared by the counting pass and the contraction: Y grouped by contract
 // key, and X surveyed against it.
 struct Prepared {
+  KeyPlan kx{}, ky{};        // the plan's, with the id map
   uint32_t* yoff = nullptr;  // [K + 1]
   void* yfk = nullptr;       // [nY], Y free keys in contract-key order (u32 when key32, else u64)
   bool key32 = false;
@@ -609,9 +614,9 @@ enum class Survey { kSurvivors, kSurvivorsGroups, kDenseGroups };
 stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, const Plan& pl, Survey mode,
                    cudaStream_t s, StageTimer& tm, Prepared& pr) {
   const bool groups = mode != Survey::kSurvivors;
-  const uint64_t bins = pl.K * pl.ky.nseg;
-  if (pl.K > kMaxDirectBins || bins > kMaxDirectBins)
-    return fail(STC_ERR_UNSUPPORTED, "contract key space %llu exceeds %llu bins", (unsigned long long)pl.K,
+  const uint64_t bins = pl.Kb * pl.ky.nseg;
+  if (pl.Kb > kMaxDirectBins || bins > kMaxDirectBins)
+    return fail(STC_ERR_UNSUPPORTED, "contract key space %llu exceeds %llu bins", (unsigned long long)pl.Kb,
                 (unsigned long long)kMaxDirectBins);
   const int64_t nX = X->nnz, nY = Y->nnz;
   CallCounters* cc = nullptr;
@@ -619,6 +624,16 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
   pr.ctr = &cc->c;
   STC_CUDA(cudaMemsetAsync(cc, 0, sizeof(CallCounters), s));
   uint32_t* status = &pr.ctr->status;
+  pr.kx = pl.kx;
+  pr.ky = pl.ky;
+  if (pl.id_map) {
+    uint2* map = nullptr;
+    uint32_t* scratch = nullptr;
+    STC_TRY(ar.alloc(&map, (size_t)id_map_pairs(pl.K)));
+    STC_TRY(ar.alloc(&scratch, (size_t)id_map_scratch(pl.K)));
+    STC_CUDA(launch_id_map(Y->coords, nY, pl.ky, pl.K, map, scratch, &cc->g.ids, status, ctx->sms, s));
+    pr.kx.idmap = pr.ky.idmap = map;
+  }
 
   // Y: count per contract key, exclusive scan, scatter (Section 4.1.1 counting sort).
   uint32_t *ycnt = nullptr, *ycur = nullptr, *scr = nullptr;
@@ -656,16 +671,16 @@ stc_status prepare(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc_coo* Y, 
     if (ne_words) nonempty = ycnt + bins;
   }
   STC_CUDA(cudaMemsetAsync(ycnt, 0, counts * sizeof(uint32_t), s));
-  STC_CUDA(launch_y_count(Y->coords, nY, pl.ky, ycnt, status, ctx->sms, s, nonempty));
+  STC_CUDA(launch_y_count(Y->coords, nY, pr.ky, ycnt, status, ctx->sms, s, nonempty));
   STC_CUDA(scan_u32(ycnt, pr.yoff, (int64_t)bins, scr, s, ycur));
-  STC_CUDA(launch_y_scatter(Y->coords, Y->vals, nY, pl.ky, pl.FY, ycur, pr.yfk, pr.key32, pr.yv, ctx->sms, s));
+  STC_CUDA(launch_y_scatter(Y->coords, Y->vals, nY, pr.ky, pl.FY, ycur, pr.yfk, pr.key32, pr.yv, ctx->sms, s));
   tm.mark(0);
 
   // X: find each entry's Y run and count the products exactly (Section 4.3).
   if (pr.dense) {
-    STC_CUDA(launch_x_count(X->coords, nX, pl.kx, pr.yoff, &pr.ctr->P, pr.gcnt, status, ctx->sms, s));
+    STC_CUDA(launch_x_count(X->coords, nX, pr.kx, pr.yoff, &pr.ctr->P, pr.gcnt, status, ctx->sms, s));
   } else {
-    STC_CUDA(launch_x_survey(X->coords, X->vals, nX, pl.kx, pr.yoff, pl.K, pr.sv, &pr.ctr->P, pr.gcnt, status,
+    STC_CUDA(launch_x_survey(X->coords, X->vals, nX, pr.kx, pr.yoff, pl.K, pr.sv, &pr.ctr->P, pr.gcnt, status,
                              nonempty, ctx->sms, s, nonempty != nullptr));
   }
   tm.mark(1);
@@ -689,6 +704,20 @@ stc_status read_counters(const Prepared& pr, Pinned& pin, CallCounters& h) {
   return status_word(h.c.status);
 }
 
+// Device bytes of the counting of Y's contract keys.
+uint64_t bins_bytes(const Plan& pl) {
+  uint64_t b = sizeof(CallCounters) + pl.Kb * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.Kb) * 4;
+  return b + (pl.id_map ? id_map_pairs(pl.K) * 8 + (uint64_t)id_map_scratch(pl.K) * 4 : (pl.K + 31) / 32 * 4);
+}
+
+// Whether the one-global-table strategy writes outputs as their keys are claimed: where the output
+// key space is at least twice the products, so that few are expected to repeat a key, and the list
+// of those that do stays below 1 GB. 3.2e6 products over 1.2e15 keys: 0.34 ms against 0.43 for
+// accumulating in the table and passing over its 2^23 slots.
+bool direct_global(uint64_t P, uint64_t F, uint64_t cap) {
+  return P <= F / 2 && P <= (1ull << 26) && cap <= (1ull << 32);
+}
+
 // Peak device bytes of the GLOBAL strategy for these counts.
 uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint64_t P, double alpha) {
   // Small output key spaces are sized from F itself (no host read of P), with a prefix over nX.
@@ -697,10 +726,11 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
   if (from_f) ns = (uint64_t)nX;
   const uint64_t cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)target / alpha) + 1));
   const uint64_t out_cap = std::min(target, cap);
-  uint64_t b = sizeof(CallCounters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
+  uint64_t b = bins_bytes(pl);
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
   b += (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
   b += cap * 16 + out_cap * (4ull * pl.ocols + 8);
+  if (!from_f && direct_global(P, pl.F, cap)) b += P * 12;
   return b;
 }
 
@@ -710,12 +740,16 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
 // twice the output bound.
 uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
   const uint64_t out = std::min<uint64_t>(P, pl.F);
-  uint64_t b = sizeof(CallCounters) + pl.K * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.K) * 4 + (pl.K + 31) / 32 * 4;
+  uint64_t b = bins_bytes(pl);
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
   b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
   b += out * (4ull * pl.ocols + 8);  // the positions chunked reservations leave over only where there is room
   return b;
 }
+
+// Whether GROUPED counts X without a survivor list: Y's runs cover the contract keys on average, or
+// Y's keys were few enough beside its entries that ids are reported (ids cover them all).
+bool x_dense(const Plan& pl, const stc_coo* Y) { return (uint64_t)Y->nnz >= pl.K || pl.report_ids; }
 
 // GROUPED strategy (Sections 4.1 and 4.3): survivors are counting-sorted by X free key,
 // each group is binned by its table size, and the class kernels accumulate one group per
@@ -735,7 +769,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   if (pl.FY <= (1ull << 20) && (o.accumulator == STC_ACC_AUTO || o.accumulator == STC_ACC_DENSE)) {
     seg = (uint32_t)std::min<uint64_t>(kDenseSeg, pow2_at_least(std::max<uint64_t>(pl.FY, 64)));
     nseg = (uint32_t)((pl.FY + seg - 1) / seg);
-    dense_rows = pl.K * nseg <= kMaxDirectBins;
+    dense_rows = pl.Kb * nseg <= kMaxDirectBins;
   }
   if (dense_rows) {
     pl.ky.nseg = pl.kx.nseg = nseg;
@@ -745,7 +779,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   pr.keep_ck = dense_rows;
   // Dense when Y's runs cover the contract keys on average: then nearly every X entry has a
   // run and a survivor list would only be written and read back.
-  const Survey mode = ((uint64_t)Y->nnz >= pl.K) ? Survey::kDenseGroups : Survey::kSurvivorsGroups;
+  const Survey mode = x_dense(pl, Y) ? Survey::kDenseGroups : Survey::kSurvivorsGroups;
   STC_TRY(prepare(ctx, ar, X, Y, pl, mode, s, tm, pr));
 
   const bool wide = pl.FY > 0xffffffffull;
@@ -788,7 +822,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   b.status = &pr.ctr->status;
   STC_CUDA(scan_u32(pr.gcnt, goff, (int64_t)pl.FX, scr, s, gcur));
   if (pr.dense) {
-    STC_CUDA(launch_x_scatter_dense(X->coords, X->vals, nX, pl.kx, pr.yoff, gcur, gx, &pr.ctr->status, ctx->sms, s));
+    STC_CUDA(launch_x_scatter_dense(X->coords, X->vals, nX, pr.kx, pr.yoff, gcur, gx, &pr.ctr->status, ctx->sms, s));
   } else {
     STC_CUDA(launch_x_group_scatter(pr.sv, gcur, gx, nX, ctx->sms, s));
   }
@@ -802,6 +836,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   tm.mark(3);
   r->stats.products = h.P;
   r->stats.survivors = h.ns;
+  if (pl.report_ids) r->stats.contract_ids = hg.ids;
   uint64_t groups = 0, dense_groups = 0;
   for (int c = 0; c < kMaxClasses + 4; c++) groups += hg.count[c];
   dense_groups = hg.count[kMaxClasses + 1] + hg.count[kMaxClasses + 2] + hg.count[kMaxClasses + 3];
@@ -1000,6 +1035,20 @@ bool use_dense_ids(const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode)
   if (pl.K <= 1 || mode == STC_IDS_DIRECT) return false;
   if (mode == STC_IDS_DENSE) return true;
   return pl.K > (1ull << 22) && pl.K > 8ull * (uint64_t)(X->nnz + Y->nnz);
+}
+
+// Whether AUTO numbers the contract keys through a bitmap of the key space instead (KeyPlan::idmap):
+// the keys that would be renumbered, and those that direct counting would count in more than four
+// times as many bins as Y has entries. Two bits per key of bitmap and ranks are cleared and scanned;
+// past 2^30 keys, or 256 per entry, the table of id_insert_rows_kernel is smaller. Lengths 2,000 x
+// 3,000 x 14,000 x 17,000, 3e6 entries, K = 4.2e7: 1.07 -> 0.80 ms for the contraction, by direct
+// counting before; 63,891 x 63,890 x 1,847, 7.4e5 entries, K = 1.2e8: 0.42 -> 0.35, by the table.
+bool use_id_map(const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode, bool dense_ids) {
+  const uint64_t nX = (uint64_t)X->nnz, nY = (uint64_t)Y->nnz;
+  if (mode != STC_IDS_AUTO || nX == 0 || nY == 0 || nY >= kMaxDirectBins - 1) return false;
+  if (pl.K <= (1ull << 22) || pl.K <= 4 * nY || pl.K > (1ull << 30) || pl.K > 256 * (nX + nY)) return false;
+  // Where the strategy depends on how many entries share a key, the table's count decides it.
+  return !dense_ids || pl.FX <= 2 * nX + (1ull << 20) || pl.FX > 16 * nX + (1ull << 20);
 }
 
 // A contraction whose contract key space is too large to count directly, restated over
@@ -1698,7 +1747,12 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     (*out)->stats.swapped = 1;
     return STC_OK;
   }
-  if (!xfree && use_dense_ids(pl, X, Y, o.contract_ids)) {
+  const bool dense_ids = !xfree && use_dense_ids(pl, X, Y, o.contract_ids);
+  if (!xfree && use_id_map(pl, X, Y, o.contract_ids, dense_ids)) {
+    pl.id_map = true;
+    pl.report_ids = dense_ids;
+    pl.Kb = (uint64_t)Y->nnz;
+  } else if (dense_ids) {
     DeviceGuard g(ctx->device);
     if (!g.ok) return fail(STC_ERR_CUDA, "cannot make device %d current", ctx->device);
     Relabelled rl(ctx, static_cast<cudaStream_t>(stream));
@@ -1794,6 +1848,7 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
       r->nnz = (int64_t)h.nz;
       r->stats.products = h.P;
       r->stats.survivors = h.ns;
+      if (pl.report_ids) r->stats.contract_ids = hc.g.ids;
       r->stats.table_slots = cap;
       r->stats.out_capacity = out_cap;
       return STC_OK;
@@ -1825,6 +1880,7 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
   r->shape = pl.zshape;
   r->stats.products = h.P;
   r->stats.survivors = h.ns;
+  if (pl.report_ids) r->stats.contract_ids = hc.g.ids;
   r->stats.strategy = STC_STRATEGY_GLOBAL;
 
   if (h.P > 0) {
@@ -1838,6 +1894,34 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     u64* wscr = nullptr;
     stc_status st = STC_OK;
     auto run = [&]() -> stc_status {
+      if (direct_global(h.P, pl.F, cap) && o.table_shrink == 0 && o.probe == 0) {
+        DirectTable dt{};
+        dt.mask = cap - 1;
+        dt.nreps = reinterpret_cast<u64*>(&reinterpret_cast<CallCounters*>(pr.ctr)->g.fill_counters[0]);
+        if (ar.alloc(&dt.keys, cap) == STC_OK && ar.alloc(&dt.pos, cap) == STC_OK && ar.alloc(&dt.rep_slot, h.P) == STC_OK &&
+            ar.alloc(&dt.rep_val, h.P) == STC_OK) {
+          STC_TRY(ar.alloc(&wpre, (size_t)h.ns + 1));
+          STC_TRY(ar.alloc(&wscr, (size_t)scan_scratch_elems((int64_t)h.ns)));
+          STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
+          STC_TRY(ar.alloc_own(&r->vals, out_cap));
+          STC_CUDA(scan_u32_u64(pr.sv.w, wpre, (int64_t)h.ns, wscr, s));
+          STC_CUDA(cudaMemsetAsync(dt.keys, 0xff, cap * sizeof(u64), s));
+          tm.mark(3);
+          STC_CUDA(launch_expand_direct(wpre, (int64_t)h.ns, h.P, pr.sv, static_cast<const u64*>(pr.yfk), pr.yv, pl.FY,
+                                        dt, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status, ctx->sms,
+                                        s));
+          tm.mark(4);
+          CallCounters hc2{};
+          STC_TRY(read_counters(pr, pin, hc2));
+          r->nnz = (int64_t)hc2.c.nz;
+          return STC_OK;
+        }
+        g_last_error.clear();  // no memory for the list of repeats: the table of values below
+        ar.release(dt.keys);
+        ar.release(dt.pos);
+        ar.release(dt.rep_slot);
+        ar.release(dt.rep_val);
+      }
       STC_TRY(ar.alloc(&t.keys, cap));
       STC_TRY(ar.alloc(&t.vals, cap));
       STC_TRY(ar.alloc(&wpre, (size_t)h.ns + 1));
@@ -2091,7 +2175,12 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   DeviceGuard g(ctx->device);
   if (!g.ok) return fail(STC_ERR_CUDA, "cannot make device %d current", ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (use_dense_ids(pl, X, Y, STC_IDS_AUTO)) {
+  const bool dense_ids = use_dense_ids(pl, X, Y, STC_IDS_AUTO);
+  if (use_id_map(pl, X, Y, STC_IDS_AUTO, dense_ids)) {
+    pl.id_map = true;
+    pl.report_ids = dense_ids;
+    pl.Kb = (uint64_t)Y->nnz;
+  } else if (dense_ids) {
     Relabelled rl(ctx, s);
     STC_TRY(relabel(ctx, X, Y, pl, false, s, rl));
     uint64_t b = 0;
@@ -2107,7 +2196,7 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   StageTimer tm;
   Prepared pr;
   const int strategy = pick_strategy(pl, X, Y, STC_STRATEGY_AUTO);
-  const bool dense = strategy == STC_STRATEGY_GROUPED && (uint64_t)Y->nnz >= pl.K;
+  const bool dense = strategy == STC_STRATEGY_GROUPED && x_dense(pl, Y);
   STC_TRY(prepare(ctx, ar, X, Y, pl, dense ? Survey::kDenseGroups : Survey::kSurvivors, s, tm, pr));
   Pinned pin(ctx, s);
   CallCounters hc{};

@@ -40,7 +40,19 @@ struct KeyPlan {
   int64_t size[kMaxOrder];
   uint64_t cstride[kMaxOrder];
   uint64_t fstride[kMaxOrder];
+  // Contract key spaces far larger than Y: null, or one {bits, rank} pair per 32 contract keys. The
+  // bits mark the keys that Y has; a key's dense id, which takes its place, is the pair's rank (the
+  // marked keys before it) plus the marked keys below it in the pair.
+  const uint2* idmap;
 };
+
+// Replaces contract key ck by its dense id; false if Y has no entry with it. (idmap not null.)
+__device__ __forceinline__ bool dense_key(const KeyPlan& p, uint64_t& ck) {
+  const uint2 w = __ldg(p.idmap + (ck >> 5));
+  const uint32_t bit = 1u << (ck & 31);
+  ck = w.y + __popc(w.x & (bit - 1u));
+  return (w.x & bit) != 0;
+}
 
 // How an output key zkey = fX * F_Y + fY decodes into output coordinates. zkey is a
 // mixed-radix number whose digits, least significant first, are the output coordinates at

@@ -162,6 +162,162 @@ __global__ void __launch_bounds__(kExThreads) expand_global_kernel(
   }
 }
 
+// ---- sparse outputs: about as many output keys as products. A product that claims a new key writes
+// its output entry at once; the table holds keys and output positions, and no values, so there is no
+// pass over it afterwards. A product whose key is there already goes to a list (the slot and the
+// value), and is added to the slot's entry by a kernel of its own, once every position is known.
+// Each thread takes kDirectItems products of a tile together: their searches, gathers and claims
+// overlap. One atomic per tile reserves the positions of its new keys, and one the repeats' places.
+constexpr int kDirectItems = 4;
+constexpr int kDirectTile = kDirectItems * kExThreads;
+__global__ void __launch_bounds__(kExThreads, 4) expand_direct_kernel(
+    const u64* __restrict__ wpre, int64_t ns, u64 P, const u64* __restrict__ sfk, const uint32_t* __restrict__ systart,
+    const double* __restrict__ sv, const u64* __restrict__ yfk, const double* __restrict__ yv, u64 FY, DirectTable t,
+    const __grid_constant__ OutPlan op, int32_t* __restrict__ coords, double* __restrict__ vals, u64 out_cap,
+    u64* __restrict__ nz, uint32_t* status) {
+  constexpr int NW = kExThreads / 32, D = kDirectItems;
+  __shared__ u64 s_pre[kDirectTile + 1];
+  __shared__ int64_t s_lo;
+  __shared__ int s_n;
+  __shared__ uint32_t s_warp[NW];
+  __shared__ u64 s_base, s_rbase;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const uint64_t pol = policy_evict_first();
+  const u64 ntiles = (P + kDirectTile - 1) / kDirectTile;
+  for (u64 tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const u64 p0 = tile * kDirectTile;
+    const u64 p1 = (p0 + kDirectTile < P) ? p0 + kDirectTile : P;
+    if (warp < 2) {
+      // Largest s with wpre[s] <= p0 (warp 0) and <= p1 - 1 (warp 1), 32 ways at a time.
+      const u64 p = warp ? p1 - 1 : p0;
+      int64_t a = 0, b = ns;  // wpre[a] <= p < wpre[b]
+      while (b - a > 1) {
+        const int64_t w = (b - a + 32) / 33;
+        const int64_t at = a + w * (lane + 1);
+        const unsigned le = __ballot_sync(0xffffffffu, at < b && wpre[at] <= p);
+        const int64_t k = __popc(le);
+        const int64_t hi = a + w * (k + 1);
+        a += w * k;
+        if (hi < b) b = hi;
+      }
+      if (lane == 0) {
+        if (warp) s_n = (int)(a & 0x7fffffff); else s_lo = a;
+      }
+    }
+    __syncthreads();
+    const int64_t lo = s_lo;
+    const int n = s_n - (int)lo + 1;
+    for (int k = threadIdx.x; k <= n; k += kExThreads) s_pre[k] = wpre[lo + k];
+    __syncthreads();
+    u64 key[D], j[D];
+    double v[D];
+    uint32_t slot[D];
+    uint32_t state = 0;  // bit u: product u claimed its key; bit 16 + u: its key was there
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      const u64 g = p0 + (u64)u * kExThreads + threadIdx.x;
+      if (g < p1) {
+        int a = 0, b = n - 1;
+        while (a < b) {
+          const int mid = (a + b + 1) >> 1;
+          if (s_pre[mid] <= g) a = mid; else b = mid - 1;
+        }
+        const int64_t s = lo + a;
+        j[u] = (u64)__ldg(systart + s) + (g - s_pre[a]);
+        key[u] = __ldg(sfk + s);
+        v[u] = __ldg(sv + s);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < D; u++)
+      if (p0 + (u64)u * kExThreads + threadIdx.x < p1) {
+        key[u] = key[u] * FY + __ldg(yfk + j[u]);
+        v[u] = __dmul_rn(v[u], __ldg(yv + j[u]));
+      }
+    // The first probes claim without looking first, all of a thread's at once; the few that meet
+    // another key go on one by one.
+    u64 cur[D];
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      slot[u] = 0;
+      cur[u] = 0;
+      if (p0 + (u64)u * kExThreads + threadIdx.x < p1) {
+        slot[u] = (uint32_t)(mix64(key[u]) & t.mask);
+        cur[u] = atomicCAS(t.keys + slot[u], kEmpty64, key[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      if (p0 + (u64)u * kExThreads + threadIdx.x >= p1) continue;
+      u64 probe = 0;
+      while (cur[u] != kEmpty64 && cur[u] != key[u] && probe++ < t.mask) {
+        slot[u] = (uint32_t)((slot[u] + 1) & t.mask);
+        cur[u] = __ldcg(t.keys + slot[u]);
+        if (cur[u] == kEmpty64) cur[u] = atomicCAS(t.keys + slot[u], kEmpty64, key[u]);
+      }
+      if (cur[u] == kEmpty64)
+        state |= 1u << u;
+      else if (cur[u] == key[u])
+        state |= 0x10000u << u;
+      else
+        atomicOr(status, kStatTableFull);
+    }
+    // The tile's new keys: positions in the order of (warp, product of the thread, lane).
+    uint32_t mine = 0, rank[D];
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      const uint32_t m = __ballot_sync(0xffffffffu, (state >> u) & 1u);
+      rank[u] = mine + __popc(m & lanemask_lt());
+      mine += __popc(m);
+    }
+    uint32_t reps = 0, rrank[D];
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      const uint32_t m = __ballot_sync(0xffffffffu, (state >> (16 + u)) & 1u);
+      rrank[u] = reps + __popc(m & lanemask_lt());
+      reps += __popc(m);
+    }
+    if (lane == 0) s_warp[warp] = mine | (reps << 16);  // both at most kDirectTile
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      uint32_t run = 0;
+      for (int w = 0; w < NW; w++) {
+        const uint32_t c = s_warp[w];
+        s_warp[w] = run;
+        run += c;
+      }
+      s_base = run & 0xffffu ? atomicAdd(nz, (u64)(run & 0xffffu)) : 0;
+      s_rbase = run >> 16 ? atomicAdd(t.nreps, (u64)(run >> 16)) : 0;
+    }
+    __syncthreads();
+    const u64 base = s_base + (s_warp[warp] & 0xffffu), rbase = s_rbase + (s_warp[warp] >> 16);
+#pragma unroll
+    for (int u = 0; u < D; u++) {
+      if ((state >> u) & 1u) {
+        const u64 pos = base + rank[u];
+        t.pos[slot[u]] = (uint32_t)pos;
+        if (pos < out_cap)
+          store_output(coords, vals, pos, key[u], v[u], op, pol);
+        else
+          atomicOr(status, kStatOutOverflow);
+      }
+      if ((state >> (16 + u)) & 1u) {
+        t.rep_slot[rbase + rrank[u]] = slot[u];
+        t.rep_val[rbase + rrank[u]] = v[u];
+      }
+    }
+    __syncthreads();  // the tile's shared arrays are rewritten by the next
+  }
+}
+
+__global__ void __launch_bounds__(kExThreads) add_repeats_kernel(DirectTable t, double* __restrict__ vals, u64 out_cap) {
+  const u64 n = *t.nreps;
+  for (u64 i = (u64)blockIdx.x * kExThreads + threadIdx.x; i < n; i += (u64)gridDim.x * kExThreads) {
+    const uint32_t pos = t.pos[t.rep_slot[i]];
+    if (pos < out_cap) atomicAdd(vals + pos, t.rep_val[i]);
+  }
+}
+
 // Each CTA takes 2048 consecutive slots at a time (8 per thread, coalesced), ranks the
 // occupied ones with a block scan and reserves their output positions with one atomic.
 constexpr int kCpItems = 8;
@@ -251,6 +407,19 @@ cudaError_t launch_expand_global_dev(const u64* wpre, const unsigned* dns, const
   expand_for(probe)<<<(unsigned)sms * 8, kExThreads, 0, s>>>(wpre, 0, 0, sv.fk, sv.ystart, sv.v, yfk, yv, FY, t,
                                                              status, dP, dns);
   note_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_expand_direct(const u64* wpre, int64_t ns, u64 P, Survivors sv, const u64* yfk, const double* yv,
+                                 u64 FY, const DirectTable& t, const OutPlan& op, int32_t* coords, double* vals,
+                                 u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s) {
+  if (P == 0 || ns <= 0) return cudaSuccess;
+  const u64 ntiles = (P + kDirectTile - 1) / kDirectTile, cap = (u64)sms * 8;
+  const unsigned g = (unsigned)(ntiles < cap ? ntiles : cap);
+  expand_direct_kernel<<<g, kExThreads, 0, s>>>(wpre, ns, P, sv.fk, sv.ystart, sv.v, yfk, yv, FY, t, op, coords, vals,
+                                                out_cap, nz, status);
+  add_repeats_kernel<<<g, kExThreads, 0, s>>>(t, vals, out_cap);
+  note_launch(2);
   return cudaGetLastError();
 }
 

@@ -49,6 +49,13 @@ uint32_t stream_dead_key(u64 FY);
 cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p, u64 FY,
                              uint32_t* cursor, void* yfk, bool key32, double* yv, int sms, cudaStream_t s);
 
+// The id map of a contract key space of K keys (KeyPlan::idmap, id_map_pairs(K) pairs): Y's contract
+// keys marked and ranked. *ids receives their number. scratch: id_map_scratch(K) elements.
+constexpr u64 id_map_pairs(u64 K) { return (K + 31) / 32; }
+int64_t id_map_scratch(u64 K);
+cudaError_t launch_id_map(const int32_t* coords, int64_t n, const KeyPlan& p, u64 K, uint2* map, uint32_t* scratch,
+                          uint32_t* ids, uint32_t* status, int sms, cudaStream_t s);
+
 // X entries whose contract key has a non-empty Y run ("survivors"), compacted, with the
 // run they will read and the total product count P (Section 4.3).
 struct Survivors {
@@ -135,6 +142,19 @@ cudaError_t launch_expand_global(const u64* wpre, int64_t ns, u64 P, Survivors s
 cudaError_t launch_expand_global_dev(const u64* wpre, const unsigned* dns, const u64* dP, Survivors sv, const u64* yfk,
                                      const double* yv, u64 FY, GlobalTable t, uint32_t* status, int sms,
                                      cudaStream_t s, int probe);
+// The same for outputs with few repeats: outputs written as their keys are claimed, repeats listed
+// and added by a second kernel.
+struct DirectTable {
+  u64* keys;           // [mask + 1], kEmpty64 when free
+  uint32_t* pos;       // [mask + 1] output position of the slot's key
+  u64 mask;            // mask + 1 <= 2^32
+  uint32_t* rep_slot;  // [P]
+  double* rep_val;     // [P]
+  u64* nreps;          // zeroed by the caller
+};
+cudaError_t launch_expand_direct(const u64* wpre, int64_t ns, u64 P, Survivors sv, const u64* yfk, const double* yv,
+                                 u64 FY, const DirectTable& t, const OutPlan& op, int32_t* coords, double* vals,
+                                 u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);
 // Occupied slots -> COO output (coordinates decoded from the key).
 cudaError_t launch_compact_global(GlobalTable t, const OutPlan& op, int32_t* coords, double* vals,
                                   u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);

@@ -91,6 +91,7 @@ __global__ void __launch_bounds__(kThreads) y_count_kernel(const int32_t* __rest
       if (!ok[r]) {
         atomicOr(status, kStatCoordRange);
       } else if (ck[r] != kEmpty64) {
+        if (p.idmap) dense_key(p, ck[r]);
         uint32_t* const bin = cnt + ck[r] * p.nseg + (p.nseg > 1 ? (fk[r] >> p.seg_shift) : 0);
         if (nonempty) {
           if (atomicAdd(bin, 1u) == 0u) atomicOr(nonempty + (ck[r] >> 5), 1u << (ck[r] & 31));
@@ -99,6 +100,82 @@ __global__ void __launch_bounds__(kThreads) y_count_kernel(const int32_t* __rest
         }
       }
     }
+  }
+}
+
+// Marks Y's contract keys in the pairs of an id map.
+template <int ORDER, bool VEC>
+__global__ void __launch_bounds__(kThreads) id_mark_kernel(const int32_t* __restrict__ coords, int64_t n, KeyPlan p,
+                                                           uint2* __restrict__ map, uint32_t* status) {
+  const int64_t step = (int64_t)gridDim.x * kThreads * kRows;
+  for (int64_t base = (int64_t)blockIdx.x * kThreads * kRows + threadIdx.x; base < n; base += step) {
+    uint64_t ck[kRows], fk[kRows];
+    bool ok[kRows];
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+      const int64_t i = base + (int64_t)r * kThreads;
+      ok[r] = false;
+      if (i < n) {
+        ok[r] = row_keys<ORDER, VEC>(coords, i, p, ck[r], fk[r]);
+        if (!ok[r]) atomicOr(status, kStatCoordRange);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < kRows; r++)
+      if (ok[r]) atomicOr(&map[ck[r] >> 5].x, 1u << (ck[r] & 31));
+  }
+}
+
+// Marked keys per tile of kIdTile pairs; then, given the tiles' exclusive prefix, every pair's rank.
+constexpr int kIdItems = 16;
+constexpr int kIdTile = kThreads * kIdItems;
+__global__ void __launch_bounds__(kThreads) id_sums_kernel(const uint2* __restrict__ map, u64 pairs,
+                                                           uint32_t* __restrict__ sums) {
+  __shared__ uint32_t s_warp[kThreads / 32];
+  const u64 base = (u64)blockIdx.x * kIdTile;
+  uint32_t c = 0;
+#pragma unroll
+  for (int k = 0; k < kIdItems; k++) {
+    const u64 i = base + (u64)k * kThreads + threadIdx.x;
+    if (i < pairs) c += __popc(map[i].x);
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if (lane_id() == 0) s_warp[threadIdx.x >> 5] = c;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+    for (int w = 0; w < kThreads / 32; w++) t += s_warp[w];
+    sums[blockIdx.x] = t;
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) id_ranks_kernel(uint2* __restrict__ map, u64 pairs,
+                                                            const uint32_t* __restrict__ offs, uint32_t* ids) {
+  __shared__ uint32_t s_warp[kThreads / 32];
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  uint32_t run = offs[blockIdx.x];
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ids = offs[gridDim.x];
+  // Row by row of kThreads consecutive pairs, so that loads and stores are coalesced.
+  for (int k = 0; k < kIdItems; k++) {
+    const u64 i = (u64)blockIdx.x * kIdTile + (u64)k * kThreads + threadIdx.x;
+    const uint32_t c = i < pairs ? __popc(map[i].x) : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((int)lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; w++) {
+      if (w < (int)warp) before += s_warp[w];
+      total += s_warp[w];
+    }
+    if (i < pairs) map[i].y = run + before + x - c;
+    run += total;
+    __syncthreads();
   }
 }
 
@@ -128,6 +205,7 @@ __global__ void __launch_bounds__(kThreads) y_scatter_kernel(const int32_t* __re
 #pragma unroll
     for (int r = 0; r < kRows; r++) {
       if (!ok[r]) continue;
+      if (p.idmap) dense_key(p, ck[r]);
       const uint32_t pos = atomicAdd(cursor + ck[r] * p.nseg + (p.nseg > 1 ? (fk[r] >> p.seg_shift) : 0), 1u);
       yfk[pos] = (YK)fk[r];
       yv[pos] = v[r];
@@ -218,6 +296,11 @@ __device__ __forceinline__ void rows_runs(const int32_t* __restrict__ coords, in
 #pragma unroll
     for (int r = 0; r < kRows; r++)
       if (ok[r]) ok[r] = (nonempty[ck[r] >> 5] >> (ck[r] & 31)) & 1u;
+  }
+  if (p.idmap) {
+#pragma unroll
+    for (int r = 0; r < kRows; r++)
+      if (ok[r]) ok[r] = dense_key(p, ck[r]);
   }
 #pragma unroll
   for (int r = 0; r < kRows; r++) {
@@ -344,7 +427,11 @@ __global__ void __launch_bounds__(kThreads, 3) x_survey_kernel(const int32_t* __
         else if (ne) live[r] = (ne[ck[r] >> 5] >> (ck[r] & 31)) & 1u;
       }
     }
-    if (!ne) {
+    if (p.idmap) {
+#pragma unroll
+      for (int r = 0; r < kRows; r++)
+        if (live[r]) live[r] = dense_key(p, ck[r]);
+    } else if (!ne) {
 #pragma unroll
       for (int r = 0; r < kRows; r++)
         if (live[r]) live[r] = __ldg(yoff + (ck[r] + 1) * p.nseg) > __ldg(yoff + ck[r] * p.nseg);
@@ -771,6 +858,36 @@ cudaError_t launch_y_count(const int32_t* coords, int64_t n, const KeyPlan& p, u
     note_launch();
     return cudaGetLastError();
   });
+}
+
+int64_t id_map_scratch(u64 K) {
+  const int64_t nb = (int64_t)((id_map_pairs(K) + kIdTile - 1) / kIdTile);
+  return 2 * nb + 1 + scan_scratch_elems(nb);
+}
+
+cudaError_t launch_id_map(const int32_t* coords, int64_t n, const KeyPlan& p, u64 K, uint2* map, uint32_t* scratch,
+                          uint32_t* ids, uint32_t* status, int sms, cudaStream_t s) {
+  const u64 pairs = id_map_pairs(K);
+  const int64_t nb = (int64_t)((pairs + kIdTile - 1) / kIdTile);
+  cudaError_t e = cudaMemsetAsync(map, 0, pairs * sizeof(uint2), s);
+  if (e != cudaSuccess) return e;
+  if (n > 0) {
+    const unsigned g = grid_for((n + kRows - 1) / kRows, sms);
+    e = dispatch_order(p.order, vec_ok(coords, p.order), [&]<int O, bool V>() {
+      id_mark_kernel<O, V><<<g, kThreads, 0, s>>>(coords, n, p, map, status);
+      note_launch();
+      return cudaGetLastError();
+    });
+    if (e != cudaSuccess) return e;
+  }
+  id_sums_kernel<<<(unsigned)nb, kThreads, 0, s>>>(map, pairs, scratch);
+  note_launch();
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  uint32_t* const offs = scratch + nb;
+  if ((e = scan_u32(scratch, offs, nb, offs + nb + 1, s)) != cudaSuccess) return e;
+  id_ranks_kernel<<<(unsigned)nb, kThreads, 0, s>>>(map, pairs, offs, ids);
+  note_launch();
+  return cudaGetLastError();
 }
 
 cudaError_t launch_y_scatter(const int32_t* coords, const double* vals, int64_t n, const KeyPlan& p, u64 FY,
