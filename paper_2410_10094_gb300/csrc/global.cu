@@ -93,47 +93,63 @@ __device__ __forceinline__ void table_add_coop(u64* __restrict__ keys, double* _
   }
 }
 
+// The largest a in [0, n) with pre[a] <= p, given pre[0] <= p, by all lanes of a warp: 33 ways per
+// round of loads.
+__device__ __forceinline__ int64_t warp_upper(const u64* __restrict__ pre, int64_t n, u64 p) {
+  int64_t a = 0, b = n;  // pre[a] <= p < pre[b]
+  while (b - a > 1) {
+    const int64_t w = (b - a + 32) / 33;
+    const int64_t at = a + w * ((int64_t)lane_id() + 1);
+    const int64_t k = __popc(__ballot_sync(0xffffffffu, at < b && pre[at] <= p));
+    a += w * k;
+    if (a + w < b) b = a + w;
+  }
+  return a;
+}
+
+// The owners of 32 consecutive products g0 + lane of a warp: the largest a in [0, n) with
+// pre[a] <= g0 + lane, where pre (shared memory, pre[0] <= g0) increases by at least one per entry.
+// The first owner by a search of all lanes; the others from where the entries after it begin.
+__device__ __forceinline__ int warp_owners(const u64* pre, int n, u64 g0) {
+  const int lane = (int)lane_id();
+  int a = 0, b = n;  // pre[a] <= g0 < pre[b]
+  while (b - a > 1) {
+    const int w = (b - a + 32) / 33;
+    const int at = a + w * (lane + 1);
+    a += w * __popc(__ballot_sync(0xffffffffu, at < b && pre[at] <= g0));
+    if (a + w < b) b = a + w;
+  }
+  const u64 d = a + 1 + lane < n ? pre[a + 1 + lane] - g0 : 32;
+  const uint32_t begins = __reduce_or_sync(0xffffffffu, d < 32 ? 1u << d : 0u);
+  return a + __popc(begins & (0xffffffffu >> (31 - lane)));
+}
+
 // Each CTA takes tiles of kExTile consecutive products. Products are numbered by the
 // survivors' exclusive prefix `wpre`: survivor s owns products [wpre[s], wpre[s+1]), its
 // r-th product pairs it with slot ystart[s] + r of its Y run. Within a tile, thread t
 // handles products t, t+256, ...; consecutive threads read consecutive Y slots.
-// With dP / dns non-null, P and the survivor count are read on the device (the grid then is a
-// persistent one sized by the host without them). G = 1: each lane probes on its own
-// (table_add); G > 1: tiles of G lanes probe buckets together (table_add_coop). The loop over
-// a tile's products is uniform over each warp, so all lanes reach the cooperative probe.
+// G = 1: each lane probes on its own (table_add); G > 1: tiles of G lanes probe buckets together
+// (table_add_coop). The loop over a tile's products is uniform over each warp, so all lanes reach the
+// cooperative probe.
 template <int G>
 __global__ void __launch_bounds__(kExThreads) expand_global_kernel(
     const u64* __restrict__ wpre, int64_t ns, u64 P, const u64* __restrict__ sfk, const uint32_t* __restrict__ systart,
     const double* __restrict__ sv, const u64* __restrict__ yfk, const double* __restrict__ yv, u64 FY,
-    GlobalTable t, uint32_t* status, const u64* dP, const unsigned* dns) {
-  if (dP) P = *dP;
-  if (dns) ns = (int64_t)*dns;
-  if (P == 0 || ns <= 0) return;
+    GlobalTable t, uint32_t* status) {
   __shared__ u64 s_pre[kExTile + 1];
-  __shared__ int64_t s_lo;
-  __shared__ int s_n;
+  __shared__ int64_t s_lo, s_hi;
+  const unsigned warp = threadIdx.x >> 5;
   const u64 ntiles = (P + kExTile - 1) / kExTile;
   for (u64 tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const u64 p0 = tile * kExTile;
     const u64 p1 = (p0 + kExTile < P) ? p0 + kExTile : P;
-    if (threadIdx.x == 0) {
-      // Largest s with wpre[s] <= p0, then largest s with wpre[s] <= p1 - 1.
-      int64_t a = 0, b = ns - 1;
-      while (a < b) {
-        const int64_t mid = (a + b + 1) >> 1;
-        if (wpre[mid] <= p0) a = mid; else b = mid - 1;
-      }
-      int64_t c = a, d = ns - 1;
-      while (c < d) {
-        const int64_t mid = (c + d + 1) >> 1;
-        if (wpre[mid] <= p1 - 1) c = mid; else d = mid - 1;
-      }
-      s_lo = a;
-      s_n = (int)(c - a + 1);
+    if (warp < 2) {
+      const int64_t at = warp_upper(wpre, ns, warp ? p1 - 1 : p0);
+      if (lane_id() == 0) (warp ? s_hi : s_lo) = at;
     }
     __syncthreads();
     const int64_t lo = s_lo;
-    const int n = s_n;
+    const int n = (int)(s_hi - lo) + 1;
     for (int k = threadIdx.x; k <= n; k += kExThreads) s_pre[k] = wpre[lo + k];
     __syncthreads();
     for (u64 g0 = p0 + (threadIdx.x & ~31u); g0 < p1; g0 += kExThreads) {
@@ -162,6 +178,127 @@ __global__ void __launch_bounds__(kExThreads) expand_global_kernel(
   }
 }
 
+// ---- the expansion without a host read and without a prefix over all survivors: the survey has
+// summed the products per block of kSurvivorBlock survivors; one CTA scans those sums, and a tile's
+// CTA scans the run lengths of the one to three blocks that its products lie in.
+constexpr int kBpThreads = 1024;
+__global__ void __launch_bounds__(kBpThreads) block_prefix_kernel(const u64* __restrict__ bsum, u64* __restrict__ bpre,
+                                                                  const unsigned* __restrict__ dns) {
+  __shared__ u64 s_warp[32];
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const unsigned nb = (*dns + kSurvivorBlock - 1) / kSurvivorBlock;
+  u64 run = 0;
+  for (unsigned b0 = 0; b0 < nb; b0 += kBpThreads) {
+    const unsigned i = b0 + threadIdx.x;
+    const u64 v = i < nb ? bsum[i] : 0;
+    u64 x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, x, o);
+      if ((int)lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    u64 t = s_warp[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 y = __shfl_up_sync(0xffffffffu, t, o);
+      if ((int)lane >= o) t += y;
+    }
+    const u64 total = __shfl_sync(0xffffffffu, t, 31);
+    const u64 before = warp ? __shfl_sync(0xffffffffu, t, warp - 1) : 0;
+    if (i < nb) bpre[i] = run + before + x - v;
+    run += total;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) bpre[nb] = run;
+}
+
+constexpr int kBxTile = 1024;  // products per tile
+
+// Adds one product to the output space: the hash table, probed by G lanes together (see
+// expand_global_kernel), or with G = 0 an array of the whole space with a byte per key that has
+// received a product.
+template <int G>
+__global__ void __launch_bounds__(kExThreads) expand_blocks_kernel(const u64* __restrict__ bpre, Survivors sv,
+                                                                   const u64* __restrict__ yfk,
+                                                                   const double* __restrict__ yv, u64 FY,
+                                                                   GlobalTable t, uint8_t* __restrict__ seen,
+                                                                   uint32_t* status) {
+  constexpr int IT = kSurvivorBlock / kExThreads, NW = kExThreads / 32;
+  const int64_t ns = (int64_t)*sv.count;
+  if (ns == 0) return;
+  const int64_t nb = (ns + kSurvivorBlock - 1) / kSurvivorBlock;
+  const u64 P = bpre[nb];
+  __shared__ u64 s_pre[kSurvivorBlock];
+  __shared__ u64 s_warp[NW];
+  __shared__ int64_t s_lo;
+  const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+  const u64 ntiles = (P + kBxTile - 1) / kBxTile;
+  for (u64 tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const u64 p0 = tile * kBxTile;
+    const u64 p1 = (p0 + kBxTile < P) ? p0 + kBxTile : P;
+    if (warp == 0) {
+      const int64_t at = warp_upper(bpre, nb, p0);
+      if (lane == 0) s_lo = at;
+    }
+    __syncthreads();
+    for (int64_t blk = s_lo; blk < nb; blk++) {
+      const u64 q0 = bpre[blk], q1 = bpre[blk + 1];
+      if (q0 >= p1) break;  // uniform
+      // The block's run lengths, IT consecutive ones per thread, scanned.
+      const int64_t s0 = blk * kSurvivorBlock;
+      u64 w[IT], sum = 0;
+#pragma unroll
+      for (int i = 0; i < IT; i++) {
+        const int64_t s = s0 + threadIdx.x * IT + i;
+        w[i] = sum;
+        sum += s < ns ? __ldg(sv.w + s) : 0u;
+      }
+      u64 x = sum;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const u64 y = __shfl_up_sync(0xffffffffu, x, o);
+        if ((int)lane >= o) x += y;
+      }
+      if (lane == 31) s_warp[warp] = x;
+      __syncthreads();
+      u64 before = q0 + x - sum;
+      for (unsigned k = 0; k < warp; k++) before += s_warp[k];
+#pragma unroll
+      for (int i = 0; i < IT; i++) s_pre[threadIdx.x * IT + i] = before + w[i];
+      __syncthreads();
+      const int n = (int)(ns - s0 < (int64_t)kSurvivorBlock ? ns - s0 : (int64_t)kSurvivorBlock);
+      const u64 a0 = q0 > p0 ? q0 : p0, a1 = q1 < p1 ? q1 : p1;
+      for (u64 g0 = a0 + warp * 32; g0 < a1; g0 += kExThreads) {
+        const int a = warp_owners(s_pre, n, g0);
+        const u64 g = g0 + lane;
+        const bool has = g < a1;
+        u64 key = 0;
+        double prod = 0.0;
+        if (has) {
+          const int64_t s = s0 + a;
+          const u64 j = (u64)__ldg(sv.ystart + s) + (g - s_pre[a]);
+          key = __ldg(sv.fk + s) * FY + __ldg(yfk + j);
+          prod = __dmul_rn(__ldg(sv.v + s), __ldg(yv + j));
+        }
+        if (G == 0) {
+          if (has) {
+            atomicAdd(t.vals + key, prod);
+            seen[key] = 1;
+          }
+        } else if (G == 1) {
+          if (has) table_add(t.keys, t.vals, t.mask, key, prod, status);
+        } else {
+          table_add_coop<G < 2 ? 2 : G>(t.keys, t.vals, t.mask, has, key, prod, status);
+        }
+      }
+      __syncthreads();  // the block's prefix is rewritten
+    }
+    __syncthreads();  // and s_lo
+  }
+}
+
 // ---- sparse outputs: about as many output keys as products. A product that claims a new key writes
 // its output entry at once; the table holds keys and output positions, and no values, so there is no
 // pass over it afterwards. A product whose key is there already goes to a list (the slot and the
@@ -177,8 +314,7 @@ __global__ void __launch_bounds__(kExThreads, 4) expand_direct_kernel(
     u64* __restrict__ nz, uint32_t* status) {
   constexpr int NW = kExThreads / 32, D = kDirectItems;
   __shared__ u64 s_pre[kDirectTile + 1];
-  __shared__ int64_t s_lo;
-  __shared__ int s_n;
+  __shared__ int64_t s_lo, s_hi;
   __shared__ uint32_t s_warp[NW];
   __shared__ u64 s_base, s_rbase;
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -188,25 +324,12 @@ __global__ void __launch_bounds__(kExThreads, 4) expand_direct_kernel(
     const u64 p0 = tile * kDirectTile;
     const u64 p1 = (p0 + kDirectTile < P) ? p0 + kDirectTile : P;
     if (warp < 2) {
-      // Largest s with wpre[s] <= p0 (warp 0) and <= p1 - 1 (warp 1), 32 ways at a time.
-      const u64 p = warp ? p1 - 1 : p0;
-      int64_t a = 0, b = ns;  // wpre[a] <= p < wpre[b]
-      while (b - a > 1) {
-        const int64_t w = (b - a + 32) / 33;
-        const int64_t at = a + w * (lane + 1);
-        const unsigned le = __ballot_sync(0xffffffffu, at < b && wpre[at] <= p);
-        const int64_t k = __popc(le);
-        const int64_t hi = a + w * (k + 1);
-        a += w * k;
-        if (hi < b) b = hi;
-      }
-      if (lane == 0) {
-        if (warp) s_n = (int)(a & 0x7fffffff); else s_lo = a;
-      }
+      const int64_t at = warp_upper(wpre, ns, warp ? p1 - 1 : p0);
+      if (lane == 0) (warp ? s_hi : s_lo) = at;
     }
     __syncthreads();
     const int64_t lo = s_lo;
-    const int n = s_n - (int)lo + 1;
+    const int n = (int)(s_hi - lo) + 1;
     for (int k = threadIdx.x; k <= n; k += kExThreads) s_pre[k] = wpre[lo + k];
     __syncthreads();
     u64 key[D], j[D];
@@ -215,17 +338,15 @@ __global__ void __launch_bounds__(kExThreads, 4) expand_direct_kernel(
     uint32_t state = 0;  // bit u: product u claimed its key; bit 16 + u: its key was there
 #pragma unroll
     for (int u = 0; u < D; u++) {
-      const u64 g = p0 + (u64)u * kExThreads + threadIdx.x;
-      if (g < p1) {
-        int a = 0, b = n - 1;
-        while (a < b) {
-          const int mid = (a + b + 1) >> 1;
-          if (s_pre[mid] <= g) a = mid; else b = mid - 1;
+      const u64 g0 = p0 + (u64)u * kExThreads + warp * 32, g = g0 + lane;
+      if (g0 < p1) {
+        const int a = warp_owners(s_pre, n, g0);
+        if (g < p1) {
+          const int64_t s = lo + a;
+          j[u] = (u64)__ldg(systart + s) + (g - s_pre[a]);
+          key[u] = __ldg(sfk + s);
+          v[u] = __ldg(sv + s);
         }
-        const int64_t s = lo + a;
-        j[u] = (u64)__ldg(systart + s) + (g - s_pre[a]);
-        key[u] = __ldg(sfk + s);
-        v[u] = __ldg(sv + s);
       }
     }
 #pragma unroll
@@ -321,7 +442,9 @@ __global__ void __launch_bounds__(kExThreads) add_repeats_kernel(DirectTable t, 
 // Each CTA takes 2048 consecutive slots at a time (8 per thread, coalesced), ranks the
 // occupied ones with a block scan and reserves their output positions with one atomic.
 constexpr int kCpItems = 8;
-__global__ void __launch_bounds__(kCpThreads) compact_global_kernel(GlobalTable t, OutPlan op,
+// With `seen`, the occupied slots are the bytes set in it, and a slot's number is its key.
+__global__ void __launch_bounds__(kCpThreads) compact_global_kernel(GlobalTable t, const uint8_t* __restrict__ seen,
+                                                                    OutPlan op,
                                                                     int32_t* __restrict__ coords,
                                                                     double* __restrict__ vals, u64 out_cap,
                                                                     u64* __restrict__ nz, uint32_t* status) {
@@ -337,7 +460,8 @@ __global__ void __launch_bounds__(kCpThreads) compact_global_kernel(GlobalTable 
 #pragma unroll
     for (int it = 0; it < kCpItems; it++) {
       const int64_t i = base + (int64_t)it * kCpThreads + threadIdx.x;
-      k[it] = i < cap ? __ldcs(t.keys + i) : kEmpty64;
+      k[it] = kEmpty64;
+      if (i < cap) k[it] = !seen ? __ldcs(t.keys + i) : (seen[i] ? (u64)i : kEmpty64);
       cnt += k[it] != kEmpty64;
     }
     uint32_t x = cnt;
@@ -379,7 +503,7 @@ __global__ void __launch_bounds__(kCpThreads) compact_global_kernel(GlobalTable 
 
 namespace {
 using ExpandKernel = void (*)(const u64*, int64_t, u64, const u64*, const uint32_t*, const double*, const u64*,
-                              const double*, u64, GlobalTable, uint32_t*, const u64*, const unsigned*);
+                              const double*, u64, GlobalTable, uint32_t*);
 ExpandKernel expand_for(int probe) {
   switch (probe) {
     case 4: return expand_global_kernel<4>;
@@ -395,18 +519,19 @@ cudaError_t launch_expand_global(const u64* wpre, int64_t ns, u64 P, Survivors s
   const u64 ntiles = (P + kExTile - 1) / kExTile;
   const u64 cap = (u64)sms * 8;
   const unsigned g = (unsigned)(ntiles < cap ? ntiles : cap);
-  expand_for(probe)<<<g, kExThreads, 0, s>>>(wpre, ns, P, sv.fk, sv.ystart, sv.v, yfk, yv, FY, t, status, nullptr,
-                                             nullptr);
+  expand_for(probe)<<<g, kExThreads, 0, s>>>(wpre, ns, P, sv.fk, sv.ystart, sv.v, yfk, yv, FY, t, status);
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_expand_global_dev(const u64* wpre, const unsigned* dns, const u64* dP, Survivors sv, const u64* yfk,
-                                     const double* yv, u64 FY, GlobalTable t, uint32_t* status, int sms,
-                                     cudaStream_t s, int probe) {
-  expand_for(probe)<<<(unsigned)sms * 8, kExThreads, 0, s>>>(wpre, 0, 0, sv.fk, sv.ystart, sv.v, yfk, yv, FY, t,
-                                                             status, dP, dns);
-  note_launch();
+cudaError_t launch_expand_blocks(Survivors sv, u64* bpre, const u64* yfk, const double* yv, u64 FY, GlobalTable t,
+                                 uint8_t* seen, uint32_t* status, int sms, cudaStream_t s, int probe) {
+  block_prefix_kernel<<<1, kBpThreads, 0, s>>>(sv.bsum, bpre, sv.count);
+  auto kern = expand_blocks_kernel<0>;
+  if (!seen)
+    kern = probe == 4 ? expand_blocks_kernel<4> : (probe == 8 ? expand_blocks_kernel<8> : expand_blocks_kernel<1>);
+  kern<<<(unsigned)sms * 8, kExThreads, 0, s>>>(bpre, sv, yfk, yv, FY, t, seen, status);
+  note_launch(2);
   return cudaGetLastError();
 }
 
@@ -423,13 +548,13 @@ cudaError_t launch_expand_direct(const u64* wpre, int64_t ns, u64 P, Survivors s
   return cudaGetLastError();
 }
 
-cudaError_t launch_compact_global(GlobalTable t, const OutPlan& op, int32_t* coords, double* vals, u64 out_cap,
-                                  u64* nz, uint32_t* status, int sms, cudaStream_t s) {
+cudaError_t launch_compact_global(GlobalTable t, const uint8_t* seen, const OutPlan& op, int32_t* coords, double* vals,
+                                  u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s) {
   const u64 cap = t.mask + 1;
   const u64 want = (cap + kCpThreads * kCpItems - 1) / (kCpThreads * kCpItems);
   const u64 lim = (u64)sms * 8;
-  compact_global_kernel<<<(unsigned)(want < lim ? want : lim), kCpThreads, 0, s>>>(t, op, coords, vals, out_cap, nz,
-                                                                                  status);
+  compact_global_kernel<<<(unsigned)(want < lim ? want : lim), kCpThreads, 0, s>>>(t, seen, op, coords, vals, out_cap,
+                                                                                  nz, status);
   note_launch();
   return cudaGetLastError();
 }

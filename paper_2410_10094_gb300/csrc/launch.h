@@ -20,10 +20,6 @@ cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scr
                      uint32_t* out2 = nullptr);
 cudaError_t scan_u32_u64(const uint32_t* in, u64* out, int64_t n, u64* scratch, cudaStream_t s);
 cudaError_t scan_u64(const u64* in, u64* out, int64_t n, u64* scratch, cudaStream_t s);
-// scan_u32_u64 over the first min(*dn, nmax) elements, the count read on the device (the grid
-// and scratch sized for nmax); out[min(*dn, nmax)] = total.
-cudaError_t scan_u32_u64_dev(const uint32_t* in, u64* out, int64_t nmax, const unsigned* dn, u64* scratch,
-                             cudaStream_t s);
 
 // ------------------------------------------------------------------ preparation (prep.cu)
 // Contract key of every entry (the LN key of the contract modes): keys[i] = ckey(i).
@@ -65,7 +61,9 @@ struct Survivors {
   uint32_t* w;      // run length = products this entry makes
   double* v;        // X value
   unsigned* count;  // number of survivors (device counter)
+  u64* bsum;        // null, or products of every block of kSurvivorBlock survivors (zeroed by the caller)
 };
+constexpr unsigned kSurvivorBlock = 1024;
 // With gcnt non-null, also counts survivors per X free key.
 // `nonempty` (K / 32 words of scratch, may be null) is used when K <= kNonemptyMaxKeys: a
 // bitmap of the contract keys that have a Y run, held in shared memory by the survey so that
@@ -137,11 +135,13 @@ struct GlobalTable {
 cudaError_t launch_expand_global(const u64* wpre, int64_t ns, u64 P, Survivors sv, const u64* yfk,
                                  const double* yv, u64 FY, GlobalTable t, uint32_t* status, int sms,
                                  cudaStream_t s, int probe);
-// The same with P and the survivor count read on the device (no host read between the survey
-// and the expansion).
-cudaError_t launch_expand_global_dev(const u64* wpre, const unsigned* dns, const u64* dP, Survivors sv, const u64* yfk,
-                                     const double* yv, u64 FY, GlobalTable t, uint32_t* status, int sms,
-                                     cudaStream_t s, int probe);
+// The same with everything read on the device (no host read between the survey and the expansion):
+// the survivor count, and the products per block of survivors (sv.bsum), whose prefix a first kernel
+// writes to bpre (one element more than sv.bsum). With `seen` the table is an array of the whole
+// output key space (t.vals, zeroed, mask + 1 = F) and seen[F], zeroed, receives 1 for every key that
+// has a product.
+cudaError_t launch_expand_blocks(Survivors sv, u64* bpre, const u64* yfk, const double* yv, u64 FY, GlobalTable t,
+                                 uint8_t* seen, uint32_t* status, int sms, cudaStream_t s, int probe);
 // The same for outputs with few repeats: outputs written as their keys are claimed, repeats listed
 // and added by a second kernel.
 struct DirectTable {
@@ -155,8 +155,8 @@ struct DirectTable {
 cudaError_t launch_expand_direct(const u64* wpre, int64_t ns, u64 P, Survivors sv, const u64* yfk, const double* yv,
                                  u64 FY, const DirectTable& t, const OutPlan& op, int32_t* coords, double* vals,
                                  u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);
-// Occupied slots -> COO output (coordinates decoded from the key).
-cudaError_t launch_compact_global(GlobalTable t, const OutPlan& op, int32_t* coords, double* vals,
+// Occupied slots -> COO output (coordinates decoded from the key); seen: see launch_expand_blocks.
+cudaError_t launch_compact_global(GlobalTable t, const uint8_t* seen, const OutPlan& op, int32_t* coords, double* vals,
                                   u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ per-group tables (grouped.cu)

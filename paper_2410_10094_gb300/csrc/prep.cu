@@ -367,6 +367,20 @@ struct RowBlock {
   }
 };
 
+// Adds a warp's freshly appended survivors (fewer than 64, from position pos on) to the product sums
+// of the one or two blocks of kSurvivorBlock survivors that they lie in.
+__device__ __forceinline__ void add_block_sums(const Survivors& sv, unsigned pos, u64 first, u64 both) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    first += __shfl_xor_sync(0xffffffffu, first, o);
+    both += __shfl_xor_sync(0xffffffffu, both, o);
+  }
+  if (lane_id() == 0) {
+    atomicAdd(sv.bsum + pos / kSurvivorBlock, first);
+    if (both != first) atomicAdd(sv.bsum + pos / kSurvivorBlock + 1, both - first);
+  }
+}
+
 template <int ORDER, bool VEC, bool GROUPS>
 __global__ void __launch_bounds__(kThreads, 3) x_survey_kernel(const int32_t* __restrict__ coords,
                                                             const double* __restrict__ vals, int64_t n, KeyPlan p,
@@ -397,6 +411,7 @@ __global__ void __launch_bounds__(kThreads, 3) x_survey_kernel(const int32_t* __
     unsigned pos = 0;
     if (lane == 0) pos = atomicAdd(sv.count, held);
     pos = __shfl_sync(0xffffffffu, pos, 0);
+    u64 first = 0, both = 0;  // products of the entries in the first block, and of all
     for (uint32_t k = lane; k < held; k += 32) {
       const uint32_t c = b_ck[wq][k];
       const u64 fk = b_fk[wq][k];
@@ -408,9 +423,12 @@ __global__ void __launch_bounds__(kThreads, 3) x_survey_kernel(const int32_t* __
       sv.ystart[pos + k] = lo;
       sv.w[pos + k] = w;
       sv.v[pos + k] = v;
-      my_p += w;
+      both += w;
+      if ((pos + k) / kSurvivorBlock == pos / kSurvivorBlock) first += w;
       if (GROUPS) atomicAdd(gcnt + fk, 1u);
     }
+    my_p += both;
+    if (sv.bsum) add_block_sums(sv, pos, first, both);
     __syncwarp();
     held = 0;
   };
@@ -658,6 +676,7 @@ __global__ void __launch_bounds__(kSvThreads, 1) x_survey_bulk_kernel(const int3
     unsigned pos = 0;
     if (lane == 0) pos = atomicAdd(sv.count, held);
     pos = __shfl_sync(0xffffffffu, pos, 0);
+    u64 first = 0, both = 0;  // products of the entries in the first block, and of all
     for (uint32_t k = lane; k < held; k += 32) {
       const uint32_t c = b_ck[wq][k];
       const u64 fk = b_fk[wq][k];
@@ -669,9 +688,12 @@ __global__ void __launch_bounds__(kSvThreads, 1) x_survey_bulk_kernel(const int3
       sv.ystart[pos + k] = lo;
       sv.w[pos + k] = w;
       sv.v[pos + k] = v;
-      my_p += w;
+      both += w;
+      if ((pos + k) / kSurvivorBlock == pos / kSurvivorBlock) first += w;
       if (GROUPS) atomicAdd(gcnt + fk, 1u);
     }
+    my_p += both;
+    if (sv.bsum) add_block_sums(sv, pos, first, both);
     __syncwarp();
     held = 0;
   };

@@ -41,18 +41,11 @@ __device__ T block_exclusive_scan(T v, T& total, T* warp_sums) {
   return before + x - v;
 }
 
-// With `dn` the scan's length is min(*dn, n), read on the device (n bounds it and sizes the
-// grid); tiles past it sum to zero.
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kThreads) tile_sums_kernel(const TI* __restrict__ in, int64_t n,
-                                                             TO* __restrict__ sums, const unsigned* dn) {
-  if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
+                                                             TO* __restrict__ sums) {
   __shared__ TO warp_sums[kWarps];
   const int64_t base = (int64_t)blockIdx.x * kTile;
-  if (base >= n) {  // a tile past the end (device-side length): its sum is zero
-    if (threadIdx.x == 0) sums[blockIdx.x] = TO(0);
-    return;
-  }
   TO acc = 0;
 #pragma unroll
   for (int k = 0; k < kItems; k++) {
@@ -70,16 +63,12 @@ __global__ void __launch_bounds__(kThreads) tile_sums_kernel(const TI* __restric
 template <typename TI, typename TO>
 __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restrict__ in, int64_t n,
                                                              TO* __restrict__ out, TO* __restrict__ out2,
-                                                             const TO* __restrict__ tile_offsets, bool raw,
-                                                             const unsigned* dn) {
-  if (dn && (int64_t)*dn < n) n = (int64_t)*dn;
+                                                             const TO* __restrict__ tile_offsets, bool raw) {
   // Padded so that thread t's run of kItems consecutive elements spreads over banks.
   __shared__ TO tile[kTile + kTile / 32];
   __shared__ TO warp_sums[kWarps];
   auto at = [](int e) { return e + (e >> 5); };
   const int64_t base = (int64_t)blockIdx.x * kTile;
-  // A tile past the end writes nothing (the tile starting exactly at the end writes the total).
-  if (base > n) return;
   TO off = 0;
   if (raw) {
     TO part = 0;
@@ -127,18 +116,17 @@ __global__ void __launch_bounds__(kThreads) tile_scan_kernel(const TI* __restric
 }
 
 template <typename TI, typename TO>
-cudaError_t exclusive_scan(const TI* in, TO* out, int64_t n, TO* scratch, cudaStream_t s,
-                           const unsigned* dn = nullptr, TO* out2 = nullptr) {
+cudaError_t exclusive_scan(const TI* in, TO* out, int64_t n, TO* scratch, cudaStream_t s, TO* out2 = nullptr) {
   if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(TO), s);
   const int64_t nb = (n + kTile - 1) / kTile;
   if (nb == 1) {
-    tile_scan_kernel<TI, TO><<<1, kThreads, 0, s>>>(in, n, out, out2, nullptr, false, dn);
+    tile_scan_kernel<TI, TO><<<1, kThreads, 0, s>>>(in, n, out, out2, nullptr, false);
     note_launch();
     return cudaGetLastError();
   }
   TO* sums = scratch;
   TO* offs = scratch + nb;
-  tile_sums_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, sums, dn);
+  tile_sums_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, sums);
   note_launch();
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
@@ -147,7 +135,7 @@ cudaError_t exclusive_scan(const TI* in, TO* out, int64_t n, TO* scratch, cudaSt
     e = exclusive_scan<TO, TO>(sums, offs, nb, scratch + 2 * nb + 1, s);
     if (e != cudaSuccess) return e;
   }
-  tile_scan_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, out, out2, raw ? sums : offs, raw, dn);
+  tile_scan_kernel<TI, TO><<<(unsigned)nb, kThreads, 0, s>>>(in, n, out, out2, raw ? sums : offs, raw);
   note_launch();
   return cudaGetLastError();
 }
@@ -172,14 +160,10 @@ int64_t scan_scratch_elems(int64_t n) {
 
 cudaError_t scan_u32(const uint32_t* in, uint32_t* out, int64_t n, uint32_t* scratch, cudaStream_t s,
                      uint32_t* out2) {
-  return exclusive_scan<uint32_t, uint32_t>(in, out, n, scratch, s, nullptr, out2);
+  return exclusive_scan<uint32_t, uint32_t>(in, out, n, scratch, s, out2);
 }
 cudaError_t scan_u32_u64(const uint32_t* in, u64* out, int64_t n, u64* scratch, cudaStream_t s) {
   return exclusive_scan<uint32_t, u64>(in, out, n, scratch, s);
-}
-cudaError_t scan_u32_u64_dev(const uint32_t* in, u64* out, int64_t nmax, const unsigned* dn, u64* scratch,
-                             cudaStream_t s) {
-  return exclusive_scan<uint32_t, u64>(in, out, nmax, scratch, s, dn);
 }
 cudaError_t scan_u64(const u64* in, u64* out, int64_t n, u64* scratch, cudaStream_t s) {
   return exclusive_scan<u64, u64>(in, out, n, scratch, s);

@@ -1,0 +1,53 @@
+"""Small output key spaces (F up to 2^18) accumulated in an array of the whole space, against the
+oracle: survivors around a block of 1,024 and none at all, products around a tile of 1,024, runs
+long and short, spaces that are no multiple of a word, keys that only receive zeros."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def check(X, Y, **kw):
+    import oracle
+    from gpu_util import assert_matches_oracle, gpu_contract, result_host
+
+    res = gpu_contract(W.Problem(X, Y, (1,), (0,)), strategy=1, **kw)
+    ref = oracle.contract(X, Y, (1,), (0,))
+    assert_matches_oracle(*result_host(res), ref)
+    assert res.stats.products == ref.products and res.stats.survivors == np.isin(X.coords[:, 1], Y.coords[:, 0]).sum()
+
+
+@pytest.mark.parametrize("probe", [0, 1])
+@pytest.mark.parametrize("survivors", [0, 1, 31, 1023, 1024, 1025, 5000])
+@pytest.mark.parametrize("run", [1, 3, 700])
+def test_survivors(survivors, run, probe):
+    rng = W.rng_for(8900 + survivors + run)
+    nx = survivors + 4000
+    X = W.uniform_coo(rng, (61, 3000), nx)
+    X.coords[:, 1] = 1000 + X.coords[:, 1] % 2000
+    X.coords[rng.permutation(nx)[:survivors], 1] = rng.integers(0, 40, survivors)
+    Y = W.uniform_coo(rng, (3000, 97), 40 * run)
+    Y.coords[:, 0] = np.repeat(np.arange(40), run)
+    check(X, Y, probe=probe)
+
+
+@pytest.mark.parametrize("f", [(1, 1), (1, 7), (33, 31), (512, 512), (262_144, 1), (3, 87_381)])
+def test_spaces(f):
+    rng = W.rng_for(8950 + f[0])
+    check(W.uniform_coo(rng, (f[0], 90), 9_000), W.uniform_coo(rng, (90, f[1]), 5_000))
+
+
+def test_cancelled_outputs_stay():
+    X = W.COO((4, 2), np.array([[1, 0], [1, 1], [3, 0]], np.int32), np.array([2.0, -2.0, 1.0]))
+    Y = W.COO((2, 5), np.array([[0, 4], [1, 4]], np.int32), np.array([3.0, 3.0]))
+    check(X, Y)
+
+
+def test_one_long_run_among_short_ones():
+    rng = W.rng_for(8960)
+    Y = W.uniform_coo(rng, (500, 64), 20_000)
+    Y.coords[:15_000, 0] = 77
+    X = W.uniform_coo(rng, (900, 500), 30_000)
+    check(X, Y)
