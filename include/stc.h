@@ -81,7 +81,8 @@ enum { STC_STRATEGY_AUTO = 0, STC_STRATEGY_GLOBAL = 1, STC_STRATEGY_GROUPED = 2 
 
 /* Per-group accumulator of the GROUPED strategy. HASH: a probing table sized from the
  * group's bound (Section 4.3); where keys and output positions fit 32 bits, each output is
- * written as soon as its key is first claimed. HASH_SCAN: the same table, accumulated in
+ * written as soon as its key is first claimed (a batch's larger groups over up to 2^18 free keys
+ * mark their keys in a bitmap instead, unless the context has a budget). HASH_SCAN: the same table, accumulated in
  * shared memory and written by a scan of the table after the group. DENSE: the group's output
  * row swept in segments of 2^16 Y free keys; the keys present are found with a bitmap over the
  * segment (no hashing or probing), products are stashed in shared memory and repeated keys

@@ -492,10 +492,14 @@ stc_status make_plan(const stc_coo* X, const stc_coo* Y, int32_t m, const int32_
     const unsigned N = pl.op.z32 ? 32 : 64;
     const unsigned __int128 num = ((unsigned __int128)(((unsigned __int128)1 << l) - d)) << N;
     pl.op.magic[j] = (uint64_t)(num / d + 1);
+    pl.op.magic32[j] = (uint32_t)(((((unsigned __int128)1 << l) - d) << 32) / d + 1);
     pl.op.dpos[j] = (uint8_t)pos_of[t];
     pl.op.dsh1[j] = (uint8_t)(l < 1 ? l : 1);
     pl.op.dsh2[j] = (uint8_t)(l > 1 ? l - 1 : 0);
   }
+  pl.op.ny = (int32_t)yf.size();
+  pl.op.split = pl.op.ident && !pl.op.pow2 && pl.oz >= 2 && pl.oz <= 8 &&
+                pl.FX <= (1ull << 32) && pl.FY <= (1ull << 32);
   pl.ocols = pl.oz;
   pl.keys_out = keys_out;
   if (keys_out) {
@@ -1178,8 +1182,8 @@ struct BatchDev {
 };
 
 // Plans, descriptors and scratch of a batch (no kernel runs; the descriptors are copied on s).
-stc_status batch_setup(stc_ctx* ctx, int32_t n, const stc_problem* problems, Arena& ar, cudaStream_t s,
-                       BatchDev& bd) {
+stc_status batch_setup(stc_ctx* ctx, int32_t n, const stc_problem* problems, const stc_opts& o, Arena& ar,
+                       cudaStream_t s, BatchDev& bd) {
   bd.n = n;
   bd.plans.assign(n, Plan{});
   std::vector<BatchProb> hb(n);
@@ -1303,6 +1307,10 @@ stc_status batch_setup(stc_ctx* ctx, int32_t n, const stc_problem* problems, Are
   b = Bins{};
   b.nclasses = ncls;
   for (int c = 0; c < ncls; c++) STC_TRY(ar.alloc(&b.list[c], maxg));
+  // The two-pass lists, unless the caller asks for scanned tables or a budget could refuse them (the
+  // hash tables take the same groups).
+  if (!bd.wide && o.accumulator != STC_ACC_HASH_SCAN && ctx->budget == 0)
+    for (int d = 0; d < 3; d++) STC_TRY(ar.alloc(&b.dense_list[d], maxg));
   STC_TRY(ar.alloc(&b.huge_list, maxg));
   STC_TRY(ar.alloc(&b.huge_off, maxg));
   STC_TRY(ar.alloc(&b.huge_cap, maxg));
@@ -1448,6 +1456,7 @@ stc_status batch_finish_eager(stc_ctx* ctx, BatchDev& bd, const stc_opts& o, Are
     const bool direct = !bd.wide && sz.maxcap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
     tune_mark(ctx, bd.tune_bucket, tune_cand, false, s);
     STC_CUDA(launch_group_classes(a, bd.wide, direct, bd.b, hg.count, ctx->sms, s, bd.depth));
+    if (bd.b.dense_list[0]) STC_CUDA(launch_group_twopass(a, bd.b, hg.count, ctx->sms, s));
     STC_CUDA(launch_group_huge(a, hh, bd.wide, ctx->sms, s));
     tune_mark(ctx, bd.tune_bucket, tune_cand, true, s);
     if (timed) *timed = true;
@@ -1533,6 +1542,7 @@ stc_status plan_capture(stc_batch_plan* pl) {
     const bool direct =
         !bd.wide && pl->sizes.maxcap < 0x7fffffffull && pl->opts.accumulator != STC_ACC_HASH_SCAN;
     STC_CUDA(launch_group_classes(a, bd.wide, direct, bd.b, nullptr, ctx->sms, ps, bd.depth));
+    if (bd.b.dense_list[0]) STC_CUDA(launch_group_twopass(a, bd.b, nullptr, ctx->sms, ps));
     HugeGroups hh{};
     hh.count = kCountOnDevice;
     hh.countp = bd.gc->count + kMaxClasses;
@@ -2007,7 +2017,7 @@ stc_status stc_contract_batch(stc_ctx* ctx, int32_t n, const stc_problem* proble
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Arena ar(ctx, s);
   BatchDev bd;
-  STC_TRY(batch_setup(ctx, n, problems, ar, s, bd));
+  STC_TRY(batch_setup(ctx, n, problems, o, ar, s, bd));
   // Load factor: given, or picked by the autotuner for this size bucket (entries, problems).
   int tune_cand = -1;
   const TuneChoice ch =
@@ -2080,7 +2090,7 @@ stc_status stc_batch_plan_create(stc_ctx* ctx, int32_t n, const stc_problem* pro
   }
   STC_CUDA(cudaStreamCreateWithFlags(&pl->stream, cudaStreamNonBlocking));
   pl->scratch.reset(new Arena(ctx, pl->stream));
-  stc_status st = batch_setup(ctx, n, pl->probs.data(), *pl->scratch, pl->stream, pl->bd);
+  stc_status st = batch_setup(ctx, n, pl->probs.data(), pl->opts, *pl->scratch, pl->stream, pl->bd);
   cudaError_t e = cudaSuccess;
   if (st == STC_OK) {
     e = cudaMallocHost(&pl->h_args, sizeof(BatchLayoutArgs));

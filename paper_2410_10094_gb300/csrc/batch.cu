@@ -288,8 +288,14 @@ __global__ void __launch_bounds__(kThreads) batch_group_scatter_kernel(Survivors
 }
 
 // One thread per group: its bound (sum of its entries' run lengths; groups here are mostly a
-// single X entry), its problem and X free key, its class. Appends to the class lists are
-// aggregated per warp; each problem's output bound sums min(B_g, F_Y) over its groups.
+// single X entry), its problem and X free key, its list. The lists' counters are few, and every
+// atomic on one takes its turn, so that a CTA reserves once per list for kBinItems groups of each of
+// its threads; each problem's output bound sums min(B_g, F_Y) over its groups. Latency-bound on the
+// chain offsets -> run lengths -> list; 2.2e6 groups of 256 problems: 0.18 ms, against 0.41 with one
+// reservation per warp and list and the problems searched in global memory.
+constexpr int kBinItems = 4;
+constexpr int kBinProblems = 1024;
+constexpr int kBinLists = kMaxClasses + 4;  // classes, overflow groups, two-pass forms
 __global__ void __launch_bounds__(kThreads) bin_batch_kernel(u64 G, const uint32_t* __restrict__ goff,
                                                              const uint32_t* __restrict__ gw,
                                                              const u64* __restrict__ gkey,
@@ -298,62 +304,115 @@ __global__ void __launch_bounds__(kThreads) bin_batch_kernel(u64 G, const uint32
                                                              uint32_t* __restrict__ gprob, u64* __restrict__ gfk,
                                                              u64* __restrict__ pcap) {
   __shared__ u64 s_cap[kThreads / 32];
+  __shared__ uint32_t s_count[kBinLists], s_at[kBinLists];
+  // Batches of up to kBinProblems: the problems' offsets, searched once per group, and the CTA's sums
+  // per problem.
+  __shared__ u64 s_fxoff[kBinProblems + 1], s_pcap[kBinProblems];
   const unsigned lane = lane_id();
+  const bool local = n <= kBinProblems;
+  if (local) {
+    for (int i = threadIdx.x; i <= n; i += kThreads) s_fxoff[i] = fxoff[i];
+    for (int i = threadIdx.x; i < n; i += kThreads) s_pcap[i] = 0;
+    __syncthreads();
+  }
   u64 my_cap = 0;
-  for (u64 base = (u64)blockIdx.x * kThreads + (threadIdx.x & ~31u); base < G; base += (u64)gridDim.x * kThreads) {
-    const u64 g = base + lane;
-    int cls = -1;
-    int p = -1;
-    u64 t = 0;
-    if (g < G && goff[g] != goff[g + 1]) {
-      u64 bnd = 0;
-      for (uint32_t i = goff[g]; i < goff[g + 1]; i++) bnd += gw[i];
-      const u64 key = gkey[g];
-      p = key_problem(fxoff, n, key);
-      gprob[g] = (uint32_t)p;
-      gfk[g] = key - fxoff[p];
-      const u64 FY = pb[p].FY;
-      t = bnd < FY ? bnd : FY;
-      my_cap += t;
-      cls = 0;
-      while (cls < b.nclasses && t > b.tmax[cls]) cls++;
-      if (cls == b.nclasses && t > (1ull << 30)) {
-        atomicOr(b.status, kStatTooLarge);
-        cls = -1;
-      }
-    }
-    for (int c = 0; c <= b.nclasses; c++) {
-      const bool in = cls == c;
-      const uint32_t pos = warp_reserve<uint32_t>(in, b.count + (c < b.nclasses ? c : kMaxClasses));
-      if (in) {
-        if (c < b.nclasses) {
-          b.list[c][pos] = (uint32_t)g;
+  for (u64 base = (u64)blockIdx.x * kThreads * kBinItems; base < G; base += (u64)gridDim.x * kThreads * kBinItems) {
+    if (threadIdx.x < kBinLists) s_count[threadIdx.x] = 0;
+    __syncthreads();
+    int list[kBinItems];
+    uint32_t rank[kBinItems];
+    u64 bound[kBinItems];
+#pragma unroll
+    for (int it = 0; it < kBinItems; it++) {
+      const u64 g = base + (u64)it * kThreads + threadIdx.x;
+      list[it] = -1;
+      int p = -1;
+      u64 t = 0;
+      if (g < G && goff[g] != goff[g + 1]) {
+        const uint32_t x0 = goff[g], x1 = goff[g + 1];
+        u64 bnd = 0;
+        for (uint32_t i = x0; i < x1; i++) bnd += gw[i];
+        const u64 key = gkey[g];
+        if (local) {
+          int lo = 0, hi = n - 1;
+          while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (s_fxoff[mid] <= key) lo = mid; else hi = mid - 1;
+          }
+          p = lo;
         } else {
-          u64 cap = 64;
-          while (cap < 2 * t) cap <<= 1;
-          b.huge_list[pos] = (uint32_t)g;
-          b.huge_off[pos] = atomicAdd(b.huge_slots, cap);
-          b.huge_cap[pos] = cap;
+          p = key_problem(fxoff, n, key);
+        }
+        gprob[g] = (uint32_t)p;
+        gfk[g] = key - fxoff[p];
+        const u64 FY = pb[p].FY;
+        t = bnd < FY ? bnd : FY;
+        my_cap += t;
+        if (local) atomicAdd(s_pcap + p, t);
+        int cls = 0;
+        while (cls < b.nclasses && t > b.tmax[cls]) cls++;
+        list[it] = cls < b.nclasses ? cls : kMaxClasses;
+        if (cls > 1 && b.dense_list[0]) {
+          const int d = twopass_list(bnd, x1 - x0, FY);
+          if (d >= 0) list[it] = kMaxClasses + 1 + d;
+        }
+        if (list[it] == kMaxClasses && t > (1ull << 30)) {
+          atomicOr(b.status, kStatTooLarge);
+          list[it] = -1;
         }
       }
-    }
-    // Output bound per problem, one atomic per (warp, problem).
-    unsigned todo = __ballot_sync(0xffffffffu, p >= 0);
-    while (todo) {
-      const int leader = __ffs(todo) - 1;
-      const int pl = __shfl_sync(0xffffffffu, p, leader);
-      const bool mine = p == pl;
-      u64 sum = mine ? t : 0ull;
+      bound[it] = t;
+      for (int l = 0; l < kBinLists; l++) {
+        const unsigned in = __ballot_sync(0xffffffffu, list[it] == l);
+        if (!in) continue;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(s_count + l, (uint32_t)__popc(in));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (list[it] == l) rank[it] = at + __popc(in & lanemask_lt());
+      }
+      // Output bound per problem, one atomic per (warp, problem).
+      unsigned todo = __ballot_sync(0xffffffffu, !local && p >= 0);
+      while (todo) {
+        const int leader = __ffs(todo) - 1;
+        const int pl = __shfl_sync(0xffffffffu, p, leader);
+        const bool mine = p == pl;
+        u64 sum = mine ? t : 0ull;
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      if ((int)lane == leader) atomicAdd(pcap + pl, sum);
-      todo &= ~__ballot_sync(0xffffffffu, mine);
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if ((int)lane == leader) atomicAdd(pcap + pl, sum);
+        todo &= ~__ballot_sync(0xffffffffu, mine);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < kBinLists) {
+      const uint32_t c = s_count[threadIdx.x];
+      s_at[threadIdx.x] = c ? atomicAdd(b.count + threadIdx.x, c) : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kBinItems; it++) {
+      if (list[it] < 0) continue;
+      const uint32_t g = (uint32_t)(base + (u64)it * kThreads + threadIdx.x), pos = s_at[list[it]] + rank[it];
+      if (list[it] < kMaxClasses) {
+        b.list[list[it]][pos] = g;
+      } else if (list[it] > kMaxClasses) {
+        b.dense_list[list[it] - kMaxClasses - 1][pos] = g;
+      } else {
+        u64 cap = 64;
+        while (cap < 2 * bound[it]) cap <<= 1;
+        b.huge_list[pos] = g;
+        b.huge_off[pos] = atomicAdd(b.huge_slots, cap);
+        b.huge_cap[pos] = cap;
+      }
     }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) my_cap += __shfl_down_sync(0xffffffffu, my_cap, o);
   if (lane == 0) s_cap[threadIdx.x >> 5] = my_cap;
   __syncthreads();
+  if (local)
+    for (int i = threadIdx.x; i < n; i += kThreads)
+      if (s_pcap[i]) atomicAdd(pcap + i, s_pcap[i]);
   if (threadIdx.x == 0) {
     u64 tot = 0;
     for (int w = 0; w < kThreads / 32; w++) tot += s_cap[w];
@@ -500,8 +559,8 @@ cudaError_t launch_batch_group(const BatchArgs& ba, GroupedX gx, const Bins& b, 
   e = cudaMemcpyAsync(ba.gcur, ba.goff, (size_t)G * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
   if (e != cudaSuccess) return e;
   batch_group_scatter_kernel<<<grid_for(ba.total_x, sms), kThreads, 0, s>>>(ba.sv, ba.gid, ba.gcur, gx);
-  bin_batch_kernel<<<grid_for(G, sms), kThreads, 0, s>>>((u64)G, ba.goff, gx.w, ba.idmap.keys, ba.fxoff, ba.n, ba.pb,
-                                                         b, gprob, gfk, ba.pcap);
+  bin_batch_kernel<<<grid_for((G + kBinItems - 1) / kBinItems, sms), kThreads, 0, s>>>(
+      (u64)G, ba.goff, gx.w, ba.idmap.keys, ba.fxoff, ba.n, ba.pb, b, gprob, gfk, ba.pcap);
   note_launch(2);
   return cudaGetLastError();
 }

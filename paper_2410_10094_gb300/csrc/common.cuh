@@ -75,6 +75,12 @@ struct OutPlan {
   uint8_t dsh1[kMaxOutOrder];
   uint8_t dsh2[kMaxOutOrder];
   uint8_t pad2_[kMaxOutOrder];
+  // Plans with `split`: modes in concatenation order, 2 to 8 of them, not all powers of two, X and Y
+  // free keys of at most 32 bits. The last ny digits are Y's, and each part can be decoded in 32
+  // bits, whatever the output key takes (magic32: the multipliers for N = 32).
+  int32_t split;
+  int32_t ny;
+  uint32_t magic32[kMaxOutOrder];
 };
 
 // MurmurHash3's 64-bit finaliser (fmix64, Austin Appleby, public domain): a bijective
@@ -256,6 +262,48 @@ __device__ __forceinline__ void store_row_fixed(int32_t* __restrict__ dst, uint6
       c[O - 1 - j] = (int32_t)(z - q * op.mod[O - 1 - j]);
       z = q;
     }
+  }
+  const int first = (reinterpret_cast<uintptr_t>(dst) & 7u) ? 1 : 0;  // 0 or 1 single store first
+  if (first) st_stream_s32(dst, c[0], pol);
+#pragma unroll
+  for (int k = 0; k < O; k++) {
+    if (k < first || ((k - first) & 1)) continue;
+    if (k + 1 < O) {
+      asm volatile("st.global.L2::cache_hint.v2.s32 [%0], {%1, %2}, %3;" ::"l"(dst + k), "r"(c[k]), "r"(c[k + 1]),
+                   "l"(pol)
+                   : "memory");
+    } else {
+      st_stream_s32(dst + k, c[k], pol);
+    }
+  }
+}
+
+// Digit j of z in a split plan; z becomes the quotient.
+__device__ __forceinline__ int32_t split_digit(uint32_t& z, const OutPlan& op, int j) {
+  const uint32_t t = __umulhi(z, op.magic32[j]);
+  const uint32_t q = (t + ((z - t) >> op.dsh1[j])) >> op.dsh2[j];
+  const int32_t c = (int32_t)(z - q * (uint32_t)op.mod[op.order - 1 - j]);
+  z = q;
+  return c;
+}
+
+// The X part of a split plan's row: its coordinates, from the X free key.
+__device__ __forceinline__ void decode_x_part(uint32_t fx, const OutPlan& op, int32_t* xc) {
+#pragma unroll 1
+  for (int j = op.ny; j < op.order; j++) xc[op.order - 1 - j] = split_digit(fx, op, j);
+}
+
+// A row of O coordinates of a split plan: the X part from xc (decode_x_part), the Y part from fy.
+// Stored in 16 or 8 bytes where the row allows.
+template <int O>
+__device__ __forceinline__ void store_row_split(int32_t* __restrict__ dst, const int32_t* xc, uint32_t fy,
+                                                const OutPlan& op, uint64_t pol) {
+  int32_t c[O];
+#pragma unroll
+  for (int j = 0; j < O; j++) c[O - 1 - j] = j < op.ny ? split_digit(fy, op, j) : xc[O - 1 - j];
+  if (O == 4 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+    st_stream_v4(dst, make_int4(c[0], c[1], c[O > 2 ? 2 : 0], c[O > 3 ? 3 : 0]), pol);
+    return;
   }
   const int first = (reinterpret_cast<uintptr_t>(dst) & 7u) ? 1 : 0;  // 0 or 1 single store first
   if (first) st_stream_s32(dst, c[0], pol);

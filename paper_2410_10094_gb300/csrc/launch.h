@@ -184,11 +184,12 @@ struct Bins {
   int nclasses;
   u64 tmax[kMaxClasses];      // a group goes to the first class with t <= tmax
   uint32_t* list[kMaxClasses];
-  uint32_t* count;            // [kMaxClasses + 4]: classes, overflow groups, stream, rank, stash
+  // [kMaxClasses + 4]: classes, overflow groups, stream, rank, stash (batches: the two-pass forms)
+  uint32_t* count;
   // Dense rows (single contractions with per-segment runs): groups with t >= dense_min go to
   // the stream list (0), the stash list (2) or the rank list (1) by their size and expected
   // repeats (bin_groups_kernel). A streamed group's output bound is B_g itself.
-  uint32_t* dense_list[3];    // null when not used
+  uint32_t* dense_list[3];    // null when not used; batches: the two-pass kernel's forms
   u64 dense_min;
   u64 stream_cap;
   u64 stash_cap;
@@ -250,6 +251,7 @@ struct GroupArgs {
 // Where one group's outputs go, resolved once per group.
 struct OutTarget {
   u64 FY;        // Y free key space of the group's problem
+  u64 fx;        // X free key of the group
   u64 zrow;      // output key of the group's row: fX * F_Y
   u64 base;      // first output position reserved for the group
   u64 cap;       // output capacity of the group's problem
@@ -258,6 +260,7 @@ struct OutTarget {
   u64* counter;  // the problem's output counter (positions are reserved from it)
   uint32_t prob; // problem whose output plan `op` holds (kNoProb before the first group)
   OutPlan op;
+  int32_t xc[8]; // split plans: the group's coordinates, its row's X part
 };
 constexpr uint32_t kNoProb = 0xffffffffu;
 
@@ -367,6 +370,21 @@ cudaError_t launch_batch_group(const BatchArgs& ba, GroupedX gx, const Bins& b, 
 constexpr uint32_t kDenseSeg = 65536;
 constexpr size_t kBitmapSmemPerCta = 112 * 1024;  // two CTAs per SM
 uint32_t dense_stash_cap();
+
+// ------------------------------------------------------------------ batches' larger groups (twopass.cu)
+// The list (form) of the two-pass kernel for a group of `products` products by `entries` X entries over
+// F_Y free keys, or -1 where the group belongs to the hash tables. Measured against those with 3e7
+// products in groups of one size: 1.4 to 1.5 times as fast at 3,750 products (F_Y 6e4), 2.6 to 4.0
+// beyond 8,192 (whose tables lie in global memory); the lead falls as keys repeat, 1.12 to 1.19 at 2 to
+// 4 products per key and 0.96 to 1.14 at 8, where the line is drawn. Groups of the 1,024-slot warp
+// tables lose (the batch of 256 pairs: 15.3 against 13.8 ms with those above 320 products taken in).
+__host__ __device__ constexpr int twopass_list(u64 products, uint32_t entries, u64 FY) {
+  if (FY > (1u << 18) || products > 49152 || entries > 1024 || products > 4 * FY) return -1;
+  if (FY <= (1u << 16) && products <= 8192 && entries <= 256) return 0;
+  return products <= 16384 && entries <= 512 ? 1 : 2;
+}
+// counts: as for launch_group_classes.
+cudaError_t launch_group_twopass(const GroupArgs& a, const Bins& b, const uint32_t* counts, int sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ streamed groups (stream.cu)
 struct StreamArgs {
