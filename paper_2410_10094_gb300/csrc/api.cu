@@ -731,7 +731,8 @@ bool direct_global(uint64_t P, uint64_t F, uint64_t cap) {
 }
 
 // Peak device bytes of the GLOBAL strategy for these counts.
-uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint64_t P, double alpha) {
+uint64_t global_bytes(const stc_ctx* ctx, const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint64_t P,
+                      double alpha) {
   // Small output key spaces are sized from F itself (no host read of P), with a prefix over nX.
   const bool from_f = pl.F <= kGlobalFromF;
   const uint64_t target = from_f ? pl.F : std::min<uint64_t>(P, pl.F);
@@ -741,7 +742,7 @@ uint64_t global_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint6
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
   b += from_f ? (2 * survivor_blocks(nX) + 1) * 8 : (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
   b += cap * 16 + out_cap * (4ull * pl.ocols + 8);
-  if (!from_f && direct_global(P, pl.F, cap)) b += P * 12;
+  if (!from_f && direct_global(P, pl.F, cap) && ctx->budget == 0) b += P * 12;
   return b;
 }
 
@@ -1054,10 +1055,12 @@ bool use_dense_ids(const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode)
 // past 2^30 keys, or 256 per entry, the table of id_insert_rows_kernel is smaller. Lengths 2,000 x
 // 3,000 x 14,000 x 17,000, 3e6 entries, K = 4.2e7: 1.07 -> 0.80 ms for the contraction, by direct
 // counting before; 63,891 x 63,890 x 1,847, 7.4e5 entries, K = 1.2e8: 0.42 -> 0.35, by the table.
-bool use_id_map(const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode, bool dense_ids) {
+bool use_id_map(const stc_ctx* ctx, const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode, bool dense_ids) {
   const uint64_t nX = (uint64_t)X->nnz, nY = (uint64_t)Y->nnz;
   if (mode != STC_IDS_AUTO || nX == 0 || nY == 0 || nY >= kMaxDirectBins - 1) return false;
   if (pl.K <= (1ull << 22) || pl.K <= 4 * nY || pl.K > (1ull << 30) || pl.K > 256 * (nX + nY)) return false;
+  // The map may take more memory than the table of the keys met: a budget that held the table holds.
+  if (dense_ids && ctx->budget) return false;
   // Where the strategy depends on how many entries share a key, the table's count decides it.
   return !dense_ids || pl.FX <= 2 * nX + (1ull << 20) || pl.FX > 16 * nX + (1ull << 20);
 }
@@ -1765,7 +1768,7 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     return STC_OK;
   }
   const bool dense_ids = !xfree && use_dense_ids(pl, X, Y, o.contract_ids);
-  if (!xfree && use_id_map(pl, X, Y, o.contract_ids, dense_ids)) {
+  if (!xfree && use_id_map(ctx, pl, X, Y, o.contract_ids, dense_ids)) {
     pl.id_map = true;
     pl.report_ids = dense_ids;
     pl.Kb = (uint64_t)Y->nnz;
@@ -1920,7 +1923,8 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     u64* wscr = nullptr;
     stc_status st = STC_OK;
     auto run = [&]() -> stc_status {
-      if (direct_global(h.P, pl.F, cap) && o.table_shrink == 0 && o.probe == 0) {
+      // (The list of repeats may take more than the table of values saves: not under a budget.)
+      if (direct_global(h.P, pl.F, cap) && o.table_shrink == 0 && o.probe == 0 && ctx->budget == 0) {
         DirectTable dt{};
         dt.mask = cap - 1;
         dt.nreps = reinterpret_cast<u64*>(&reinterpret_cast<CallCounters*>(pr.ctr)->g.fill_counters[0]);
@@ -2202,7 +2206,7 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   if (!g.ok) return fail(STC_ERR_CUDA, "cannot make device %d current", ctx->device);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const bool dense_ids = use_dense_ids(pl, X, Y, STC_IDS_AUTO);
-  if (use_id_map(pl, X, Y, STC_IDS_AUTO, dense_ids)) {
+  if (use_id_map(ctx, pl, X, Y, STC_IDS_AUTO, dense_ids)) {
     pl.id_map = true;
     pl.report_ids = dense_ids;
     pl.Kb = (uint64_t)Y->nnz;
@@ -2231,7 +2235,7 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   if (products) *products = h.P;
   if (bytes_bound)
     *bytes_bound = strategy == STC_STRATEGY_GROUPED ? grouped_bytes(pl, X->nnz, Y->nnz, h.P)
-                                                    : global_bytes(pl, X->nnz, Y->nnz, h.ns, h.P, 0.5);
+                                                    : global_bytes(ctx, pl, X->nnz, Y->nnz, h.ns, h.P, 0.5);
   return STC_OK;
 }
 

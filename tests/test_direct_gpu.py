@@ -73,3 +73,24 @@ def test_output_keys_beyond_32_bits():
     order = np.argsort(got)
     np.testing.assert_array_equal(got[order], want)
     assert np.all(np.abs(a.vals.cpu().numpy()[order] - ref.vals) <= 1e-12 * ref.abs)
+
+
+def test_within_the_counted_bytes():
+    """A context whose budget is the bound of stc_count keeps the table of values."""
+    import gc
+
+    import oracle
+    import paper_2410_10094_gb300 as stc
+    from gpu_util import assert_matches_oracle, result_host, to_dev
+
+    rng = W.rng_for(8850)
+    X, Y = W.uniform_coo(rng, (2_000_000, 40), 30_000), W.uniform_coo(rng, (40, 90_000), 4_000)
+    wide = stc.Context(mem_budget_bytes=8 << 30)
+    _, need = stc.count(to_dev(X), to_dev(Y), (1,), (0,), ctx=wide)
+    tight = stc.Context(mem_budget_bytes=need)
+    res = stc.contract(to_dev(X), to_dev(Y), (1,), (0,), ctx=tight)
+    assert_matches_oracle(*result_host(res), oracle.contract(X, Y, (1,), (0,), None))
+    del res
+    gc.collect()
+    wide.close()
+    tight.close()

@@ -93,3 +93,26 @@ def test_out_of_range(which, value):
     with pytest.raises(stc.StcError) as e:
         stc.contract(to_dev(X), to_dev(Y), (1,), (0,))
     assert e.value.status == 8
+
+
+def test_budget_keeps_the_table():
+    """Under a budget the keys that were renumbered through the table still are."""
+    import gc
+
+    import oracle
+    import paper_2410_10094_gb300 as stc
+    from gpu_util import assert_matches_oracle, result_host, to_dev
+
+    rng = W.rng_for(8960)
+    X, Y = W.uniform_coo(rng, (1 << 23, 50), 60_000), W.uniform_coo(rng, (1 << 23, 30), 50_000)
+    X.coords[:, 0] = Y.coords[rng.integers(0, 50_000, 60_000), 0]
+    wide = stc.Context(mem_budget_bytes=8 << 30)
+    _, need = stc.count(to_dev(X), to_dev(Y), (0,), (0,), ctx=wide)
+    tight = stc.Context(mem_budget_bytes=need)
+    res = stc.contract(to_dev(X), to_dev(Y), (0,), (0,), ctx=tight)
+    assert res.stats.contract_ids == len(np.unique(Y.coords[:, 0]))
+    assert_matches_oracle(*result_host(res), oracle.contract(X, Y, (0,), (0,), None))
+    del res
+    gc.collect()
+    wide.close()
+    tight.close()
