@@ -57,7 +57,7 @@ struct StreamSmem {
   uint16_t rk[kList];
   u64 base;                  // positions reserved for the group
   uint32_t warp_tot[NW + 1];
-  uint32_t firsts, repeats;
+  uint32_t firsts, repeats;  // places given out from the front and from the back
 };
 static_assert(4 * (sizeof(StreamSmem) + 1024 + 64) <= 228 * 1024, "four CTAs per SM");
 static_assert(sizeof(uint2) * kQuarters >= kCap, "the map of ranks fits the quarter-slot table");
@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(T, 4)
   };
   for (uint32_t i = threadIdx.x; i < kWords; i += T) sm.bits[i] = sm.rbits[i] = 0;
   for (uint32_t i = threadIdx.x; i < kHash; i += T) sm.hash[i] = kHashEmpty;
-  if (threadIdx.x == 0) sm.firsts = sm.repeats = 0;
   __syncthreads();
   if (!SEG && threadIdx.x == 0) sm.bits[dead >> 5] |= 1u << (dead & 31);
   // Prefetched staging of the next group, when it is staged in one piece.
@@ -186,6 +185,10 @@ __global__ void __launch_bounds__(T, 4)
       }
     }
     for (uint32_t q = 0; q < (SEG ? nseg : 1u); q++) {
+      // The counts of the last segment or group were read before the barrier that ends it; the
+      // staging's barriers publish the cleared ones. (Every thread derives the leftover positions
+      // from its own reading, so the clearing must not overtake a warp that has yet to read.)
+      if (threadIdx.x == 0) sm.firsts = sm.repeats = 0;
       // The products, and their positions (a pass of its own for groups of several pieces).
       uint32_t products = 0, r = 0;
       auto reserve = [&](uint32_t n) {  // thread 0
@@ -463,8 +466,7 @@ __global__ void __launch_bounds__(T, 4)
       // ---- clear the bitmaps for the next segment or group.
       for (uint32_t i = threadIdx.x; i < nwords; i += T)
         sm.bits[i] = (!SEG && i == dead >> 5) ? 1u << (dead & 31) : 0u;
-      if (threadIdx.x == 0) sm.firsts = sm.repeats = 0;
-      __syncthreads();
+      __syncthreads();  // also ends the reading of this segment's counts
     }
   }
   if (threadIdx.x == 0) add_hole(cur, left);

@@ -72,6 +72,25 @@ def test_list_of_repeats(reps):
     assert res.nnz == 900 * (6000 - reps)
 
 
+@pytest.mark.parametrize("length", [800, 1_301])
+@pytest.mark.parametrize("repeats", [False, True])
+def test_groups_handing_on_positions(length, repeats):
+    """Many groups per CTA whose leftover positions the next group fills: groups without a repeat
+    between groups that leave hundreds, so that every thread of a CTA has to carry the same leftovers
+    on (a group without repeats has no barrier between its counts and the end of the group)."""
+    rng = W.rng_for(8250 + length + repeats)
+    fy = 30_000
+    Y = runs(rng, 12, length, fy, distinct=True)
+    groups = 5_000
+    c = np.stack([np.arange(groups), rng.integers(0, 12, groups)], 1)
+    if repeats:  # every third group meets its run twice: as many repeats as outputs
+        c = np.concatenate([c, c[::3]])
+    X = W.COO((groups, 12), c.astype(np.int32), W.nonzero_values(rng, len(c)))
+    for _ in range(2):
+        res = check(W.Problem(X, Y, (1,), (0,)), accumulator=2)
+        assert res.nnz == groups * length
+
+
 @pytest.mark.parametrize("xs,ys,out", [((30, 5), (40, 25), None), ((32, 4), (64, 16), None), ((32, 4), (64, 16), (3, 1, 0, 2)),
                                        ((7, 5), (9, 120), (1, 0, 3, 2)), ((100,), (50, 20), None), ((100,), (1000,), None),
                                        ((10, 10), (10, 10, 10), None), ((5, 4, 3), (12, 9, 10), None),
