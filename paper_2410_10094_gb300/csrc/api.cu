@@ -873,7 +873,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
   bool direct = !wide && !lane_rows && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
   // Room for the positions that chunked reservations may leave over, where the budget has it.
-  uint32_t chunk = direct ? warp_chunk(hg.count, out_cap, ctx->sms) : 0u;
+  uint32_t chunk = direct ? warp_chunk(hg.count, pl.FY, out_cap, ctx->sms) : 0u;
   const uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
   if (out_cap + slack >= 0xffffffffull ||
       (chunk && (ar.alloc_own(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||

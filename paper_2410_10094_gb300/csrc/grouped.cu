@@ -2124,6 +2124,11 @@ cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, 
   return cudaGetLastError();
 }
 
+// Whether the warp classes of a single contraction take several groups per warp (group_pack_kernel).
+static bool packs(uint32_t small, uint32_t medium, u64 FY) {
+  return (u64)small + medium >= kPackMinGroups && FY < (1u << kPackBits);
+}
+
 uint32_t warp_chunk_warps(const uint32_t* counts, int sms) {
   const uint32_t most = (uint32_t)sms * 64;
   return std::min(counts[0], most) + std::min(counts[1], most);
@@ -2132,8 +2137,8 @@ uint32_t warp_chunk_warps(const uint32_t* counts, int sms) {
 // One reservation per group and round would be one atomic on the same address each, at about 0.7 ns:
 // 0.27 ms for 4e5 groups. Chunks of up to 512 positions per warp cost at most half of the output's
 // bound in positions left over, which are filled from the output's end.
-uint32_t warp_chunk(const uint32_t* counts, u64 out_cap, int sms) {
-  if ((u64)counts[0] + counts[1] < kPackMinGroups) return 0;
+uint32_t warp_chunk(const uint32_t* counts, u64 FY, u64 out_cap, int sms) {
+  if (!packs(counts[0], counts[1], FY)) return 0;
   const u64 c = out_cap / (2 * (u64)warp_chunk_warps(counts, sms));
   return c < 32 ? 0 : (uint32_t)(c < 512 ? c : 512);
 }
@@ -2146,8 +2151,7 @@ cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct
   uint32_t h[kMaxClasses];
   for (int c = 0; c < kMaxClasses; c++) h[c] = counts ? counts[c] : kCountOnDevice;
   const uint32_t* d = b.count;
-  if (!wide_keys && direct && !a.gprob && a.FY < (1u << kPackBits) && counts &&
-      (u64)h[0] + h[1] >= kPackMinGroups) {
+  if (!wide_keys && direct && !a.gprob && counts && packs(h[0], h[1], a.FY)) {
     // Small groups of a single contraction, many of them. Four share a table of 1,024 slots where
     // each takes at most 256 (and the load factor leaves room, as it does for one group in 256).
     if ((e = launch_pack<4>(a, b.list[0], d + 0, h[0], sms, s))) return e;

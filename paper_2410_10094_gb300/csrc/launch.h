@@ -291,9 +291,9 @@ cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct
                                  const uint32_t* counts, int sms, cudaStream_t s, int depth = 0);
 cudaError_t launch_group_huge(const GroupArgs& a, const HugeGroups& h, bool wide_keys, int sms, cudaStream_t s);
 // Most warps that the warp classes' direct kernels run for these counts, and the chunk of
-// positions each should reserve at a time (GroupArgs::chunk).
+// positions each should reserve at a time (GroupArgs::chunk; 0 where they do not share counters).
 uint32_t warp_chunk_warps(const uint32_t* counts, int sms);
-uint32_t warp_chunk(const uint32_t* counts, u64 out_cap, int sms);
+uint32_t warp_chunk(const uint32_t* counts, u64 FY, u64 out_cap, int sms);
 
 // ------------------------------------------------------------------ batches (batch.cu)
 // One problem of a batch as the device kernels see it.
