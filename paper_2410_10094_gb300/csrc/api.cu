@@ -872,13 +872,28 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   hh.cap = b.huge_cap;
   const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
   bool direct = !wide && !lane_rows && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
-  // Room for the positions that chunked reservations may leave over, where the budget has it.
-  uint32_t chunk = direct ? warp_chunk(hg.count, pl.FY, out_cap, ctx->sms) : 0u;
-  const uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
-  if (out_cap + slack >= 0xffffffffull ||
-      (chunk && (ar.alloc_own(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
-                 ar.alloc_own(&r->vals, out_cap + slack) != STC_OK))) {
+  // Chunked reservations leave positions over, at most `slack`, which the output then has room for.
+  // That is memory which a call without them does not need: none under a budget, and none that the
+  // call's other requests, made first, leave no room for.
+  uint32_t chunk = direct && ctx->budget == 0 ? warp_chunk(hg.count, pl.FY, out_cap, ctx->sms) : 0u;
+  uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
+  if (out_cap + slack >= 0xffffffffull) chunk = 0, slack = 0;
+  BatchOut* dbo = nullptr;
+  STC_TRY(ar.alloc(&dbo, 1));
+  StreamArgs sa{};
+  if (nstream || chunk)
+    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms) +
+                                    (chunk ? warp_chunk_warps(hg.count, ctx->sms) : 0u)));
+  if (hh.count) {
+    STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
+    STC_TRY(ar.alloc(&hh.vals, hg.huge_slots));
+    STC_CUDA(cudaMemsetAsync(hh.keys, 0xff, hg.huge_slots * sizeof(u64), s));
+    STC_CUDA(cudaMemsetAsync(hh.vals, 0, hg.huge_slots * sizeof(double), s));
+  }
+  if (chunk && (ar.alloc_own(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
+                ar.alloc_own(&r->vals, out_cap + slack) != STC_OK)) {
     chunk = 0;
+    slack = 0;
     g_last_error.clear();
     if (r->coords) ar.release(r->coords);
     r->coords = nullptr;
@@ -890,12 +905,6 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
     STC_TRY(ar.alloc_own(&r->vals, out_cap));
   }
-  if (hh.count) {
-    STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
-    STC_TRY(ar.alloc(&hh.vals, hg.huge_slots));
-    STC_CUDA(cudaMemsetAsync(hh.keys, 0xff, hg.huge_slots * sizeof(u64), s));
-    STC_CUDA(cudaMemsetAsync(hh.vals, 0, hg.huge_slots * sizeof(double), s));
-  }
   BatchOut bo_here{};
   static_assert(sizeof(BatchOut) <= kPinnedBytes / 2, "a page-locked block holds the counters and a descriptor");
   BatchOut& hbo = pin.p ? *reinterpret_cast<BatchOut*>(static_cast<char*>(pin.p) + kPinnedBytes / 2) : bo_here;
@@ -905,8 +914,6 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   hbo.coords = r->coords;
   hbo.vals = r->vals;
   hbo.op = pl.op;
-  BatchOut* dbo = nullptr;
-  STC_TRY(ar.alloc(&dbo, 1));
   pin.busy = true;
   STC_CUDA(cudaMemcpyAsync(dbo, &hbo, sizeof(BatchOut), cudaMemcpyHostToDevice, s));
   GroupArgs a{};
@@ -923,10 +930,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   a.status = &pr.ctr->status;
   a.bout = dbo;
   a.bnz = &pr.ctr->nz;
-  StreamArgs sa{};
   if (nstream || chunk) {
-    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms) +
-                                    (chunk ? warp_chunk_warps(hg.count, ctx->sms) : 0u)));
     sa.nholes = &gc->nholes;
     sa.hole_total = &gc->holes;
     sa.ny_entries = (uint32_t)Y->nnz;

@@ -2,6 +2,8 @@
 oracle: one product per group up to the class's limit and past it, runs that repeat keys, more
 products than keys, groups of more than 32 entries, and free key spaces at the limit of the packed
 key (2^30)."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -52,3 +54,56 @@ def test_widest_packed_key(fy):
     res = check(X, Y, out_order=(1, 0))
     if fy == 1 << 30:  # not packed: no room for chunks either (no group has as many products as free keys)
         assert res.stats.out_capacity == res.stats.products
+
+
+def smallest_budget(call):
+    """The smallest budget of a context in which call(ctx) finds its memory."""
+    import paper_2410_10094_gb300 as stc
+
+    def fits(budget):
+        ctx = stc.Context(mem_budget_bytes=budget)
+        try:
+            call(ctx)
+            return True
+        except stc.StcError as e:
+            assert e.status == 4
+            return False
+        finally:
+            gc.collect()
+            ctx.close()
+
+    lo, hi = 1, 1 << 33
+    assert fits(hi)
+    while hi - lo > 1:
+        mid = (lo + hi) // 2
+        lo, hi = (lo, mid) if fits(mid) else (mid, hi)
+    return hi
+
+
+def test_budget_of_the_unchunked_call():
+    """Small groups enough to share counters, beside groups whose tables lie in global memory, in the
+    smallest budget of the call that scans its tables (which reserves no chunks): the call with direct
+    output needs no more, and its result holds no more."""
+    import oracle
+    import paper_2410_10094_gb300 as stc
+    from gpu_util import assert_matches_oracle, result_host, to_dev
+
+    rng = W.rng_for(8670)
+    small, large, fy = 20_000, 10, 60_000
+    length = np.array([45] * 40 + [5_000] * 5)
+    yk = np.repeat(np.arange(45), length)
+    Y = W.COO((45, fy), np.stack([yk, rng.integers(0, fy, len(yk))], 1).astype(np.int32), W.nonzero_values(rng, len(yk)))
+    xc = np.stack([np.concatenate([np.arange(small), small + np.repeat(np.arange(large), 5)]),
+                   np.concatenate([rng.integers(0, 40, small), np.tile(np.arange(40, 45), large)])], 1)
+    X = W.COO((small + large, 45), xc.astype(np.int32), W.nonzero_values(rng, len(xc)))
+    dev = to_dev(X), to_dev(Y), (1,), (0,)
+    how = dict(strategy=2, operands=stc.OPERANDS_AS_GIVEN)
+    need = smallest_budget(lambda ctx: stc.contract(*dev, accumulator=3, ctx=ctx, **how))
+    ctx = stc.Context(mem_budget_bytes=need)
+    res = stc.contract(*dev, accumulator=1, ctx=ctx, **how)
+    assert res.stats.table_slots > 0  # some groups' tables did lie in global memory
+    assert res.stats.out_capacity == res.stats.products  # every group has fewer products than free keys
+    assert_matches_oracle(*result_host(res), oracle.contract(X, Y, (1,), (0,), None))
+    del res
+    gc.collect()
+    ctx.close()
