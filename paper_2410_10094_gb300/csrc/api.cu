@@ -882,7 +882,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   STC_TRY(ar.alloc(&dbo, 1));
   StreamArgs sa{};
   if (nstream || chunk)
-    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg, ctx->sms) +
+    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg) +
                                     (chunk ? warp_chunk_warps(hg.count, ctx->sms) : 0u)));
   if (hh.count) {
     STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
@@ -951,37 +951,45 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     STC_CUDA(launch_group_stream(a, pr.yoff, nseg, seg, b.dense_list[0], nstream, sa, ctx->sms, s));
   }
   tm.mark(4);
-  // The holes are filled from the output's end before their number is known here, with scratch for
-  // as many as are to be expected: the chunks' rests, the streaming CTAs' last groups and the
-  // pieces they drop. More (or no memory for so many) take another pass below.
-  u64 most = 0;
-  u64* dst = nullptr;
-  uint8_t* marked = nullptr;
+  // The holes are filled from the output's end before their number is known here, in one round for
+  // as many positions as are to be expected: the chunks' rests, the streaming CTAs' last groups and
+  // the pieces they drop. More take further rounds below. The scratch is one word per position; where
+  // there is no memory for it, an array of the grouped X serves, which nothing reads any more.
+  HoleRound rd{};
   auto fill = [&]() -> stc_status {
-    STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, &pr.ctr->nz, &gc->holes, most, marked, dst, gc->fill_counters,
-                              r->coords, r->vals, pl.ocols, &pr.ctr->status, ctx->sms, s));
+    STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, &pr.ctr->nz, &gc->holes, rd, gc->fill_counters, r->coords, r->vals,
+                              pl.ocols, &pr.ctr->status, ctx->sms, s));
     tm.mark(5);
     return STC_OK;
   };
-  if (nstream || chunk) {
-    most = std::min<uint64_t>(out_cap, slack + std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64);
-    if (ar.alloc(&dst, (size_t)most) != STC_OK || ar.alloc(&marked, (size_t)most) != STC_OK) {
-      most = 0;
+  auto room = [&](uint64_t most) {
+    rd.win = most;
+    if (most > (uint64_t)nX) {
+      if (ar.alloc(&rd.dst, (size_t)most) == STC_OK) return;
       g_last_error.clear();
     }
+    rd.dst = gx.ystart;
+    rd.win = std::min<uint64_t>(most, (uint64_t)nX);
+  };
+  if (nstream || chunk) {
+    room(std::min<uint64_t>(out_cap, slack + std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64));
     STC_TRY(fill());
   }
   CallCounters hc2{};
   STC_TRY(read_counters(pr, pin, hc2));
   const u64 holes = hc2.g.holes;
   r->nnz = (int64_t)(hc2.c.nz - holes);
-  if (holes > most) {
-    most = holes;
-    STC_TRY(ar.alloc(&dst, (size_t)holes));
-    STC_TRY(ar.alloc(&marked, (size_t)holes));
-    STC_TRY(fill());
-    STC_TRY(read_counters(pr, pin, hc2));
+  if (holes > rd.win) {
+    const u64 done = rd.win;
+    room(holes - done);
+    for (rd.at = done; rd.at < holes; rd.at += rd.win) {
+      rd.base = hc2.g.fill_counters[1];
+      STC_TRY(fill());
+      STC_TRY(read_counters(pr, pin, hc2));
+    }
   }
+  if (hc2.g.fill_counters[0] != hc2.g.fill_counters[1])
+    return fail(STC_ERR_CUDA, "holes and entries to fill them do not match");
   r->stats.out_capacity = out_cap;
   r->mem = adopt(ar, ctx, s, {r->coords, r->vals});
   return STC_OK;

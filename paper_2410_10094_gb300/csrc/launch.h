@@ -388,7 +388,7 @@ cudaError_t launch_group_twopass(const GroupArgs& a, const Bins& b, const uint32
 
 // ------------------------------------------------------------------ streamed groups (stream.cu)
 struct StreamArgs {
-  StreamHole* holes;    // [stream_max_holes]
+  StreamHole* holes;    // [stream_max_holes], of fewer than 2^16 positions each
   unsigned* nholes;
   u64* hole_total;
   uint32_t ny_entries;  // entries of Y; the arrays hold one more (stream_dead_key)
@@ -399,16 +399,23 @@ struct StreamArgs {
   uint32_t ymod[6], ymagic[6], ysh1[6], ysh2[6];
 };
 uint32_t stream_cap();  // most products of a streamed group
-size_t stream_max_holes(uint32_t count, uint32_t nseg, int sms);
+size_t stream_max_holes(uint32_t count, uint32_t nseg);
 cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                 const uint32_t* list, uint32_t count, const StreamArgs& sa, int sms, cudaStream_t s);
-// Moves the last of the `*reserved` positions' entries into the holes, of which there are
-// *hole_total positions: the outputs are then the first *reserved - *hole_total. Both are read on
-// the device; with more than `most` hole positions nothing is moved. marked [most] and dst [most]
-// are scratch.
-cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, const u64* reserved,
-                             const u64* hole_total, u64 most, uint8_t* marked, u64* dst, u64* counters2,
-                             int32_t* coords, double* vals, int oz, uint32_t* status, int sms, cudaStream_t s);
+// One round of filling the holes: moves entries from the last *hole_total of the *reserved positions
+// into the holes before them; after the rounds that cover all *hole_total positions, the outputs are
+// the first *reserved - *hole_total. Both counts are read on the device.
+struct HoleRound {
+  u64 at;         // the window of those positions that this round moves entries from: [at, at + win);
+  u64 win;        // the rounds start at 0 and follow one another (part of it may lie past the end)
+  u64 base;       // entries moved by the rounds before (counters2[1])
+  uint32_t* dst;  // [win] scratch
+};
+// holes: rewritten by the first round. counters2: zeroed before the first round; destinations and
+// entries moved.
+cudaError_t launch_hole_fill(StreamHole* holes, const unsigned* nholes, const u64* reserved, const u64* hole_total,
+                             const HoleRound& rd, u64* counters2, int32_t* coords, double* vals, int oz,
+                             uint32_t* status, int sms, cudaStream_t s);
 
 // Lane-private dense rows for output rows of at most 64 free keys (FY <= 64, 32-bit Y free
 // keys): one warp per group g in [0, ngroups) (empty groups skipped), outputs in key order.

@@ -42,7 +42,7 @@ constexpr uint32_t kList = 512;   // repeats kept in shared memory
 constexpr uint32_t kHash = 1024;  // table of their keys
 constexpr uint32_t kHashEmpty = 0xffffffffu, kNoPlace = 0x8000u;
 static_assert(kQuarters % kStep == 0, "the quarter-slot table holds whole steps");
-static_assert(kEntries <= 4096 && kCap <= 65536, "field widths");
+static_assert(kEntries <= 4096 && kCap < 65536, "field widths");
 
 struct StreamSmem {
   uint32_t bits[kWords + 4]; // keys met (and the lanes' without a product, at most key 2^16);
@@ -472,50 +472,65 @@ __global__ void __launch_bounds__(T, 4)
   if (threadIdx.x == 0) add_hole(cur, left);
 }
 
-// Holes below the final count nnz become destinations (numbered through *ndst), those above it are
-// marked.
-__global__ void __launch_bounds__(256) hole_mark_kernel(const StreamHole* __restrict__ holes,
+// Filling the holes. With `tail` hole positions in all, the final count is nnz = reserved - tail: the
+// entries at nnz and above (sources) move to the hole positions below (destinations), of which there
+// are as many. Sources are taken a window of the tail at a time, in rounds that share one small array,
+// so that the filling works with whatever scratch there is.
+
+// A hole's words at and above nnz are marked in place: all ones, in a row's first and last word, is no
+// output (coordinates are at least 0 and keys below 2^64 - 1).
+__device__ __forceinline__ bool hole_marked(const int32_t* row, int oz) { return (row[0] & row[oz - 1]) == -1; }
+
+// FIRST: holes above nnz are marked, the positions below are numbered through *ndst, and each hole
+// becomes {position, number of its first destination << 16 | destinations}. Then the round's
+// destinations [base, base + win) are listed: dst[k - base] is the hole that number k lies in.
+template <bool FIRST>
+__global__ void __launch_bounds__(256) hole_list_kernel(StreamHole* __restrict__ holes,
                                                         const unsigned* __restrict__ nholes,
                                                         const u64* __restrict__ reserved,
-                                                        const u64* __restrict__ hole_total, u64 most,
-                                                        uint8_t* __restrict__ marked, u64* __restrict__ dst,
-                                                        u64* __restrict__ ndst) {
+                                                        const u64* __restrict__ hole_total, HoleRound rd,
+                                                        int32_t* __restrict__ coords, int oz, u64* __restrict__ ndst) {
   const unsigned lane = lane_id(), n = *nholes;
-  const u64 tail = *hole_total;
-  if (tail > most) return;
-  const u64 nnz = *reserved - tail;
+  const u64 nnz = *reserved - *hole_total;
   for (unsigned i = blockIdx.x * 8 + (threadIdx.x >> 5); i < n; i += gridDim.x * 8) {
-    const StreamHole h = holes[i];
-    const u64 end = h.pos + h.len, cut = end < nnz ? end : (h.pos < nnz ? nnz : h.pos);
-    const u64 below = cut - h.pos;
-    u64 k = 0;
-    if (lane == 0 && below) k = atomicAdd(ndst, below);
-    k = __shfl_sync(0xffffffffu, k, 0);
-    for (u64 j = lane; j < below; j += 32) dst[k + j] = h.pos + j;
-    for (u64 q = cut + lane; q < end; q += 32) marked[q - nnz] = 1;
+    StreamHole h = holes[i];
+    if (FIRST) {
+      const u64 end = h.pos + h.len, cut = end < nnz ? end : (h.pos < nnz ? nnz : h.pos);
+      const u64 below = cut - h.pos;
+      u64 k = 0;
+      if (lane == 0 && below) k = atomicAdd(ndst, below);
+      k = __shfl_sync(0xffffffffu, k, 0);
+      for (u64 q = cut + lane; q < end; q += 32) coords[q * oz] = coords[q * oz + oz - 1] = -1;
+      h.len = k << 16 | below;
+      if (lane == 0) holes[i] = h;
+    }
+    const u64 k0 = h.len >> 16, k1 = k0 + (h.len & 0xffffu);
+    const u64 a = k0 > rd.base ? k0 : rd.base, e = k1 < rd.base + rd.win ? k1 : rd.base + rd.win;
+    for (u64 k = a + lane; k < e; k += 32) rd.dst[k - rd.base] = i;
   }
 }
 
-// The entries of [nnz, nnz + tail) that are no holes move to the destinations.
-__global__ void __launch_bounds__(256) hole_fill_kernel(const uint8_t* __restrict__ marked,
+// The window's entries that are no holes move to the destinations that follow the last round's.
+__global__ void __launch_bounds__(256) hole_fill_kernel(const StreamHole* __restrict__ holes,
                                                         const u64* __restrict__ reserved,
-                                                        const u64* __restrict__ hole_total, u64 most,
-                                                        const u64* __restrict__ dst, u64* __restrict__ nsrc,
+                                                        const u64* __restrict__ hole_total, HoleRound rd,
+                                                        const u64* __restrict__ ndst, u64* __restrict__ nsrc,
                                                         int32_t* __restrict__ coords, double* __restrict__ vals,
                                                         int oz, uint32_t* status) {
-  const u64 tail = *hole_total;
-  if (tail > most) return;
+  const u64 tail = *hole_total, last = *ndst;
   const u64 nnz = *reserved - tail;
-  for (u64 t0 = ((u64)blockIdx.x * 256 + threadIdx.x) & ~31ull; t0 < tail; t0 += (u64)gridDim.x * 256) {
-    const u64 t = t0 + lane_id();
-    const bool has = t < tail && !marked[t];
+  const u64 end = tail < rd.at + rd.win ? tail : rd.at + rd.win;
+  for (u64 t0 = rd.at + (((u64)blockIdx.x * 256 + threadIdx.x) & ~31ull); t0 < end; t0 += (u64)gridDim.x * 256) {
+    const u64 t = t0 + lane_id(), s = nnz + t;
+    const bool has = t < end && !hole_marked(coords + s * oz, oz);
     const u64 k = warp_reserve(has, nsrc);
     if (!has) continue;
-    const u64 d = k < tail ? dst[k] : nnz, s = nnz + t;
-    if (d >= nnz) {
+    if (k >= last) {
       atomicOr(status, kStatOutOverflow);
       continue;
     }
+    const StreamHole h = holes[rd.dst[k - rd.base]];
+    const u64 d = h.pos + (k - (h.len >> 16));
     if (oz == 4 && ((reinterpret_cast<uintptr_t>(coords) & 15u) == 0)) {
       reinterpret_cast<int4*>(coords)[d] = reinterpret_cast<const int4*>(coords)[s];
     } else {
@@ -553,7 +568,9 @@ uint32_t stream_dead_key(u64 FY) { return FY > kDenseSeg ? 0xffffffffu : (uint32
 
 uint32_t stream_cap() { return kCap; }
 
-size_t stream_max_holes(uint32_t count, uint32_t nseg, int sms) { return (size_t)count * nseg + (size_t)sms * 4; }
+// A CTA drops positions at most once per segment, never in its first (it has none left over yet), and
+// lists what it has left over at its end.
+size_t stream_max_holes(uint32_t count, uint32_t nseg) { return (size_t)count * nseg; }
 
 cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                 const uint32_t* list, uint32_t count, const StreamArgs& sa_in, int sms,
@@ -594,17 +611,15 @@ cudaError_t launch_group_stream(const GroupArgs& a, const uint32_t* yoff, uint32
                   : launch_rows<false>(a, yoff, nseg, seg, list, count, sa, rows, sms, s);
 }
 
-cudaError_t launch_hole_fill(const StreamHole* holes, const unsigned* nholes, const u64* reserved,
-                             const u64* hole_total, u64 most, uint8_t* marked, u64* dst, u64* counters2,
-                             int32_t* coords, double* vals, int oz, uint32_t* status, int sms, cudaStream_t s) {
-  if (most == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(counters2, 0, 2 * sizeof(u64), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(marked, 0, most, s);
-  if (e != cudaSuccess) return e;
-  const u64 g = (u64)sms * 8, want = (most + 255) / 256;
-  hole_mark_kernel<<<(unsigned)(want < (u64)sms ? want : (u64)sms), 256, 0, s>>>(holes, nholes, reserved, hole_total,
-                                                                                most, marked, dst, counters2);
-  hole_fill_kernel<<<(unsigned)(want < g ? want : g), 256, 0, s>>>(marked, reserved, hole_total, most, dst,
+cudaError_t launch_hole_fill(StreamHole* holes, const unsigned* nholes, const u64* reserved, const u64* hole_total,
+                             const HoleRound& rd, u64* counters2, int32_t* coords, double* vals, int oz,
+                             uint32_t* status, int sms, cudaStream_t s) {
+  if (rd.win == 0 || oz <= 0) return cudaErrorInvalidValue;  // an output without modes has no holes
+  const u64 g = (u64)sms * 8, want = (rd.win + 255) / 256;
+  auto list = rd.at == 0 ? hole_list_kernel<true> : hole_list_kernel<false>;
+  list<<<(unsigned)(want < (u64)sms ? want : (u64)sms), 256, 0, s>>>(holes, nholes, reserved, hole_total, rd, coords, oz,
+                                                                     counters2);
+  hole_fill_kernel<<<(unsigned)(want < g ? want : g), 256, 0, s>>>(holes, reserved, hole_total, rd, counters2,
                                                                    counters2 + 1, coords, vals, oz, status);
   note_launch(2);
   return cudaGetLastError();

@@ -91,6 +91,43 @@ def test_groups_handing_on_positions(length, repeats):
         assert res.nnz == groups * length
 
 
+def mostly_repeats(rng):
+    """4,000 groups of 6,000 products on 500 to 520 keys each: more than ten million positions left over,
+    where the first filling of holes expects five."""
+    pool = rng.permutation(8192)[:520]
+    c = np.stack([np.repeat(np.arange(12), 500), np.concatenate([rng.permutation(pool)[:500] for _ in range(12)])], 1)
+    Y = W.COO((12, 8192), c.astype(np.int32), W.nonzero_values(rng, len(c)))
+    return W.Problem(rows(rng, 4_000, 12, 12), Y, (1,), (0,))
+
+
+def test_more_holes_than_expected():
+    """Filled in further rounds, with scratch for all of them."""
+    check(mostly_repeats(W.rng_for(8260)), accumulator=2)
+
+
+def test_holes_without_memory_for_them():
+    """A context with room for the call's arrays and its output: the holes are filled in rounds through
+    an array that the call has already."""
+    import gc
+
+    import oracle
+    import paper_2410_10094_gb300 as stc
+    from gpu_util import assert_matches_oracle, result_host, to_dev
+
+    p = mostly_repeats(W.rng_for(8270))
+    dev = to_dev(p.X), to_dev(p.Y), p.cx, p.cy
+    wide = stc.Context(mem_budget_bytes=8 << 30)
+    _, need = stc.count(*dev, ctx=wide)
+    wide.close()
+    tight = stc.Context(mem_budget_bytes=need + (1 << 20))
+    res = stc.contract(*dev, ctx=tight, strategy=2, accumulator=2, operands=stc.OPERANDS_AS_GIVEN)
+    assert res.stats.out_capacity == res.stats.products == 24_000_000
+    assert_matches_oracle(*result_host(res), oracle.contract(p.X, p.Y, p.cx, p.cy, None))
+    del res
+    gc.collect()
+    tight.close()
+
+
 @pytest.mark.parametrize("xs,ys,out", [((30, 5), (40, 25), None), ((32, 4), (64, 16), None), ((32, 4), (64, 16), (3, 1, 0, 2)),
                                        ((7, 5), (9, 120), (1, 0, 3, 2)), ((100,), (50, 20), None), ((100,), (1000,), None),
                                        ((10, 10), (10, 10, 10), None), ((5, 4, 3), (12, 9, 10), None),

@@ -12,14 +12,14 @@ import emulator
 HARNESS = r"""
 extern "C" int run_stream(uint32_t order, int sms, uint64_t FY, uint32_t groups, const uint32_t* goff, uint32_t* ystart,
                           uint32_t* w, uint32_t* ck, double* xv, const uint32_t* yoff, const uint32_t* yfk,
-                          const double* yv, uint32_t ny, uint64_t cap, int32_t* coords, double* vals, uint64_t* nnz,
+                          const double* yv, uint32_t ny, uint64_t cap, uint64_t win, int32_t* coords, double* vals, uint64_t* nnz,
                           uint64_t* holes) {
   using namespace stc;
   const uint32_t seg = FY > kDenseSeg ? kDenseSeg : [&] { uint32_t c = 64; while (c < FY) c <<= 1; return c; }();
   const uint32_t nseg = (uint32_t)((FY + seg - 1) / seg);
   std::vector<uint32_t> list(groups);
   for (uint32_t g = 0; g < groups; g++) list[g] = g;
-  std::vector<StreamHole> hl(stream_max_holes(groups, nseg, sms));
+  std::vector<StreamHole> hl(stream_max_holes(groups, nseg));
   unsigned nholes = 0;
   u64 nz = 0, total = 0, fill[2] = {0, 0};
   uint32_t status = 0;
@@ -47,12 +47,16 @@ extern "C" int run_stream(uint32_t order, int sms, uint64_t FY, uint32_t groups,
   emu::stuck = false;
   if (launch_group_stream(a, yoff, nseg, seg, list.data(), groups, sa, sms, nullptr)) return 1;
   if (nholes > hl.size() || nz > cap) return 2;
-  const u64 most = total;
-  std::vector<uint8_t> marked(most + 1);
-  std::vector<u64> dst(most + 1);
-  if (launch_hole_fill(hl.data(), &nholes, &nz, &total, most, marked.data(), dst.data(), fill, coords, vals, 2, &status,
-                       sms, nullptr))
-    return 3;
+  for (const StreamHole& h : hl)
+    if (h.len >= 65536) return 3;
+  std::vector<uint32_t> dst(win);
+  HoleRound rd{0, win, 0, dst.data()};
+  do {
+    rd.base = fill[1];
+    if (launch_hole_fill(hl.data(), &nholes, &nz, &total, rd, fill, coords, vals, 2, &status, sms, nullptr)) return 3;
+    rd.at += win;
+  } while (rd.at < total);
+  if (fill[0] != fill[1]) return 6;
   *nnz = nz - total;
   *holes = total;
   return emu::stuck ? 4 : status ? 5 : 0;
@@ -69,7 +73,7 @@ def ptr(a):
     return a.ctypes.data_as(ctypes.c_void_p)
 
 
-def run(lib, order, X, Y, FX, K, FY, sms=1):
+def run(lib, order, X, Y, FX, K, FY, sms=1, window=100_000):
     """X, Y: (free key, contract key, value) arrays; checks the outputs against plain sums."""
     xf, xk, xv = X
     yf, yk, yv = Y
@@ -95,7 +99,7 @@ def run(lib, order, X, Y, FX, K, FY, sms=1):
     a = [ystart.astype(np.uint32), w.astype(np.uint32), xk.astype(np.uint32), np.ascontiguousarray(xv), yoff,
          np.append(yf, dead).astype(np.uint32), np.append(yv, 0.0)]
     rc = lib.run_stream(ctypes.c_uint32(order), sms, ctypes.c_uint64(FY), ctypes.c_uint32(FX), ptr(goff), *map(ptr, a),
-                        ctypes.c_uint32(len(yf)), ctypes.c_uint64(products), ptr(coords), ptr(vals), ctypes.byref(nnz),
+                        ctypes.c_uint32(len(yf)), ctypes.c_uint64(products), ctypes.c_uint64(window), ptr(coords), ptr(vals), ctypes.byref(nnz),
                         ctypes.byref(holes))
     assert rc == 0
     n = nnz.value
@@ -139,3 +143,14 @@ def test_groups_of_several_pieces(lib, order):
     rng = np.random.default_rng(3)
     X, Y = tensors(rng, 6, 300, 40, 4, 5000, False)
     run(lib, order, X, Y, 6, 40, 5000)
+
+
+@pytest.mark.parametrize("window", [1, 31, 500, 4096])
+@pytest.mark.parametrize("order", SCHEDULES[:2])
+def test_holes_in_rounds(lib, order, window):
+    """The holes filled a window of the output's end at a time, down to a position per round: groups
+    whose products are mostly repeats, which drop positions again and again."""
+    rng = np.random.default_rng(window)
+    X, Y = tensors(rng, 20, 4, 3, 30, 60, False)
+    holes = run(lib, order, X, Y, 20, 3, 60, window=window)
+    assert holes > 500
