@@ -755,7 +755,7 @@ uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
   uint64_t b = bins_bytes(pl);
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
   b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
-  b += out * (4ull * pl.ocols + 8);  // the positions chunked reservations leave over only where there is room
+  b += out * (4ull * pl.ocols + 8);
   return b;
 }
 
@@ -872,38 +872,15 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   hh.cap = b.huge_cap;
   const uint32_t nstream = (dense_rows && !lane_rows) ? hg.count[kMaxClasses + 1] : 0u;
   bool direct = !wide && !lane_rows && out_cap < 0xffffffffull && o.accumulator != STC_ACC_HASH_SCAN;
-  // Chunked reservations leave positions over, at most `slack`, which the output then has room for.
-  // That is memory which a call without them does not need: none under a budget, and none that the
-  // call's other requests, made first, leave no room for.
-  uint32_t chunk = direct && ctx->budget == 0 ? warp_chunk(hg.count, pl.FY, out_cap, ctx->sms) : 0u;
-  uint64_t slack = (uint64_t)chunk * warp_chunk_warps(hg.count, ctx->sms);
-  if (out_cap + slack >= 0xffffffffull) chunk = 0, slack = 0;
+  STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
+  STC_TRY(ar.alloc_own(&r->vals, out_cap));
   BatchOut* dbo = nullptr;
   STC_TRY(ar.alloc(&dbo, 1));
-  StreamArgs sa{};
-  if (nstream || chunk)
-    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg) +
-                                    (chunk ? warp_chunk_warps(hg.count, ctx->sms) : 0u)));
   if (hh.count) {
     STC_TRY(ar.alloc(&hh.keys, hg.huge_slots));
     STC_TRY(ar.alloc(&hh.vals, hg.huge_slots));
     STC_CUDA(cudaMemsetAsync(hh.keys, 0xff, hg.huge_slots * sizeof(u64), s));
     STC_CUDA(cudaMemsetAsync(hh.vals, 0, hg.huge_slots * sizeof(double), s));
-  }
-  if (chunk && (ar.alloc_own(&r->coords, (out_cap + slack) * (size_t)pl.ocols) != STC_OK ||
-                ar.alloc_own(&r->vals, out_cap + slack) != STC_OK)) {
-    chunk = 0;
-    slack = 0;
-    g_last_error.clear();
-    if (r->coords) ar.release(r->coords);
-    r->coords = nullptr;
-    r->vals = nullptr;
-  }
-  if (chunk) {
-    out_cap += slack;
-  } else {
-    STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
-    STC_TRY(ar.alloc_own(&r->vals, out_cap));
   }
   BatchOut bo_here{};
   static_assert(sizeof(BatchOut) <= kPinnedBytes / 2, "a page-locked block holds the counters and a descriptor");
@@ -930,14 +907,12 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   a.status = &pr.ctr->status;
   a.bout = dbo;
   a.bnz = &pr.ctr->nz;
-  if (nstream || chunk) {
+  StreamArgs sa{};
+  if (nstream) {
+    STC_TRY(ar.alloc(&sa.holes, stream_max_holes(nstream, nseg)));
     sa.nholes = &gc->nholes;
     sa.hole_total = &gc->holes;
     sa.ny_entries = (uint32_t)Y->nnz;
-    a.chunk = chunk;
-    a.holes = sa.holes;
-    a.nholes = sa.nholes;
-    a.hole_total = sa.hole_total;
   }
   if (lane_rows) {
     STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, h.P, ctx->sms, s));
@@ -952,9 +927,9 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   }
   tm.mark(4);
   // The holes are filled from the output's end before their number is known here, in one round for
-  // as many positions as are to be expected: the chunks' rests, the streaming CTAs' last groups and
-  // the pieces they drop. More take further rounds below. The scratch is one word per position; where
-  // there is no memory for it, an array of the grouped X serves, which nothing reads any more.
+  // as many positions as are to be expected: the streaming CTAs' last groups and the pieces they
+  // drop. More take further rounds below. The scratch is one word per position; where there is no
+  // memory for it, an array of the grouped X serves, which nothing reads any more.
   HoleRound rd{};
   auto fill = [&]() -> stc_status {
     STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, &pr.ctr->nz, &gc->holes, rd, gc->fill_counters, r->coords, r->vals,
@@ -963,16 +938,20 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     return STC_OK;
   };
   auto room = [&](uint64_t most) {
-    rd.win = most;
+    uint32_t* more = nullptr;
     if (most > (uint64_t)nX) {
-      if (ar.alloc(&rd.dst, (size_t)most) == STC_OK) return;
+      if (ar.alloc(&more, (size_t)most) == STC_OK) {
+        rd.dst = more;
+        rd.win = most;
+        return;
+      }
       g_last_error.clear();
     }
-    rd.dst = gx.ystart;
-    rd.win = std::min<uint64_t>(most, (uint64_t)nX);
+    if (!rd.dst) rd.dst = gx.ystart, rd.win = (uint64_t)nX;
+    rd.win = std::min<uint64_t>(rd.win, most);
   };
-  if (nstream || chunk) {
-    room(std::min<uint64_t>(out_cap, slack + std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64));
+  if (nstream) {
+    room(std::min<uint64_t>(out_cap, std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64));
     STC_TRY(fill());
   }
   CallCounters hc2{};

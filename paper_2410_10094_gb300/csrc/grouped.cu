@@ -1715,10 +1715,9 @@ cudaError_t launch_warp_direct_class(const GroupArgs& a, const uint32_t* list, c
 
 // ---- small groups of a single contraction: a warp takes PK groups at a time and treats their X
 // entries as one list, with one table whose keys carry the group's number in their top bits, so that
-// PK groups share every load, scan and table clearing that a group alone would wait for. Output
-// positions come from chunks that the warp reserves (GroupArgs::chunk): all groups of the contraction
-// draw on one counter, whose atomics serialise. Otherwise as group_warp_direct_kernel.
-// Measured on 4e5 groups of 63 products (lengths 100, order 5 with order 4, 5e5 entries each): 0.61
+// PK groups share every load, scan, table clearing and reservation of output positions that a group
+// alone would wait for. Otherwise as group_warp_direct_kernel.
+// Measured on 4e5 groups of 63 products (lengths 100, order 5 with order 4, 5e5 entries each): 0.64
 // against 0.88 ms; on 4,096 groups of 95 the four groups of a warp wait for one another longer than
 // the idle warps would help (60 against 40 us), so few groups keep a warp each.
 constexpr uint32_t kPackMinGroups = 16384;
@@ -1750,8 +1749,6 @@ __global__ void __launch_bounds__(256) group_pack_kernel(const __grid_constant__
   const uint64_t keep = policy_evict_last();
   const uint64_t pol = policy_evict_first();
   const uint32_t* const yfk = static_cast<const uint32_t*>(a.yfk);
-  u64 cur = 0;  // positions [cur, cur + rem) are this warp's to fill
-  uint32_t rem = 0;
   const uint32_t packs = (count + PK - 1) / PK, step = gridDim.x * WARPS;
   // The next pack's groups (lane q holds the q-th) and their entries' ranges are loaded ahead.
   uint32_t g_n = 0, x0_n = 0, x1_n = 0, g_nn = 0;
@@ -1845,28 +1842,13 @@ __global__ void __launch_bounds__(256) group_pack_kernel(const __grid_constant__
           m[u] = __ballot_sync(0xffffffffu, mine);
           nclaim += __popc(m[u]);
         }
-        // nclaim positions: the i-th is pa + i below na, pb + i from there on.
-        u64 pa = cur, pb = 0;
-        uint32_t na = nclaim;
-        if (nclaim <= rem) {
-          cur += nclaim;
-          rem -= nclaim;
-        } else {
-          const uint32_t extra = nclaim - rem, size = extra > a.chunk ? extra : a.chunk;
-          u64 nb = 0;
-          if (lane == 0) nb = atomicAdd(a.nz, (u64)size);
-          nb = __shfl_sync(0xffffffffu, nb, 0);
-          na = rem;
-          pb = nb - rem;
-          cur = nb + extra;
-          rem = size - extra;
-        }
-        uint32_t off = 0;
+        u64 out = 0;
+        if (lane == 0 && nclaim) out = atomicAdd(a.nz, (u64)nclaim);
+        out = __shfl_sync(0xffffffffu, out, 0);
 #pragma unroll
         for (int u = 0; u < D; u++) {
           if ((m[u] >> lane) & 1u) {
-            const uint32_t i = off + __popc(m[u] & lt);
-            const u64 pos = i + (i < na ? pa : pb);
+            const u64 pos = out + __popc(m[u] & lt);
             ws.spos[slot[u]] = (uint32_t)pos;
             const uint32_t fk = PK > 1 ? key[u] & ((1u << kPackBits) - 1u) : key[u];
             if (pos < a.out_cap)
@@ -1874,7 +1856,7 @@ __global__ void __launch_bounds__(256) group_pack_kernel(const __grid_constant__
             else
               atomicOr(a.status, kStatOutOverflow);
           }
-          off += __popc(m[u]);
+          out += __popc(m[u]);
         }
         __syncwarp();
 #pragma unroll
@@ -1890,10 +1872,6 @@ __global__ void __launch_bounds__(256) group_pack_kernel(const __grid_constant__
     for (uint32_t i = lane; i < kPackSlots / 4; i += 32)
       reinterpret_cast<uint4*>(ws.keys)[i] = make_uint4(kEmpty32, kEmpty32, kEmpty32, kEmpty32);
     __syncwarp();
-  }
-  if (rem && lane == 0) {
-    a.holes[atomicAdd(a.nholes, 1u)] = StreamHole{cur, rem};
-    atomicAdd(a.hole_total, (u64)rem);
   }
 }
 
@@ -2127,20 +2105,6 @@ cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, 
 // Whether the warp classes of a single contraction take several groups per warp (group_pack_kernel).
 static bool packs(uint32_t small, uint32_t medium, u64 FY) {
   return (u64)small + medium >= kPackMinGroups && FY < (1u << kPackBits);
-}
-
-uint32_t warp_chunk_warps(const uint32_t* counts, int sms) {
-  const uint32_t most = (uint32_t)sms * 64;
-  return std::min(counts[0], most) + std::min(counts[1], most);
-}
-
-// One reservation per group and round would be one atomic on the same address each, at about 0.7 ns:
-// 0.27 ms for 4e5 groups. Chunks of up to 512 positions per warp cost at most half of the output's
-// bound in positions left over, which are filled from the output's end.
-uint32_t warp_chunk(const uint32_t* counts, u64 FY, u64 out_cap, int sms) {
-  if (!packs(counts[0], counts[1], FY)) return 0;
-  const u64 c = out_cap / (2 * (u64)warp_chunk_warps(counts, sms));
-  return c < 32 ? 0 : (uint32_t)(c < 512 ? c : 512);
 }
 
 cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct, const Bins& b,

@@ -240,12 +240,6 @@ struct GroupArgs {
   // different (run_unique_kernel). A group of one X entry over such a run has one product per
   // output, and the warp kernels write it as a scaled copy of the run without a table.
   const uint8_t* yuniq;
-  // Single contractions: warps of the small classes reserve positions `chunk` at a time (0: as
-  // many as they need) and list what they leave (room for warp_chunk_warps holes).
-  uint32_t chunk;
-  StreamHole* holes;
-  unsigned* nholes;
-  u64* hole_total;
 };
 
 // Where one group's outputs go, resolved once per group.
@@ -290,10 +284,6 @@ cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, 
 cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct, const Bins& b,
                                  const uint32_t* counts, int sms, cudaStream_t s, int depth = 0);
 cudaError_t launch_group_huge(const GroupArgs& a, const HugeGroups& h, bool wide_keys, int sms, cudaStream_t s);
-// Most warps that the warp classes' direct kernels run for these counts, and the chunk of
-// positions each should reserve at a time (GroupArgs::chunk; 0 where they do not share counters).
-uint32_t warp_chunk_warps(const uint32_t* counts, int sms);
-uint32_t warp_chunk(const uint32_t* counts, u64 FY, u64 out_cap, int sms);
 
 // ------------------------------------------------------------------ batches (batch.cu)
 // One problem of a batch as the device kernels see it.

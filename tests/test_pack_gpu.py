@@ -1,4 +1,4 @@
-"""Many small groups of one contraction (four to a warp, output positions in chunks), against the
+"""Many small groups of one contraction (four to a warp), against the
 oracle: one product per group up to the class's limit and past it, runs that repeat keys, more
 products than keys, groups of more than 32 entries, and free key spaces at the limit of the packed
 key (2^30)."""
@@ -52,8 +52,7 @@ def test_widest_packed_key(fy):
     yc[::7, 1] = fy - 1
     Y = W.COO((50, fy), yc.astype(np.int32), W.nonzero_values(rng, 600))
     res = check(X, Y, out_order=(1, 0))
-    if fy == 1 << 30:  # not packed: no room for chunks either (no group has as many products as free keys)
-        assert res.stats.out_capacity == res.stats.products
+    assert res.stats.out_capacity == res.stats.products  # no group has as many products as free keys
 
 
 def smallest_budget(call):
@@ -80,10 +79,10 @@ def smallest_budget(call):
     return hi
 
 
-def test_budget_of_the_unchunked_call():
-    """Small groups enough to share counters, beside groups whose tables lie in global memory, in the
-    smallest budget of the call that scans its tables (which reserves no chunks): the call with direct
-    output needs no more, and its result holds no more."""
+def test_budget_of_the_scanned_tables():
+    """Small groups enough to be packed, beside groups whose tables lie in global memory, in the smallest
+    budget of the call that scans its tables: the call with direct output needs no more, and its result
+    holds no more."""
     import oracle
     import paper_2410_10094_gb300 as stc
     from gpu_util import assert_matches_oracle, result_host, to_dev
