@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "arena.h"
 #include "launch.h"
 
 using namespace stc;
@@ -38,11 +39,8 @@ struct TuneEntry {
   cudaEvent_t ev0[kTuneCand] = {}, ev1[kTuneCand] = {};
 };
 
-struct stc_ctx {
+struct stc_ctx : DevicePool {
   int device = 0;
-  size_t budget = 0;  // 0 = no cap
-  cudaMemPool_t pool = nullptr;
-  std::atomic<size_t> held{0};
   std::atomic<int64_t> live_results{0};
   int sms = 0;
   std::mutex tune_mu;
@@ -228,82 +226,6 @@ struct Pinned {
     } catch (...) {
       cudaFreeHost(p);
     }
-  }
-};
-
-// Stream-ordered scratch from the context's pool. Everything still held when the arena
-// dies is returned to the pool in stream order; `keep` hands a block to a result instead.
-// In a context without a budget, small requests share slabs of kSlab bytes: a call makes some
-// thirty of them, at about a microsecond of host time each to take and to return. (A budget
-// counts every request for itself.)
-struct Arena {
-  static constexpr size_t kSlab = 1 << 20, kSlabMost = 1 << 16;
-  stc_ctx* ctx;
-  cudaStream_t s;
-  struct Block { void* p; size_t bytes; };
-  std::vector<Block> blocks;
-  char* slab = nullptr;
-  size_t slab_left = 0;
-  Arena(stc_ctx* c, cudaStream_t st) : ctx(c), s(st) {}
-  ~Arena() {
-    for (auto& b : blocks) {
-      cudaFreeAsync(b.p, s);
-      ctx->held -= b.bytes;
-    }
-  }
-  template <typename T>
-  stc_status alloc(T** out, size_t count) {
-    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;
-    if (bytes == 0 || bytes > kSlabMost || ctx->budget) return alloc_own(out, count);
-    if (bytes > slab_left) {
-      char* p = nullptr;
-      if (alloc_own(&p, kSlab) != STC_OK) return alloc_own(out, count);
-      slab = p;
-      slab_left = kSlab;
-    }
-    *out = reinterpret_cast<T*>(slab);
-    slab += bytes;
-    slab_left -= bytes;
-    return STC_OK;
-  }
-  // A block of its own, which `keep` and `release` can find.
-  template <typename T>
-  stc_status alloc_own(T** out, size_t count) {
-    *out = nullptr;
-    const size_t bytes = count * sizeof(T);
-    if (bytes == 0) return STC_OK;
-    const size_t after = ctx->held.fetch_add(bytes) + bytes;
-    if (ctx->budget && after > ctx->budget) {
-      ctx->held -= bytes;
-      return fail(STC_ERR_OUT_OF_MEMORY, "request of %zu bytes exceeds the context budget (%zu of %zu held)", bytes,
-                  after - bytes, ctx->budget);
-    }
-    void* p = nullptr;
-    const cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, ctx->pool, s);
-    if (e != cudaSuccess) {
-      ctx->held -= bytes;
-      cudaGetLastError();
-      return fail(STC_ERR_OUT_OF_MEMORY, "device allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
-    }
-    blocks.push_back({p, bytes});
-    *out = static_cast<T*>(p);
-    return STC_OK;
-  }
-  // Gives one block back, in stream order.
-  void release(void* p) {
-    const size_t b = keep(p);
-    if (!b) return;
-    cudaFreeAsync(p, s);
-    ctx->held -= b;
-  }
-  size_t keep(void* p) {
-    for (size_t i = 0; i < blocks.size(); i++)
-      if (blocks[i].p == p) {
-        const size_t b = blocks[i].bytes;
-        blocks.erase(blocks.begin() + i);
-        return b;
-      }
-    return 0;
   }
 };
 
