@@ -644,10 +644,16 @@ uint64_t bins_bytes(const Plan& pl) {
   return b + (pl.id_map ? id_map_pairs(pl.K) * 8 + (uint64_t)id_map_scratch(pl.K) * 4 : (pl.K + 31) / 32 * 4);
 }
 
-// Whether the one-global-table strategy writes outputs as their keys are claimed: where the output
-// key space is at least twice the products, so that few are expected to repeat a key, and the list
-// of those that do stays below 1 GB. 3.2e6 products over 1.2e15 keys: 0.34 ms against 0.43 for
-// accumulating in the table and passing over its 2^23 slots.
+// Whether the one-global-table strategy writes outputs as their keys are claimed, where the list of
+// products that find their key claimed stays below 1 GB. It is the faster form whether products repeat
+// keys or not (ms for the contraction, against accumulating in the table and passing over its slots):
+// 3.2e6 products of 1.04 per key 0.71 against 0.79, 7.4e5 of 10.8 per key 0.28 against 0.29; 2e7 over a
+// large key space of 1, 10, 1,000 and 1e5 per key 2.04 against 2.47, 1.13 against 1.69, 0.88 against
+// 1.15, 0.74 against 0.99. The most it loses is 2e6 of 1,000 per key, 0.22 against 0.20. What counts is
+// the table: it has twice the smaller of products and keys, so that in small key spaces there is little
+// of it to pass over. 2e7 uniform products on F = 2, 1, 0.5 and 0.1 keys per product: 1.99 against 2.31,
+// 1.87 against 2.22, 1.53 against 1.65, 0.95 against 0.60; 6e7: 6.09 against 6.41, 5.88 against 6.09,
+// 5.33 against 4.95, 2.79 against 2.56. The line lies on the safe side, at two keys per product.
 bool direct_global(uint64_t P, uint64_t F, uint64_t cap) {
   return P <= F / 2 && P <= (1ull << 26) && cap <= (1ull << 32);
 }

@@ -39,14 +39,17 @@ def test_uneven_runs(nx, ny, fx, fy):
     check(X, Y, (1, 0))
 
 
-def test_all_products_on_few_keys():
-    """The rule expects few repeats; here almost every product is one."""
-    rng = W.rng_for(8820)
-    X, Y = W.uniform_coo(rng, (1_000_000, 20), 6_000), W.uniform_coo(rng, (20, 1_000), 900)
-    X.coords[:, 0] = rng.integers(0, 3, 6_000) * 333_333
-    Y.coords[:, 1] = rng.integers(0, 2, 900) * 999
+@pytest.mark.parametrize("nx,ny,fx,fy", [(6_000, 900, 3, 2), (6_000, 900, 1, 1), (12_000, 10_000, 32, 32), (12_000, 10_000, 25, 41)])
+def test_all_products_on_few_keys(nx, ny, fx, fy):
+    """Almost every product finds its key claimed: on either side of the 1,024 keys whose repeats each
+    CTA sums first. Up to 2.7e5 terms of random signs in a sum: rounding errors of two orders of
+    summation differ by about sqrt(n) u = 6e-14 of sum|x*y|, well inside REL_TOL."""
+    rng = W.rng_for(8820 + fx + fy)
+    X, Y = W.uniform_coo(rng, (3_000_000, 20), nx), W.uniform_coo(rng, (20, 4_100), ny)
+    X.coords[:, 0] = rng.integers(0, fx, nx) * 30_001
+    Y.coords[:, 1] = rng.integers(0, fy, ny) * 99
     res = check(X, Y)
-    assert res.nnz == 6
+    assert res.nnz == fx * fy
 
 
 @pytest.mark.parametrize("fy", [2 * 1_300 - 1, 2 * 1_300, 2 * 1_300 + 1])
