@@ -658,10 +658,18 @@ bool direct_global(uint64_t P, uint64_t F, uint64_t cap) {
   return P <= F / 2 && P <= (1ull << 26) && cap <= (1ull << 32);
 }
 
+// Cells of the array that holds an output space of F keys (launch_clear_space). The keys of smaller
+// spaces than 2^15 are spread over as many cells, so that they share few lines: 4e7 products on 64 x 64
+// keys take 0.61 ms for the contraction, on 4,096 cells 1.09, in a table 0.83; on 4 x 4 keys 5.6, 13.4
+// and 15.6. Under a budget no more than the table would take that the array stands for.
+uint64_t space_cells(const stc_ctx* ctx, uint64_t F) {
+  return pow2_at_least(std::max<uint64_t>(F, ctx->budget ? std::min<uint64_t>(2 * F, 1 << 15) : 1 << 15));
+}
+
 // Peak device bytes of the GLOBAL strategy for these counts.
 uint64_t global_bytes(const stc_ctx* ctx, const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint64_t P,
                       double alpha) {
-  // Small output key spaces are sized from F itself (no host read of P), with a prefix over nX.
+  // Small output key spaces are sized from F itself (no host read of P), with products per block of X.
   const bool from_f = pl.F <= kGlobalFromF;
   const uint64_t target = from_f ? pl.F : std::min<uint64_t>(P, pl.F);
   const uint64_t cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)target / alpha) + 1));
@@ -669,7 +677,7 @@ uint64_t global_bytes(const stc_ctx* ctx, const Plan& pl, int64_t nX, int64_t nY
   uint64_t b = bins_bytes(pl);
   b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
   b += from_f ? (2 * survivor_blocks(nX) + 1) * 8 : (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
-  b += cap * 16 + out_cap * (4ull * pl.ocols + 8);
+  b += std::max(cap * 16, from_f ? space_cells(ctx, pl.F) * 8 : 0) + out_cap * (4ull * pl.ocols + 8);
   if (!from_f && direct_global(P, pl.F, cap) && ctx->budget == 0) b += P * 12;
   return b;
 }
@@ -1755,8 +1763,8 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     // space: no hashing and no claims (4096 x 64 outputs, 1.6e6 products, X of 2e7 entries: 0.242 ->
     // 0.225 ms for the contraction).
     const bool whole = o.probe == 0 && o.load_factor == 0.0;
-    const uint64_t cap =
-        whole ? pl.F : pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)pl.F / alpha) + 1));
+    const uint64_t cap = whole ? space_cells(ctx, pl.F)
+                               : pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)pl.F / alpha) + 1));
     const uint64_t out_cap = std::min<uint64_t>(pl.F, cap);
     const int64_t nX = X->nnz;
     stc_result* r = new stc_result;
@@ -1769,25 +1777,23 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
     auto run = [&]() -> stc_status {
       GlobalTable t{};
       u64* bpre = nullptr;
-      uint8_t* seen = nullptr;
-      if (whole) {
-        STC_TRY(ar.alloc(&t.vals, cap + (cap + 7) / 8));  // and the bytes behind them
-        seen = reinterpret_cast<uint8_t*>(t.vals + cap);
-      } else {
-        STC_TRY(ar.alloc(&t.keys, cap));
-        STC_TRY(ar.alloc(&t.vals, cap));
-      }
+      if (!whole) STC_TRY(ar.alloc(&t.keys, cap));
+      STC_TRY(ar.alloc(&t.vals, cap));
       STC_TRY(ar.alloc(&bpre, survivor_blocks(nX) + 1));
       STC_TRY(ar.alloc_own(&r->coords, out_cap * (size_t)pl.ocols));
       STC_TRY(ar.alloc_own(&r->vals, out_cap));
       t.mask = cap - 1;
-      if (!whole) STC_CUDA(cudaMemsetAsync(t.keys, 0xff, cap * sizeof(u64), s));
-      STC_CUDA(cudaMemsetAsync(t.vals, 0, cap * sizeof(double) + (whole ? cap : 0), s));
+      if (whole) {
+        STC_CUDA(launch_clear_space(t, ctx->sms, s));
+      } else {
+        STC_CUDA(cudaMemsetAsync(t.keys, 0xff, cap * sizeof(u64), s));
+        STC_CUDA(cudaMemsetAsync(t.vals, 0, cap * sizeof(double), s));
+      }
       tm.mark(3);
-      STC_CUDA(launch_expand_blocks(pr.sv, bpre, static_cast<const u64*>(pr.yfk), pr.yv, pl.FY, t, seen,
+      STC_CUDA(launch_expand_blocks(pr.sv, bpre, static_cast<const u64*>(pr.yfk), pr.yv, pl.FY, t,
                                     &pr.ctr->status, ctx->sms, s, probe));
       tm.mark(4);
-      STC_CUDA(launch_compact_global(t, seen, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status,
+      STC_CUDA(launch_compact_global(t, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status,
                                      ctx->sms, s));
       tm.mark(5);
       CallCounters hc{};
@@ -1886,7 +1892,7 @@ stc_status contract_impl(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32
         STC_CUDA(launch_expand_global(wpre, (int64_t)h.ns, h.P, pr.sv, static_cast<const u64*>(pr.yfk), pr.yv,
                                       pl.FY, t, &pr.ctr->status, ctx->sms, s, probe));
         tm.mark(4);
-        STC_CUDA(launch_compact_global(t, nullptr, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status,
+        STC_CUDA(launch_compact_global(t, pl.op, r->coords, r->vals, out_cap, &pr.ctr->nz, &pr.ctr->status,
                                        ctx->sms, s));
         tm.mark(5);
         CallCounters hc2{};

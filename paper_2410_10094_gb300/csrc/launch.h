@@ -124,7 +124,7 @@ cudaError_t launch_id_rewrite_rows(const int32_t* coords, int64_t n, const KeyPl
 
 // ------------------------------------------------------------------ one global table (global.cu)
 struct GlobalTable {
-  u64* keys;    // [cap], kEmpty64 when free
+  u64* keys;    // [cap], kEmpty64 when free; null: an array of the whole output space (cap >= F)
   double* vals; // [cap]
   u64 mask;     // cap - 1, cap a power of two
 };
@@ -137,13 +137,13 @@ cudaError_t launch_expand_global(const u64* wpre, int64_t ns, u64 P, Survivors s
                                  cudaStream_t s, int probe);
 // The same with everything read on the device (no host read between the survey and the expansion):
 // the survivor count, and the products per block of survivors (sv.bsum), whose prefix a first kernel
-// writes to bpre (one element more than sv.bsum). With `seen` the table is an array of the whole
-// output key space (t.vals, zeroed, mask + 1 = F) and seen[F], zeroed, receives 1 for every key that
-// has a product.
+// writes to bpre (one element more than sv.bsum). t.keys null: t is an array of the whole output space,
+// cleared by launch_clear_space.
 cudaError_t launch_expand_blocks(Survivors sv, u64* bpre, const u64* yfk, const double* yv, u64 FY, GlobalTable t,
-                                 uint8_t* seen, uint32_t* status, int sms, cudaStream_t s, int probe);
-// The same for outputs with few repeats: outputs written as their keys are claimed, repeats listed
-// and added by a second kernel.
+                                 uint32_t* status, int sms, cudaStream_t s, int probe);
+cudaError_t launch_clear_space(GlobalTable t, int sms, cudaStream_t s);
+// The same for large output key spaces: outputs written as their keys are claimed, repeats listed and
+// added by a second kernel.
 struct DirectTable {
   u64* keys;           // [mask + 1], kEmpty64 when free
   uint32_t* pos;       // [mask + 1] output position of the slot's key
@@ -155,9 +155,9 @@ struct DirectTable {
 cudaError_t launch_expand_direct(const u64* wpre, int64_t ns, u64 P, Survivors sv, const u64* yfk, const double* yv,
                                  u64 FY, const DirectTable& t, const OutPlan& op, int32_t* coords, double* vals,
                                  u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);
-// Occupied slots -> COO output (coordinates decoded from the key); seen: see launch_expand_blocks.
-cudaError_t launch_compact_global(GlobalTable t, const uint8_t* seen, const OutPlan& op, int32_t* coords, double* vals,
-                                  u64 out_cap, u64* nz, uint32_t* status, int sms, cudaStream_t s);
+// Occupied slots -> COO output (coordinates decoded from the key).
+cudaError_t launch_compact_global(GlobalTable t, const OutPlan& op, int32_t* coords, double* vals, u64 out_cap,
+                                  u64* nz, uint32_t* status, int sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ per-group tables (grouped.cu)
 constexpr int kMaxClasses = 5;

@@ -45,6 +45,31 @@ def test_cancelled_outputs_stay():
     check(X, Y)
 
 
+@pytest.mark.parametrize("x,y", [(-0.0, 3.0), (0.0, -3.0), (-0.0, -3.0), (1e-200, -1e-200)])
+def test_products_of_zero(x, y):
+    """Zeros of either sign, given or underflown, are products like any other: their outputs exist, and
+    are +0.0 where nothing else is added."""
+    X = W.COO((4, 2), np.array([[1, 0], [2, 0], [3, 1]], np.int32), np.array([x, x, 2.0]))
+    Y = W.COO((2, 5), np.array([[0, 4], [0, 4], [0, 0], [1, 0]], np.int32), np.array([y, y, y, 1.0]))
+    import oracle
+    from gpu_util import gpu_contract, result_host
+
+    c, v = result_host(gpu_contract(W.Problem(X, Y, (1,), (0,)), strategy=1))
+    ref = oracle.contract(X, Y, (1,), (0,))
+    at = np.lexsort(c.T[::-1])
+    np.testing.assert_array_equal(c[at], ref.coords)
+    np.testing.assert_array_equal(v[at], ref.vals)
+    assert not np.signbit(v[v == 0]).any()
+
+
+@pytest.mark.parametrize("shape,row", [((2000, 130), 1), ((4096, 64), 3), ((37, 4095), 1), ((1, 300), 1)])
+def test_most_products_on_few_rows(shape, row):
+    rng = W.rng_for(8970 + shape[0])
+    X, Y = W.uniform_coo(rng, (shape[0], 200), 8_000), W.uniform_coo(rng, (200, shape[1]), 6_000)
+    X.coords[500:, 0] = rng.integers(0, row, 7_500)
+    check(X, Y)
+
+
 def test_one_long_run_among_short_ones():
     rng = W.rng_for(8960)
     Y = W.uniform_coo(rng, (500, 64), 20_000)
