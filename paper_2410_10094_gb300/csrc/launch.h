@@ -363,13 +363,20 @@ uint32_t dense_stash_cap();
 
 // ------------------------------------------------------------------ batches' larger groups (twopass.cu)
 // The list (form) of the two-pass kernel for a group of `products` products by `entries` X entries over
-// F_Y free keys, or -1 where the group belongs to the hash tables. Measured against those with 3e7
-// products in groups of one size: 1.4 to 1.5 times as fast at 3,750 products (F_Y 6e4), 2.6 to 4.0
-// beyond 8,192 (whose tables lie in global memory); the lead falls as keys repeat, 1.12 to 1.19 at 2 to
-// 4 products per key and 0.96 to 1.14 at 8, where the line is drawn. Groups of the 1,024-slot warp
-// tables lose (the batch of 256 pairs: 15.3 against 13.8 ms with those above 320 products taken in).
+// F_Y free keys, or -1 where the group belongs to the hash tables. Accumulation of 3e7 products in groups
+// of one size, the tables' time over the two-pass kernel's:
+//   form 0, 800 to 8,000 products: even keys 1.2 to 1.8; keys by a Zipf law of exponent 1.0 0.9 to 1.5, of
+//     1.5 0.9 to 1.3; all products on 60 keys 0.7 (1,500) to 1.2
+//   form 1, 6,000 to 12,000 products: 1.5 to 1.9; 1.0 to 1.1; 0.7; 0.8 to 1.0
+//   form 2, 40,000 products, whose tables lie in global memory: 6 to 10; 3.5 to 6; 1.7 to 2.4; 1.4 to 2.2
+//   form 1 at 800 and 3,000 products over more than 2^16 keys, where half as many groups are in flight:
+//     0.7 and 1.4; 0.7 and 0.9; 0.5 and 0.6; 0.5 and 0.6, so that the tables take those up to 6,144.
+// The lead falls as even keys repeat, 1.12 to 1.19 at 2 to 4 products per key and 0.96 to 1.14 at 8, where
+// the line is drawn. Groups of the 1,024-slot warp tables lose (the batch of 256 pairs: 15.3 against 13.8
+// ms with those above 320 products taken in).
 __host__ __device__ constexpr int twopass_list(u64 products, uint32_t entries, u64 FY) {
   if (FY > (1u << 18) || products > 49152 || entries > 1024 || products > 4 * FY) return -1;
+  if (FY > (1u << 16) && products <= 6144) return -1;
   if (FY <= (1u << 16) && products <= 8192 && entries <= 256) return 0;
   return products <= 16384 && entries <= 512 ? 1 : 2;
 }
