@@ -8,7 +8,7 @@
 // and one atomic on the problem's counter reserves exactly as many positions. Pass 2 reads keys and
 // values, writes the firsts' outputs, and puts the place of those whose key repeats into a small
 // table; repeats wait in a list and are added to their firsts' entries after a barrier. Groups with
-// more than kList repeats rank the repeated keys instead, and a third pass adds the repeats.
+// more repeats than are listed rank the repeated keys instead, and a third pass adds the repeats.
 #include "target.cuh"
 
 namespace stc {
@@ -16,7 +16,11 @@ namespace stc {
 namespace {
 
 constexpr int U = 4;  // slots per warp and step
-constexpr uint32_t kList = 512, kHash = 1024;
+// Most repeats listed, by groups of up to kListSmall products (larger ones list half as many), and the
+// slots of the table of their keys. 3e7 products in groups of 7,700 over 6e4 even keys (some 490 repeats)
+// take 0.60 ms listed and 0.30 ranked; in groups of 800 over keys by a Zipf law of exponent 1.0 (some 350)
+// 0.54 listed and 0.74 ranked.
+constexpr uint32_t kList = 512, kListSmall = 2048, kHash = 1024;
 constexpr uint32_t kHashEmpty = 0xffffffffu;
 
 template <int T, uint32_t WORDS, uint32_t CAP>
@@ -211,7 +215,7 @@ __global__ void __launch_bounds__(T, MINB) group_twopass_kernel(GroupArgs a, con
       run += __popc(sm.mask[i]);
     }
     const uint32_t reps = sm.reps;
-    const bool few = reps <= kList;
+    const bool few = reps <= (tot >> 13 <= kListSmall ? kList : kList / 2);
     const uint32_t nwords = (uint32_t)((sm.tg.FY + 31) >> 5);
     if (!few) {  // the key marks are no longer needed and hold the ranks of the repeated keys
       const uint32_t wpt = (nwords + T - 1) / T;

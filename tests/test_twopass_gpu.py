@@ -1,8 +1,8 @@
 """The larger groups of a batch by the two-pass kernel, against the oracle, called (also under a
 budget, which keeps the hash tables) and replayed: group sizes, free key spaces and entry counts at the
-limits of its three forms and one past them, 512 and 513 listed repeats, keys that repeat many times,
-runs scaled by one entry, rows of 2 to 9 coordinates, and more problems than the binning holds offsets
-for."""
+limits of its three forms and one past them, as many repeats as a small and a larger group list and one
+more, keys that repeat many times, runs scaled by one entry, rows of 2 to 9 coordinates, and more
+problems than the binning holds offsets for."""
 import numpy as np
 import pytest
 
@@ -72,11 +72,13 @@ def test_keys_that_repeat(keys):
            for i, (fy, n) in enumerate([((251, 241), 6000), ((401, 503), 6000), ((401, 503), 20000)])])
 
 
-@pytest.mark.parametrize("repeats", [511, 512, 513])
-def test_listed_repeats(repeats):
-    p = problem(30, 6, (9001,), 1500 + 1300, 2, 2)
-    first, second = np.arange(1500), np.concatenate([np.arange(repeats), 1500 + np.arange(1300 - repeats)])
-    p.Y.coords[:, 0] = np.repeat([0, 1], [1500, 1300])
+@pytest.mark.parametrize("runs,repeats", [((1500, 1300), 255), ((1500, 1300), 256), ((1500, 1300), 257), ((1500, 1300), 513),
+                                          ((1100, 948), 511), ((1100, 948), 512), ((1100, 948), 513), ((1100, 949), 512)])
+def test_listed_repeats(runs, repeats):
+    m, n = runs
+    p = problem(30, 6, (9001,), m + n, 2, 2)
+    first, second = np.arange(m), np.concatenate([np.arange(repeats), m + np.arange(n - repeats)])
+    p.Y.coords[:, 0] = np.repeat([0, 1], runs)
     p.Y.coords[:, 1] = np.concatenate([first * 5, second * 5 % 9001])
     check([p])
 
