@@ -851,7 +851,7 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     sa.ny_entries = (uint32_t)Y->nnz;
   }
   if (lane_rows) {
-    STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, h.P, ctx->sms, s));
+    STC_CUDA(launch_group_lanerow(a, pl.FX, (uint32_t)pl.FY, h.P, h.ns, ctx->sms, s));
   } else {
     STC_CUDA(launch_group_classes(a, wide, direct, b, hg.count, ctx->sms, s));
     STC_CUDA(launch_group_huge(a, hh, wide, ctx->sms, s));

@@ -2258,10 +2258,10 @@ __global__ void __launch_bounds__(kRowWarps * 32) group_lanerow_kernel(GroupArgs
   }
 }
 
-// The same with one CTA per group: its warps take pieces of kPiece X entries of the group until
-// none is left, each lane with a row of its own, and the warps' sums are added in warp order.
-// Groups whose products run into the tens of thousands keep a CTA busy, and a grid of one CTA per
-// SM ends evenly, where warps that own whole groups leave the last round of groups half empty.
+// The same with one CTA per group: its warps take pieces of the group, up to kPiece X entries or a
+// 13th of them, until none is left, each lane with a row of its own, and the warps' sums are added in
+// warp order. Groups whose products run into the tens of thousands keep a CTA busy, and a grid of one CTA
+// per SM ends evenly, where warps that own whole groups leave the last round of groups half empty.
 // The loads of the next products are issued before the current ones are added, so that the FP64
 // pipe (two rounded operations per product) is what bounds the loop: 2.04e10 products in 4,096
 // groups take 82.6 ms, 0.93 of half the measured rate of FP64 multiplies; by a warp per group 143.
@@ -2269,11 +2269,21 @@ __global__ void __launch_bounds__(kRowWarps * 32) group_lanerow_kernel(GroupArgs
 // absolute sum (rms, against extended precision), by one warp's 32 rows 9.1e-18.
 constexpr int kCtaRowWarps = 13;  // 13 x 32 rows of 65 doubles: 216 KB of shared memory
 constexpr int kPiece = 16;
-// The line: a CTA per group where there are at most four groups per SM (300 groups of 4,096
-// products 39 against 69 us, 600 66 against 76, 1,200 119 against 75) or the products average
-// kCtaRowMin per group (20,000 groups of 24,576 products 3.8 against 3.0 ms, 4,096 of 65,536 1.53
-// against 2.15, of 262,144 6.0 against 8.2).
-constexpr u64 kCtaRowMin = 49152;
+// The line, against a warp per group (ms), for groups of as many X entries as warps or more:
+//   up to two groups per SM, whatever they hold: 300 groups of 3,000 products 0.040 against 0.048, of one
+//     entry 0.058 against 0.057; 152 of 60,000 0.060 against 0.58, of one entry 0.42 against 1.1
+//   up to four: 600 of 3,000 0.067 against 0.047, of 20,000 0.111 against 0.219: equal at about 6,000
+//   up to eight: 1,000 of 3,000 0.111 against 0.047, of 20,000 0.183 against 0.215: equal at about 14,000
+//   more: 3,000 of 20,000 0.50 against 0.41, of 60,000 0.97 against 1.19; 20,000 of 20,000 3.24 against
+//     2.20, of 60,000 6.31 against 6.42.
+// Fewer entries leave warps idle: 1,000 of 20,000 from 8 entries 0.187 against 0.222, from 4 0.257 against
+// 0.247; 20,000 of 60,000 from 8 7.1 against 6.4, from one 51 against 11. Empty groups count: they are
+// passed over one after another.
+constexpr bool ctarow_pays(u64 groups, u64 products, u64 entries, u64 sms) {
+  if (groups <= 2 * sms) return true;
+  if (groups <= 8 * sms) return entries >= 8 * groups && products >= (groups <= 4 * sms ? 6144 : 16384) * groups;
+  return entries >= kCtaRowWarps * groups && products >= 49152 * groups;
+}
 constexpr size_t kCtaRowSmem = (size_t)kCtaRowWarps * 32 * kRowStride * sizeof(double);
 
 __global__ void __launch_bounds__(kCtaRowWarps * 32, 1) group_ctarow_kernel(GroupArgs a, u64 ngroups, uint32_t FY) {
@@ -2304,13 +2314,14 @@ __global__ void __launch_bounds__(kCtaRowWarps * 32, 1) group_ctarow_kernel(Grou
     const uint32_t x0 = a.goff[g], n = a.goff[g + 1] - x0;
     if (n == 0) continue;  // uniform over the CTA
     u64 seen = 0;
+    const uint32_t piece = n >= kPiece * kCtaRowWarps ? kPiece : (n + kCtaRowWarps - 1) / kCtaRowWarps;
     for (;;) {
       uint32_t c0 = 0;
-      if (lane == 0) c0 = atomicAdd(&s_next, (uint32_t)kPiece);
+      if (lane == 0) c0 = atomicAdd(&s_next, piece);
       c0 = __shfl_sync(0xffffffffu, c0, 0);
       if (c0 >= n) break;
       u64 w = 0;
-      if (lane < kPiece && c0 + lane < n) {
+      if (lane < piece && c0 + lane < n) {
         w = a.gx.w[x0 + c0 + lane];
         ysv[lane] = a.gx.ystart[x0 + c0 + lane];
         xv[lane] = a.gx.v[x0 + c0 + lane];
@@ -2395,10 +2406,11 @@ __global__ void __launch_bounds__(kCtaRowWarps * 32, 1) group_ctarow_kernel(Grou
   }
 }
 
-cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, int sms, cudaStream_t s) {
+cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, u64 entries, int sms,
+                                 cudaStream_t s) {
   if (ngroups == 0) return cudaSuccess;
   if (FY == 0 || FY > kRowMax) return cudaErrorInvalidValue;
-  if (ngroups <= 4 * (u64)sms || products / kCtaRowMin >= ngroups) {
+  if (ctarow_pays(ngroups, products, entries, (u64)sms)) {
     const cudaError_t e = cudaFuncSetAttribute(group_ctarow_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)kCtaRowSmem);
     if (e != cudaSuccess) return e;

@@ -415,8 +415,10 @@ cudaError_t launch_hole_fill(StreamHole* holes, const unsigned* nholes, const u6
                              uint32_t* status, int sms, cudaStream_t s);
 
 // Lane-private dense rows for output rows of at most 64 free keys (FY <= 64, 32-bit Y free
-// keys): one warp per group g in [0, ngroups) (empty groups skipped), outputs in key order.
-cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, int sms, cudaStream_t s);
+// keys): a warp or a CTA per group g in [0, ngroups) (empty groups skipped), outputs in key order.
+// products and entries: what they hold.
+cudaError_t launch_group_lanerow(const GroupArgs& a, u64 ngroups, uint32_t FY, u64 products, u64 entries, int sms,
+                                 cudaStream_t s);
 cudaError_t launch_group_dense(const GroupArgs& a, const uint32_t* yoff, uint32_t nseg, uint32_t seg,
                                const uint32_t* stash_list, uint32_t stash_count, const uint32_t* rank_list,
                                uint32_t rank_count, int sms, cudaStream_t s);
