@@ -100,8 +100,9 @@ enum { STC_ACC_AUTO = 0, STC_ACC_HASH = 1, STC_ACC_DENSE = 2, STC_ACC_HASH_SCAN 
  * first renumbered 0..D-1 and X and Y are rewritten with the id in place of their paired modes
  * (as stc_dense_ids does); stats.contract_ids = D. AUTO: DENSE when K > 2^26 (always, since
  * direct counting stops there) or when K exceeds both 2^22 and 8 (nX + nY); DIRECT otherwise.
- * Up to 2^30 keys AUTO may number the keys through a bitmap of the key space, without a
- * rewritten copy, in either case; the result and stats.contract_ids are the same. A DIRECT request with K > 2^26 is renumbered too. */
+ * Up to 2^28 keys AUTO may number the keys through a bitmap of the key space, without a
+ * rewritten copy, in either case; the result and stats.contract_ids are the same. A DIRECT request
+ * with K > 2^26 is renumbered too. */
 enum { STC_IDS_AUTO = 0, STC_IDS_DIRECT = 1, STC_IDS_DENSE = 2 };
 
 /* Operand roles. Y is the tensor grouped by contract key (the array of Section 4.2), X the one

@@ -978,14 +978,16 @@ bool use_dense_ids(const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode)
 
 // Whether AUTO numbers the contract keys through a bitmap of the key space instead (KeyPlan::idmap):
 // the keys that would be renumbered, and those that direct counting would count in more than four
-// times as many bins as Y has entries. Two bits per key of bitmap and ranks are cleared and scanned;
-// past 2^30 keys, or 256 per entry, the table of id_insert_rows_kernel is smaller. Lengths 2,000 x
-// 3,000 x 14,000 x 17,000, 3e6 entries, K = 4.2e7: 1.07 -> 0.80 ms for the contraction, by direct
-// counting before; 63,891 x 63,890 x 1,847, 7.4e5 entries, K = 1.2e8: 0.42 -> 0.35, by the table.
+// times as many bins as Y has entries. Two bits per key of bitmap and ranks are cleared and scanned; past
+// 2^28 keys, or 256 per entry, the table of id_insert_rows_kernel is the faster. Lengths 2,000 x 3,000 x
+// 14,000 x 17,000, 3e6 entries, K = 4.2e7: 1.07 -> 0.80 ms for the contraction, by direct counting
+// before; 63,891 x 63,890 x 1,847, 7.4e5 entries, K = 1.2e8: 0.42 -> 0.35, by the table. Two tensors of
+// 2e6 entries each, by the map and by the table: K = 2^26 0.57 and 0.71, 2^28 0.65 and 0.67, 2^29 0.74
+// and 0.67; of 4e6 each over 100 x 100 outputs 0.55 and 0.77, 0.64 and 0.76, 0.79 and 0.75.
 bool use_id_map(const stc_ctx* ctx, const Plan& pl, const stc_coo* X, const stc_coo* Y, int mode, bool dense_ids) {
   const uint64_t nX = (uint64_t)X->nnz, nY = (uint64_t)Y->nnz;
   if (mode != STC_IDS_AUTO || nX == 0 || nY == 0 || nY >= kMaxDirectBins - 1) return false;
-  if (pl.K <= (1ull << 22) || pl.K <= 4 * nY || pl.K > (1ull << 30) || pl.K > 256 * (nX + nY)) return false;
+  if (pl.K <= (1ull << 22) || pl.K <= 4 * nY || pl.K > (1ull << 28) || pl.K > 256 * (nX + nY)) return false;
   // The map may take more memory than the table of the keys met: a budget that held the table holds.
   if (dense_ids && ctx->budget) return false;
   // Where the strategy depends on how many entries share a key, the table's count decides it.

@@ -41,13 +41,29 @@ def distinct(p):
 @pytest.mark.parametrize("xs,ys,cx,cy", [((2101, 2003, 9), (2101, 2003, 11), (0, 1), (0, 1)),
                                          ((7, 2003, 2101), (2101, 5, 2003), (2, 1), (0, 2)),
                                          ((5_000_003, 6), (5_000_003,), (0,), (0,)), ((9, 4_194_305), (4_194_305, 3), (1,), (0,)),
-                                         ((3, 200, 4, 150, 160), (160, 200, 150, 8, 2), (1, 3, 4), (1, 2, 0))])
+                                         ((3, 200, 4, 150, 160), (160, 200, 150, 8, 2), (1, 3, 4), (1, 2, 0)),
+                                         ((40, 4_194_310), (4_194_310, 200_000), (1,), (0,))])
 def test_forms(xs, ys, cx, cy, strategy):
     rng = W.rng_for(8700 + sum(xs) % 1000 + strategy)
     X, Y = W.uniform_coo(rng, xs, 4_000), W.uniform_coo(rng, ys, 3_000)
     pools(rng, X, Y, cx, cy)
     p = W.Problem(X, Y, cx, cy)
     check(p, distinct(p), strategy=strategy)
+
+
+@pytest.mark.parametrize("k", [(1 << 28) - 1, 1 << 28, (1 << 28) + 1])
+def test_widest_map(k):
+    """The last key spaces with a map and the first with the table again; the number is the same."""
+    rng = W.rng_for(8760 + k % 7)
+    X, Y = W.uniform_coo(rng, (40, k), 600_000), W.uniform_coo(rng, (k, 30), 500_000)
+    pools(rng, X, Y, (1,), (0,), n=100_000)
+    p = W.Problem(X, Y, (1,), (0,))
+    import oracle
+    from gpu_util import assert_matches_oracle, gpu_contract, result_host
+
+    res = gpu_contract(p)
+    assert_matches_oracle(*result_host(res), oracle.contract(X, Y, (1,), (0,)))
+    assert res.stats.contract_ids == distinct(p)
 
 
 @pytest.mark.parametrize("k,n,expect", [(1 << 22, 3_000, 0), ((1 << 22) + 1, 3_000, -1), ((1 << 22) + 1, 600_000, 0)])
