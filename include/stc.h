@@ -310,7 +310,9 @@ stc_status stc_server_destroy(stc_server* s);
 /* The exact product count of the contraction (Section 4.3: each X entry meets exactly
  * count_Y[its contract key] Y entries) and the device bytes a stc_contract of the same
  * inputs with default options would hold at its peak (scratch + result), for the operand
- * order and contract-key handling AUTO picks. Used to admit work under a budget.
+ * order and contract-key handling AUTO picks, at most: results take min(B, F_Y) entries per group.
+ * Not counted are the tables of groups that shared memory does not hold (with more than 2^20 Y free
+ * keys). Used to admit work under a budget.
  * products, bytes_bound: host, each may be NULL. Returns after its device work completes.
  * Errors: as stc_contract. */
 stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t ncontract,

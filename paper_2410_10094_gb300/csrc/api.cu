@@ -638,10 +638,30 @@ stc_status read_counters(const Prepared& pr, Pinned& pin, CallCounters& h) {
   return status_word(h.c.status);
 }
 
-// Device bytes of the counting of Y's contract keys.
-uint64_t bins_bytes(const Plan& pl) {
-  uint64_t b = sizeof(CallCounters) + pl.Kb * 4 * 3 + (uint64_t)scan_scratch_elems((int64_t)pl.Kb) * 4;
-  return b + (pl.id_map ? id_map_pairs(pl.K) * 8 + (uint64_t)id_map_scratch(pl.K) * 4 : (pl.K + 31) / 32 * 4);
+// The requests of prepare.
+void count_prepare(ArenaBytes& b, const Plan& pl, int64_t nX, int64_t nY, Survey mode, bool keep_ck) {
+  const bool groups = mode != Survey::kSurvivors;
+  const uint64_t bins = pl.Kb * pl.ky.nseg, x = (uint64_t)nX, y = (uint64_t)nY;
+  b.alloc(sizeof(CallCounters));
+  if (pl.id_map) {
+    b.alloc(id_map_pairs(pl.K) * sizeof(uint2));
+    b.alloc((uint64_t)id_map_scratch(pl.K) * 4);
+  }
+  const uint64_t ne_words = (mode != Survey::kDenseGroups && pl.K <= kNonemptyMaxKeys) ? (pl.K + 31) / 32 : 0;
+  const uint64_t lead = !groups && pl.F <= kGlobalFromF ? 2 * survivor_blocks(nX) : 0;
+  b.alloc((lead + bins + ne_words + (groups ? pl.FX : 0)) * 4);
+  b.alloc((bins + 1) * 4);
+  b.alloc(bins * 4);
+  b.alloc((uint64_t)scan_scratch_elems((int64_t)bins) * 4);
+  b.alloc(groups && pl.FY <= 0xffffffffull ? (y + 1) * 4 : y * 8);
+  b.alloc((y + 1) * 8);
+  if (mode != Survey::kDenseGroups) {
+    b.alloc(x * 8);
+    if (keep_ck) b.alloc(x * 4);
+    b.alloc(x * 4);
+    b.alloc(x * 4);
+    b.alloc(x * 8);
+  }
 }
 
 // Whether the one-global-table strategy writes outputs as their keys are claimed, where the list of
@@ -670,29 +690,88 @@ uint64_t space_cells(const stc_ctx* ctx, uint64_t F) {
 uint64_t global_bytes(const stc_ctx* ctx, const Plan& pl, int64_t nX, int64_t nY, uint64_t ns, uint64_t P,
                       double alpha) {
   // Small output key spaces are sized from F itself (no host read of P), with products per block of X.
-  const bool from_f = pl.F <= kGlobalFromF;
+  const bool from_f = pl.F <= kGlobalFromF && nX > 0 && nY > 0;
   const uint64_t target = from_f ? pl.F : std::min<uint64_t>(P, pl.F);
   const uint64_t cap = pow2_at_least(std::max<uint64_t>(64, (uint64_t)((double)target / alpha) + 1));
-  const uint64_t out_cap = std::min(target, cap);
-  uint64_t b = bins_bytes(pl);
-  b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * 24;
-  b += from_f ? (2 * survivor_blocks(nX) + 1) * 8 : (ns + 1) * 8 + (uint64_t)scan_scratch_elems((int64_t)ns) * 8;
-  b += std::max(cap * 16, from_f ? space_cells(ctx, pl.F) * 8 : 0) + out_cap * (4ull * pl.ocols + 8);
-  if (!from_f && direct_global(P, pl.F, cap) && ctx->budget == 0) b += P * 12;
-  return b;
+  const uint64_t out = std::min(target, cap) * (4ull * pl.ocols + 8);
+  ArenaBytes b(ctx);
+  count_prepare(b, pl, nX, nY, Survey::kSurvivors, false);
+  if (from_f) {
+    b.alloc(space_cells(ctx, pl.F) * 8);
+    b.alloc((survivor_blocks(nX) + 1) * 8);
+    b.alloc_own(out);
+    return b.held;
+  }
+  if (P == 0) return b.held;
+  ArenaBytes table = b;  // the table of values, also where there is no memory for the list of repeats
+  if (direct_global(P, pl.F, cap) && ctx->budget == 0) {
+    b.alloc(cap * 8);
+    b.alloc(cap * 4);
+    b.alloc(P * 4);
+    b.alloc(P * 8);
+  } else {
+    b = ArenaBytes(ctx);
+  }
+  table.alloc(cap * 8);
+  table.alloc(cap * 8);
+  for (ArenaBytes* t : {&b, &table}) {
+    t->alloc((ns + 1) * 8);
+    t->alloc((uint64_t)scan_scratch_elems((int64_t)ns) * 8);
+    t->alloc_own(out);
+  }
+  return std::max(b.held, table.held);
 }
 
+// How GROUPED sweeps rows of bitmaps: F_Y in `nseg` segments of `seg` free keys; Y is grouped per
+// (contract key, segment). For F_Y <= 2^20 and the bins' limit: for every group with the bitmap
+// accumulator, for the groups beyond the warp-sized hash classes with AUTO.
+bool dense_segments(const Plan& pl, int32_t accumulator, uint32_t& seg, uint32_t& nseg) {
+  seg = nseg = 1;
+  if (pl.FY > (1ull << 20) || (accumulator != STC_ACC_AUTO && accumulator != STC_ACC_DENSE)) return false;
+  seg = (uint32_t)std::min<uint64_t>(kDenseSeg, pow2_at_least(std::max<uint64_t>(pl.FY, 64)));
+  nseg = (uint32_t)((pl.FY + seg - 1) / seg);
+  return pl.Kb * nseg <= kMaxDirectBins;
+}
 
-// Peak device bytes of the GROUPED strategy: Y grouped, X grouped (and, at worst, a survivor
-// list), per-group arrays, and an output at its bound. Overflow-group tables are bounded by
-// twice the output bound.
-uint64_t grouped_bytes(const Plan& pl, int64_t nX, int64_t nY, uint64_t P) {
-  const uint64_t out = std::min<uint64_t>(P, pl.F);
-  uint64_t b = bins_bytes(pl);
-  b += ((uint64_t)nY + 1) * 16 + (uint64_t)nX * (24 + 16);
-  b += pl.FX * (4 * 3) + std::min<uint64_t>(pl.FX, (uint64_t)nX) * 4 * (kMaxClasses + 5);
-  b += out * (4ull * pl.ocols + 8);
-  return b;
+// Positions to be expected left over by `nstream` streamed groups: the last groups of the kernel's CTAs
+// and the pieces that they drop.
+uint64_t expected_holes(const stc_ctx* ctx, uint64_t nstream, uint64_t out_cap) {
+  return std::min<uint64_t>(out_cap, std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64);
+}
+
+// Peak device bytes of the GROUPED strategy with default options, the output at its bound, without the
+// tables of groups that are too large for shared memory (F_Y above 2^20).
+uint64_t grouped_bytes(const stc_ctx* ctx, Plan pl, int64_t nX, int64_t nY, uint64_t P, Survey mode) {
+  uint32_t seg = 1, nseg = 1;
+  const bool dense_rows = dense_segments(pl, STC_ACC_AUTO, seg, nseg);
+  if (dense_rows) pl.ky.nseg = nseg;
+  const uint64_t x = (uint64_t)nX, out = std::min<uint64_t>(P, pl.F);
+  const uint64_t maxg = std::min<uint64_t>(pl.FX, (uint64_t)std::max<int64_t>(nX, 1));
+  const bool wide = pl.FY > 0xffffffffull;
+  ArenaBytes b(ctx);
+  count_prepare(b, pl, nX, nY, mode, dense_rows);
+  b.alloc((pl.FX + 1) * 4);
+  b.alloc(pl.FX * 4);
+  b.alloc((uint64_t)scan_scratch_elems((int64_t)pl.FX) * 4);
+  b.alloc(x * 4);
+  b.alloc(x * 4);
+  b.alloc(x * 8);
+  if (dense_rows) b.alloc(x * 4);
+  for (int c = 0; c < (wide ? kNumClasses64 : kNumClasses32) + (dense_rows ? 3 : 0) + 1; c++) b.alloc(maxg * 4);
+  b.alloc(maxg * 8);
+  b.alloc(maxg * 8);
+  if (P == 0) return b.held;
+  b.alloc_own(out * 4ull * pl.ocols);
+  b.alloc_own(out * 8);
+  b.alloc(sizeof(BatchOut));
+  if (dense_rows) {
+    // Streamed groups have more products per segment than the warp classes have slots.
+    const uint64_t nstream = std::min<uint64_t>(maxg, P / (kClassShapes32[1].slots / 2 * nseg));
+    if (nstream) b.alloc(stream_max_holes((uint32_t)nstream, nseg) * sizeof(StreamHole));
+    const uint64_t holes = expected_holes(ctx, nstream, out);
+    if (ctx->budget == 0 && holes > x) b.alloc(holes * 4);  // under a budget only where there is room
+  }
+  return b.held;
 }
 
 // Whether GROUPED counts X without a survivor list: Y's runs cover the contract keys on average, or
@@ -709,16 +788,8 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   if (o.accumulator == STC_ACC_ROWS && pl.FY > kLaneRowMax)
     return fail(STC_ERR_INVALID_ARG, "the ROWS accumulator takes at most %llu Y free keys, not %llu",
                 (unsigned long long)kLaneRowMax, (unsigned long long)pl.FY);
-  // Bitmap rows: F_Y is swept in segments of `seg` free keys; Y is grouped per (contract key,
-  // segment). Used when F_Y <= 2^20: for every group with the bitmap accumulator, for the
-  // groups beyond the warp-sized hash classes with AUTO.
-  bool dense_rows = false;
   uint32_t seg = 1, nseg = 1;
-  if (pl.FY <= (1ull << 20) && (o.accumulator == STC_ACC_AUTO || o.accumulator == STC_ACC_DENSE)) {
-    seg = (uint32_t)std::min<uint64_t>(kDenseSeg, pow2_at_least(std::max<uint64_t>(pl.FY, 64)));
-    nseg = (uint32_t)((pl.FY + seg - 1) / seg);
-    dense_rows = pl.Kb * nseg <= kMaxDirectBins;
-  }
+  const bool dense_rows = dense_segments(pl, o.accumulator, seg, nseg);
   if (dense_rows) {
     pl.ky.nseg = pl.kx.nseg = nseg;
     pl.ky.seg_shift = log2_u64(seg);
@@ -863,9 +934,9 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
   }
   tm.mark(4);
   // The holes are filled from the output's end before their number is known here, in one round for
-  // as many positions as are to be expected: the streaming CTAs' last groups and the pieces they
-  // drop. More take further rounds below. The scratch is one word per position; where there is no
-  // memory for it, an array of the grouped X serves, which nothing reads any more.
+  // as many positions as are to be expected; more take further rounds below. The scratch is one word
+  // per position; where there is no memory for it, an array of the grouped X serves, which nothing
+  // reads any more.
   HoleRound rd{};
   auto fill = [&]() -> stc_status {
     STC_CUDA(launch_hole_fill(sa.holes, sa.nholes, &pr.ctr->nz, &gc->holes, rd, gc->fill_counters, r->coords, r->vals,
@@ -873,35 +944,23 @@ stc_status contract_grouped(stc_ctx* ctx, Arena& ar, const stc_coo* X, const stc
     tm.mark(5);
     return STC_OK;
   };
-  auto room = [&](uint64_t most) {
-    uint32_t* more = nullptr;
-    if (most > (uint64_t)nX) {
-      if (ar.alloc(&more, (size_t)most) == STC_OK) {
-        rd.dst = more;
-        rd.win = most;
-        return;
-      }
-      g_last_error.clear();
-    }
-    if (!rd.dst) rd.dst = gx.ystart, rd.win = (uint64_t)nX;
-    rd.win = std::min<uint64_t>(rd.win, most);
-  };
   if (nstream) {
-    room(std::min<uint64_t>(out_cap, std::min<uint64_t>(nstream, 4ull * ctx->sms) * stream_cap() + out_cap / 64));
+    rd.win = expected_holes(ctx, nstream, out_cap);
+    if (rd.win <= (uint64_t)nX || ar.alloc(&rd.dst, (size_t)rd.win) != STC_OK) {
+      if (rd.win > (uint64_t)nX) g_last_error.clear();
+      rd.win = std::min<uint64_t>(rd.win, (uint64_t)nX);
+      rd.dst = gx.ystart;
+    }
     STC_TRY(fill());
   }
   CallCounters hc2{};
   STC_TRY(read_counters(pr, pin, hc2));
   const u64 holes = hc2.g.holes;
   r->nnz = (int64_t)(hc2.c.nz - holes);
-  if (holes > rd.win) {
-    const u64 done = rd.win;
-    room(holes - done);
-    for (rd.at = done; rd.at < holes; rd.at += rd.win) {
-      rd.base = hc2.g.fill_counters[1];
-      STC_TRY(fill());
-      STC_TRY(read_counters(pr, pin, hc2));
-    }
+  for (rd.at = rd.win; rd.at < holes; rd.at += rd.win) {
+    rd.base = hc2.g.fill_counters[1];
+    STC_TRY(fill());
+    STC_TRY(read_counters(pr, pin, hc2));
   }
   if (hc2.g.fill_counters[0] != hc2.g.fill_counters[1])
     return fail(STC_ERR_CUDA, "holes and entries to fill them do not match");
@@ -2144,9 +2203,13 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
     STC_TRY(stc_count(ctx, &rl.X, &rl.Y, 1, &rl.cx, &rl.cy, stream, products, bytes_bound ? &b : nullptr));
     // The rewritten coordinates stay held beside the id table, then beside the contraction.
     const uint64_t slots = id_table_slots(Y->nnz);
-    const uint64_t table = 16 * slots + 4 * (uint64_t)scan_scratch_elems((int64_t)slots + 1) + 16;
-    if (bytes_bound)
-      *bytes_bound = std::max(b, table) + 4ull * (uint64_t)(rl.X.order * X->nnz + rl.Y.order * Y->nnz);
+    ArenaBytes rows(ctx), table(ctx);
+    rows.alloc(4ull * (uint64_t)rl.X.order * (uint64_t)X->nnz);
+    rows.alloc(4ull * (uint64_t)rl.Y.order * (uint64_t)Y->nnz);
+    for (uint64_t n : {slots * 8, (slots + 1) * 4, (slots + 2) * 4, (uint64_t)scan_scratch_elems((int64_t)slots + 1) * 4,
+                       (uint64_t)4})
+      table.alloc(n);
+    if (bytes_bound) *bytes_bound = rows.held + std::max(b, table.held);
     return STC_OK;
   }
   Arena ar(ctx, s);
@@ -2160,9 +2223,14 @@ stc_status stc_count(stc_ctx* ctx, const stc_coo* X, const stc_coo* Y, int32_t m
   STC_TRY(read_counters(pr, pin, hc));
   const Counters& h = hc.c;
   if (products) *products = h.P;
-  if (bytes_bound)
-    *bytes_bound = strategy == STC_STRATEGY_GROUPED ? grouped_bytes(pl, X->nnz, Y->nnz, h.P)
-                                                    : global_bytes(ctx, pl, X->nnz, Y->nnz, h.ns, h.P, 0.5);
+  if (!bytes_bound) return STC_OK;
+  const Survey grouped = x_dense(pl, Y) ? Survey::kDenseGroups : Survey::kSurvivorsGroups;
+  *bytes_bound = strategy == STC_STRATEGY_GROUPED ? grouped_bytes(ctx, pl, X->nnz, Y->nnz, h.P, grouped)
+                                                  : global_bytes(ctx, pl, X->nnz, Y->nnz, h.ns, h.P, 0.5);
+  // A shape that a run here finds to be rows-heavy is grouped from then on.
+  if (strategy == STC_STRATEGY_GLOBAL && pl.FY <= kLaneRowMax && pl.FX <= kMaxDirectBins &&
+      h.P >= kRowsMinPerOutput * pl.F)
+    *bytes_bound = std::max(*bytes_bound, grouped_bytes(ctx, pl, X->nnz, Y->nnz, h.P, grouped));
   return STC_OK;
 }
 

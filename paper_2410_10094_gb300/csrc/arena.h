@@ -5,6 +5,7 @@
 
 #include <atomic>
 #include <cstddef>
+#include <cstdint>
 #include <cstdio>
 #include <vector>
 
@@ -36,6 +37,11 @@ struct Arena {
   char* slab = nullptr;
   size_t slab_left = 0;
   Arena(DevicePool* c, cudaStream_t st) : ctx(c), s(st) {}
+  // Whether a request is a piece of a slab, and the bytes that it takes there.
+  static size_t piece(size_t bytes) { return (bytes + 255) & ~(size_t)255; }
+  static bool shares_slab(const DevicePool* c, size_t bytes) {
+    return bytes != 0 && piece(bytes) <= kSlabMost && !c->budget;
+  }
   Arena(const Arena&) = delete;
   Arena& operator=(const Arena&) = delete;
   ~Arena() {
@@ -46,8 +52,8 @@ struct Arena {
   }
   template <typename T>
   stc_status alloc(T** out, size_t count) {
-    const size_t bytes = (count * sizeof(T) + 255) & ~(size_t)255;
-    if (bytes == 0 || bytes > kSlabMost || ctx->budget) return alloc_own(out, count);
+    if (!shares_slab(ctx, count * sizeof(T))) return alloc_own(out, count);
+    const size_t bytes = piece(count * sizeof(T));
     if (bytes > slab_left) {
       char* p = nullptr;
       if (alloc_own(&p, kSlab) != STC_OK) return alloc_own(out, count);
@@ -103,6 +109,28 @@ struct Arena {
       }
     return 0;
   }
+};
+
+// The bytes that an arena holds after the same requests, none given back: what a call will hold at its
+// peak, counted without making it.
+struct ArenaBytes {
+  const DevicePool* ctx;
+  uint64_t held = 0;
+  size_t slab_left = 0;
+  explicit ArenaBytes(const DevicePool* c) : ctx(c) {}
+  void alloc(uint64_t bytes) {
+    if (!Arena::shares_slab(ctx, bytes)) {
+      held += bytes;
+      return;
+    }
+    const size_t b = Arena::piece(bytes);
+    if (b > slab_left) {
+      held += Arena::kSlab;
+      slab_left = Arena::kSlab;
+    }
+    slab_left -= b;
+  }
+  void alloc_own(uint64_t bytes) { held += bytes; }
 };
 
 }  // namespace stc

@@ -1,5 +1,5 @@
 """A call's device memory (csrc/arena.h) on the host, over a pool that counts: what is given back early,
-what a result keeps, and that a slab outlives every piece of it."""
+what a result keeps, that a slab outlives every piece of it, and what a sequence of requests will hold."""
 import os
 import subprocess
 
@@ -70,6 +70,25 @@ int main() {
     CHECK(pool.held == 0 && ar.alloc(&second, 5000) == STC_OK);
   }
   CHECK(pool.held == 0 && taken == given);
+  // The bytes counted for a sequence of requests are those that an arena holds after it.
+  for (int budget = 0; budget < 2; budget++) {
+    pool.budget = budget ? (size_t)1 << 40 : 0;
+    Arena ar(&pool, nullptr);
+    ArenaBytes count(&pool);
+    unsigned x = 12345;
+    for (int i = 0; i < 400; i++) {
+      x = x * 1664525u + 1013904223u;
+      const size_t n = i % 7 == 0 ? x >> 12 : x >> 17;  // up to 2^20 and 2^15
+      if (i % 29 == 0) {
+        CHECK(ar.alloc_own(&own, n) == STC_OK);
+        count.alloc_own(n);
+      } else {
+        CHECK(ar.alloc(&own, n) == STC_OK);
+        count.alloc(n);
+      }
+      CHECK(count.held == pool.held);
+    }
+  }
   return 0;
 }
 """

@@ -4,7 +4,7 @@
   bounded probe flags the overflow, the call retries at full capacity and the result still
   matches the oracle;
 * a context budget smaller than one call's bound: STC_ERR_OUT_OF_MEMORY, nothing left held,
-  and the context still serves smaller calls;
+  and the context still serves smaller calls; a budget of the counted bound is enough;
 * a request cancelled while it waits in the server's queue: its wait reports
   STC_ERR_CANCELLED, every other request finishes with its correct product count, and the
   server keeps serving.
@@ -74,6 +74,43 @@ def test_budget_smaller_than_one_call():
 
         gc.collect()
         ctx.close()
+
+
+def bounded():
+    """One contraction for each way that the counted bound is put together."""
+    rng = W.rng_for(9515)
+    yield "one table of values", W.Problem(W.uniform_coo(rng, (2_000_000, 40), 30_000), W.uniform_coo(rng, (40, 90_000), 4_000), (1,), (0,))
+    yield "a small output space", W.Problem(W.uniform_coo(rng, (300, 40), 30_000), W.uniform_coo(rng, (40, 200), 4_000), (1,), (0,))
+    yield "a tiny output space", W.Problem(W.uniform_coo(rng, (3, 4), 9), W.uniform_coo(rng, (4, 2), 6), (1,), (0,))
+    yield "streamed groups", W.Problem(W.uniform_coo(rng, (64, 64, 64), 20_000), W.uniform_coo(rng, (64, 80, 90), 20_000), (2,), (0,))
+    yield "several segments", W.Problem(W.uniform_coo(rng, (500, 50), 3_000), W.uniform_coo(rng, (50, 300_000), 90_000), (1,), (0,))
+    yield "small groups", W.Problem(W.uniform_coo(rng, (30_000, 90), 60_000), W.uniform_coo(rng, (90, 50_000), 3_000), (1,), (0,))
+    yield "numbered keys", W.Problem(W.uniform_coo(rng, (2_000, 1 << 24), 60_000), W.uniform_coo(rng, (1 << 24, 3_000), 50_000), (1,), (0,))
+    yield "few survivors", W.Problem(W.uniform_coo(rng, (5_000, 300_000), 100_000), W.uniform_coo(rng, (300_000, 2_000), 30_000), (1,), (0,))
+    yield "rows", W.Problem(W.uniform_coo(rng, (500, 20), 9_000), W.uniform_coo(rng, (20, 30), 30_000), (1,), (0,))
+    yield "nothing in common", W.Problem(W.uniform_coo(rng, (5_000_000, 40), 3_000), W.uniform_coo(rng, (40, 5_000_000), 0), (1,), (0,))
+
+
+@pytest.mark.parametrize("p", [pytest.param(p, id=n.replace(" ", "_")) for n, p in bounded()])
+def test_counted_bytes_are_enough(p):
+    """A context whose budget is the bound of stc_count runs the call, again and again."""
+    import gc
+
+    import paper_2410_10094_gb300 as stc
+
+    dev = to_dev(p.X), to_dev(p.Y), p.cx, p.cy
+    wide = stc.Context(0, mem_budget_bytes=8 << 30)
+    P, need = stc.count(*dev, ctx=wide)
+    wide.close()
+    ctx = stc.Context(0, mem_budget_bytes=need)
+    for _ in range(2):
+        r = stc.contract(*dev, ctx=ctx)
+        assert r.stats.products == P
+        c, v = result_host(r)
+        assert_matches_oracle(c, v, oracle.contract(p.X, p.Y, p.cx, p.cy))
+        del r
+        gc.collect()
+    ctx.close()
 
 
 def test_server_cancel_queued_request():

@@ -101,13 +101,13 @@ def mostly_repeats(rng):
 
 
 def test_more_holes_than_expected():
-    """Filled in further rounds, with scratch for all of them."""
+    """Filled in further rounds."""
     check(mostly_repeats(W.rng_for(8260)), accumulator=2)
 
 
 def test_holes_without_memory_for_them():
-    """A context with room for the call's arrays and its output: the holes are filled in rounds through
-    an array that the call has already."""
+    """A context whose budget is the bound of stc_count: the holes are filled in rounds through an array
+    that the call has already."""
     import gc
 
     import oracle
@@ -119,7 +119,7 @@ def test_holes_without_memory_for_them():
     wide = stc.Context(mem_budget_bytes=8 << 30)
     _, need = stc.count(*dev, ctx=wide)
     wide.close()
-    tight = stc.Context(mem_budget_bytes=need + (1 << 20))
+    tight = stc.Context(mem_budget_bytes=need)
     res = stc.contract(*dev, ctx=tight, strategy=2, accumulator=2, operands=stc.OPERANDS_AS_GIVEN)
     assert res.stats.out_capacity == res.stats.products == 24_000_000
     assert_matches_oracle(*result_host(res), oracle.contract(p.X, p.Y, p.cx, p.cy, None))
