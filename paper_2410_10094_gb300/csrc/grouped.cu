@@ -1718,8 +1718,10 @@ cudaError_t launch_warp_direct_class(const GroupArgs& a, const uint32_t* list, c
 // PK groups share every load, scan, table clearing and reservation of output positions that a group
 // alone would wait for. Otherwise as group_warp_direct_kernel.
 // Measured on 4e5 groups of 63 products (lengths 100, order 5 with order 4, 5e5 entries each): 0.64
-// against 0.88 ms; on 4,096 groups of 95 the four groups of a warp wait for one another longer than
-// the idle warps would help (60 against 40 us), so few groups keep a warp each.
+// against 0.88 ms by a warp per group; 1e5 groups of one product 35 against 88 us, of 64 98 against 133,
+// of 150 0.25 against 0.32 ms, of 700 (one per warp here too) 1.22 both. On few groups the four of a warp
+// wait for one another longer than the idle warps would help: 4,096 of 95 60 against 40 us, 17,000 of 16
+// 21 against 27, of 64 36 against 35, of 150 74 against 69, so that is where the line lies.
 constexpr uint32_t kPackMinGroups = 16384;
 constexpr uint32_t kPackSlots = 1024;
 constexpr uint32_t kPackBits = 30;  // bits of the free key where PK > 1
@@ -2102,11 +2104,6 @@ cudaError_t launch_bin_groups(u64 FX, const uint32_t* goff, const uint32_t* gw, 
   return cudaGetLastError();
 }
 
-// Whether the warp classes of a single contraction take several groups per warp (group_pack_kernel).
-static bool packs(uint32_t small, uint32_t medium, u64 FY) {
-  return (u64)small + medium >= kPackMinGroups && FY < (1u << kPackBits);
-}
-
 cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct, const Bins& b,
                                  const uint32_t* counts, int sms, cudaStream_t s, int depth) {
   cudaError_t e = cudaSuccess;
@@ -2115,7 +2112,8 @@ cudaError_t launch_group_classes(const GroupArgs& a, bool wide_keys, bool direct
   uint32_t h[kMaxClasses];
   for (int c = 0; c < kMaxClasses; c++) h[c] = counts ? counts[c] : kCountOnDevice;
   const uint32_t* d = b.count;
-  if (!wide_keys && direct && !a.gprob && counts && packs(h[0], h[1], a.FY)) {
+  if (!wide_keys && direct && !a.gprob && a.FY < (1u << kPackBits) && counts &&
+      (u64)h[0] + h[1] >= kPackMinGroups) {
     // Small groups of a single contraction, many of them. Four share a table of 1,024 slots where
     // each takes at most 256 (and the load factor leaves room, as it does for one group in 256).
     if ((e = launch_pack<4>(a, b.list[0], d + 0, h[0], sms, s))) return e;

@@ -20,9 +20,9 @@
 // unaligned positions reaches (4.9 TB/s; 6.5 where groups start on 128-byte boundaries): 1.96 ms for
 // the 3.65e8 outputs of two 256^4 tensors with 5e6 entries each. The 4.4% repeats cost 0.9 ms more:
 // the passes over the first products' keys and the barriers between them, in which a CTA stores
-// nothing. Measured on that contraction (accumulation): 2.87 ms, and 0.08 ms for the holes, against
+// nothing. Measured on that contraction (accumulation): 2.82 ms, and 0.06 ms for the holes, against
 // 3.54 and 0.24 ms with slots of 32, the repeats kept in global memory and every group's holes
-// filled; a 4 x 4 x 93 x 36 x 432 tensor of 3e5 entries with itself 2.35 against 3.40 ms.
+// filled; a 4 x 4 x 93 x 36 x 432 tensor of 3e5 entries with itself 2.31 against 3.40 ms.
 // A table of 16-bit places per free key in place of the bitmaps and their ranking (128 KB, one CTA
 // of 1,024 threads per SM) took 3.4 ms: its phases leave the memory idle between barriers.
 #include "launch.h"
