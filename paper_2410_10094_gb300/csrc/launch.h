@@ -369,14 +369,17 @@ uint32_t dense_stash_cap();
 //     1.5 0.9 to 1.3; all products on 60 keys 0.7 (1,500) to 1.2
 //   form 1, 6,000 to 12,000 products: 1.5 to 1.9; 1.0 to 1.1; 0.7; 0.8 to 1.0
 //   form 2, 40,000 products, whose tables lie in global memory: 6 to 10; 3.5 to 6; 1.7 to 2.4; 1.4 to 2.2
-//   form 1 at 800 and 3,000 products over more than 2^16 keys, where half as many groups are in flight:
-//     0.7 and 1.4; 0.7 and 0.9; 0.5 and 0.6; 0.5 and 0.6, so that the tables take those up to 6,144.
+//   form 1 at 800, 1,500 and 3,000 products over more than 2^16 keys, where half as many groups are in
+//     flight: 0.7, 1.0 and 1.4; 0.7, 0.7 and 0.9; 0.5, 0.6 and 0.6; 0.5, 0.5 and 0.6
+// A group's skew is not known before it is accumulated: the lines are those of even keys, so that the
+// tables take groups of up to 2,048 products over more than 2^16 keys. (2,048 uneven pairs: 78.3 ms with
+// this line at 6,144, 77.7 at 2,048; 256 pairs 10.58 and 10.42.)
 // The lead falls as even keys repeat, 1.12 to 1.19 at 2 to 4 products per key and 0.96 to 1.14 at 8, where
 // the line is drawn. Groups of the 1,024-slot warp tables lose (the batch of 256 pairs: 15.3 against 13.8
 // ms with those above 320 products taken in).
 __host__ __device__ constexpr int twopass_list(u64 products, uint32_t entries, u64 FY) {
   if (FY > (1u << 18) || products > 49152 || entries > 1024 || products > 4 * FY) return -1;
-  if (FY > (1u << 16) && products <= 6144) return -1;
+  if (FY > (1u << 16) && products <= 2048) return -1;
   if (FY <= (1u << 16) && products <= 8192 && entries <= 256) return 0;
   return products <= 16384 && entries <= 512 ? 1 : 2;
 }

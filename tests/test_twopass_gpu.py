@@ -50,7 +50,7 @@ def check(probs):
 
 
 @pytest.mark.parametrize("yfree", [(256, 256), (255, 257), (65537,), (512, 512), (511, 513), (262145,)])
-@pytest.mark.parametrize("products", [(770, 1025), (6144, 6145), (8192, 8193), (16384, 16385), (49152, 49153)])
+@pytest.mark.parametrize("products", [(770, 1025), (2048, 2049), (8192, 8193), (16384, 16385), (49152, 49153)])
 def test_limits(yfree, products):
     check([problem(i, 4, yfree, p, 4) for i, p in enumerate(products)])
 
