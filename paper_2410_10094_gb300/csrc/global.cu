@@ -218,7 +218,8 @@ __global__ void __launch_bounds__(kBpThreads) block_prefix_kernel(const u64* __r
 // mod the array's length, a power of two, so that the keys of one output row, of which a few may get
 // most of the products, lie on lines far apart: additions to one 128-byte line take their turns. 4e7
 // products on one row of 130 keys of 2,000 x 130: 1.14 ms for the contraction, 9.9 with the rows in
-// order, 1.26 in a table; 4e7 uniform products on 512 x 512: 0.60, 0.51 and 0.84.
+// order, 1.26 in a table; 4e7 uniform products on 512 x 512: 0.60, 0.51 and 0.84 (all with tiles of 1,024
+// products; with larger ones, kBxTileMost, 1.05 and 1.21 by array and table, and 0.38 and 0.57).
 constexpr uint32_t kSpread = 0x9e3779b1u;  // odd; 2^32 over the golden ratio
 constexpr uint32_t inverse_of(uint32_t odd) {
   uint32_t x = odd;  // the right inverse mod 8; every step doubles the bits that are right
@@ -235,7 +236,10 @@ __global__ void __launch_bounds__(kExThreads) clear_space_kernel(double* __restr
   for (u64 i = (u64)blockIdx.x * kExThreads + threadIdx.x; i < n; i += (u64)gridDim.x * kExThreads) vals[i] = -0.0;
 }
 
-constexpr int kBxTile = 1024;  // products per tile
+// Products per tile, at least, and at most: a tile scans whole blocks of survivors for the products that
+// it takes of them, so that many products come in larger tiles, about eight per CTA. 2.04e10 products of
+// some thousand per survivor on 262,144 outputs: 213 -> 105 ms by array, 305 -> 173 by table.
+constexpr u64 kBxTile = 1024, kBxTileMost = 65536;
 
 // Adds one product to the output space: the hash table, probed by G lanes together (see
 // expand_global_kernel), or with G = 0 an array of the whole space.
@@ -253,10 +257,12 @@ __global__ void __launch_bounds__(kExThreads) expand_blocks_kernel(const u64* __
   __shared__ u64 s_warp[NW];
   __shared__ int64_t s_lo;
   const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
-  const u64 ntiles = (P + kBxTile - 1) / kBxTile;
+  const u64 share = P / ((u64)gridDim.x * 8) / kBxTile * kBxTile;
+  const u64 size = share < kBxTile ? kBxTile : (share < kBxTileMost ? share : kBxTileMost);
+  const u64 ntiles = (P + size - 1) / size;
   for (u64 tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const u64 p0 = tile * kBxTile;
-    const u64 p1 = (p0 + kBxTile < P) ? p0 + kBxTile : P;
+    const u64 p0 = tile * size;
+    const u64 p1 = (p0 + size < P) ? p0 + size : P;
     if (warp == 0) {
       const int64_t at = warp_upper(bpre, nb, p0);
       if (lane == 0) s_lo = at;
@@ -289,8 +295,13 @@ __global__ void __launch_bounds__(kExThreads) expand_blocks_kernel(const u64* __
       __syncthreads();
       const int n = (int)(ns - s0 < (int64_t)kSurvivorBlock ? ns - s0 : (int64_t)kSurvivorBlock);
       const u64 a0 = q0 > p0 ? q0 : p0, a1 = q1 < p1 ? q1 : p1;
+      int e0 = 0, e1 = n;  // a larger tile looks among the entries that its own products have
+      if (size > kBxTile) {
+        e0 = __shfl_sync(0xffffffffu, warp_owners(s_pre, n, a0), 0);
+        e1 = __shfl_sync(0xffffffffu, warp_owners(s_pre, n, a1 - 1), 0) + 1;
+      }
       for (u64 g0 = a0 + warp * 32; g0 < a1; g0 += kExThreads) {
-        const int a = warp_owners(s_pre, n, g0);
+        const int a = e0 + warp_owners(s_pre + e0, e1 - e0, g0);
         const u64 g = g0 + lane;
         const bool has = g < a1;
         u64 key = 0;
