@@ -49,10 +49,16 @@ __global__ void __launch_bounds__(kThreads) x_group_scatter_kernel(Survivors sv,
 
 // The bound B_g of every X free key's group (Section 4.3) is the sum of its entries' run lengths,
 // read from the grouped X. Non-empty groups go to the first class whose table holds
-// t = min(B_g, F_Y); larger ones get a region of the overflow table. A warp takes `per` consecutive
+// t = min(B_g, F_Y), but to none of the warp classes with more than kWarpProducts products, however few
+// their keys; larger ones get a region of the overflow table. A warp takes `per` consecutive
 // groups, one per lane: short ones are summed by their lane, long ones by all lanes in turn; then
 // each list gets one reservation for the warp's groups. (With a warp and a reservation per group,
 // the counters' atomics took 0.27 ms for 4e5 groups, each on one of a few addresses.)
+// kWarpProducts: ten groups over 113 keys beside 20,000 small ones, of 2,400 products each 0.36 ms for the
+// contraction by warps and 0.22 by a CTA each, of 20,000 1.02 and 0.27; 5,000 of 2,400 0.45 and 0.36;
+// 50,000, which fill the device either way, of 1,200 0.86 and 1.01, of 2,400 1.36 and 1.52, of 10,000 4.55
+// and 4.60.
+constexpr u64 kWarpProducts = 2048;
 __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint32_t* __restrict__ goff,
                                                               const uint32_t* __restrict__ gw, u64 FY, Bins b,
                                                               uint32_t per, unsigned* entries) {
@@ -90,6 +96,7 @@ __global__ void __launch_bounds__(kThreads) bin_groups_kernel(u64 FX, const uint
     if (x1 > x0) {
       int c = 0;
       while (c < b.nclasses && t > b.tmax[c]) c++;
+      if (c < 2 && bnd > kWarpProducts) c = 2;
       if (b.dense_list[0] && t >= b.dense_min) {
         // The streaming kernel pays for every repeat, the stash kernel for every product. Measured
         // on 8,192 groups of 6,400 products: 30,000 free keys 0.59 against 0.81 ms, 10,000 keys

@@ -44,6 +44,25 @@ def test_uneven_groups():
     check(X, W.uniform_coo(rng, (60, 3_000), 700))
 
 
+@pytest.mark.parametrize("fy", [1, 100, 700, 1 << 33])
+@pytest.mark.parametrize("entries", [15, 16, 17, 400])
+def test_many_products_on_few_keys(entries, fy):
+    """Groups of 1,920 to 51,200 products among packed ones, on either side of the 2,048 that a warp takes,
+    over fewer keys than its table has slots; and with 64-bit keys."""
+    rng = W.rng_for(8655 + entries + fy % 999)
+    groups = 16_500
+    n = np.ones(groups, np.int64)
+    n[::1000] = entries
+    xc = np.stack([np.repeat(np.arange(groups), n), rng.integers(0, 50, n.sum())], 1)
+    X = W.COO((groups, 50), xc.astype(np.int32), W.nonzero_values(rng, len(xc)))
+    yc = np.stack([np.repeat(np.arange(50), 128), rng.integers(0, min(fy, 700), 50 * 128)], 1)
+    if fy > 1 << 31:  # two free modes of Y
+        yc = np.insert(yc, 2, rng.integers(0, 9, len(yc)), 1)
+        check(X, W.COO((50, 1 << 17, 1 << 16), yc.astype(np.int32), W.nonzero_values(rng, len(yc))))
+    else:
+        check(X, W.COO((50, fy), yc.astype(np.int32), W.nonzero_values(rng, len(yc))))
+
+
 @pytest.mark.parametrize("fy", [(1 << 30) - 1, 1 << 30])
 def test_widest_packed_key(fy):
     rng = W.rng_for(8660 + (fy & 3))
