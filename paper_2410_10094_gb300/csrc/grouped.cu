@@ -2269,7 +2269,7 @@ __global__ void __launch_bounds__(kRowWarps * 32) group_lanerow_kernel(GroupArgs
 // per SM ends evenly, where warps that own whole groups leave the last round of groups half empty.
 // The loads of the next products are issued before the current ones are added, so that the FP64
 // pipe (two rounded operations per product) is what bounds the loop: 2.04e10 products in 4,096
-// groups take 82.6 ms, 0.93 of half the measured rate of FP64 multiplies; by a warp per group 143.
+// groups take 81.2 ms, 0.95 of half the measured rate of FP64 multiplies; by a warp per group 143.
 // More and shorter chains also round less: 78,000 random products summed this way err by 3.0e-18 of their
 // absolute sum (rms, against extended precision), by one warp's 32 rows 9.1e-18.
 constexpr int kCtaRowWarps = 13;  // 13 x 32 rows of 65 doubles: 216 KB of shared memory
